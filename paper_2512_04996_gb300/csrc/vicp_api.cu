@@ -537,17 +537,46 @@ vicp_status run_localised(vicp_ctx *c, const float4 *src, int m, const double *p
     });
 }
 
-// Correspond + global search into nn/d2 (shared by vicp_correspond and the step).
-vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, int *nn, float *d2, int honor_stop)
+// The global searches and dense segments that a localised search listed;
+// hv_store: the store the dense segments lie in.
+vicp_status run_global(vicp_ctx *c, const float4 *src, int m, const double *pose, int *nn, float *d2,
+                       const float4 *hv_store, int honor_stop, int *n_global_out)
 {
-    DevCtl *d = ctl_of(c);
+    const bool sparse = sparse_of(c);
+    FallbackArgs a{};
+    a.src = src;
+    a.pose = pose;
+    a.g = c->geom;
+    a.occ = (const unsigned *)c->occ[c->occ_cur].p;
+    a.off = (const unsigned *)(sparse ? c->ooff.p : c->off.p);
+    a.csr = (const float4 *)c->csr.p;
+    if (sparse)
+        a.okeys = table_of(c->okeys[c->o_cur], c->cap_o);
+    a.bpts = (const float4 *)c->bpts.p;
+    a.bbox = (const float4 *)c->brick_box.p;
+    a.sb_box = (const float4 *)c->sb_box.p;
+    a.tgt = c->target;
+    a.n_tgt = c->n_target;
+    a.outside = (const int *)c->outside.p;
+    a.fb_list = (const int *)c->fb_list.p;
+    a.hv_list = (const int *)c->hv_list.p;
+    a.hv_range = (const uint2 *)c->hv_range.p;
+    a.hv_store = hv_store;
+    a.ctl = ctl_of(c);
+    a.nn = nn;
+    a.d2 = d2;
+    a.m = m;
+    a.honor_stop = honor_stop;
+    a.n_global_out = n_global_out;
+    return launch(c, K_FALLBACK, [&] { return launch_fallback(a, c->stream); });
+}
+
+// Correspond + global search into nn/d2 (shared by vicp_correspond and the step).
+vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, int *nn, float *d2, int honor_stop,
+                    int *n_global_out = nullptr)
+{
     TRY(run_localised(c, src, m, pose, nn, d2, honor_stop));
-    TRY(launch(c, K_FALLBACK, [&] {
-        return launch_fallback(src, pose, (const float4 *)c->bpts.p, (const float4 *)c->brick_box.p,
-                               (const float4 *)c->sb_box.p, c->target, c->n_target, (const int *)c->outside.p,
-                               (const int *)c->fb_list.p, (const int *)c->hv_list.p, (const uint2 *)c->hv_range.p,
-                               (const float4 *)c->csr.p, d, nn, d2, m, honor_stop, c->stream);
-    }));
+    TRY(run_global(c, src, m, pose, nn, d2, (const float4 *)c->csr.p, honor_stop, n_global_out));
     cudaError_t e = cudaEventRecord(c->ev_nns, c->stream);   // a later dilation waits for this search
     c->nns_in_capture = c->capturing;
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
@@ -1296,26 +1325,7 @@ vicp_status vicp_correspond(vicp_ctx *c, const float *src_xyzw, int32_t n_src, c
         return fail(c, VICP_ERR_STATE, "vicp_correspond needs vicp_build_grid and vicp_dilate first");
     TRY(ensure_query_buffers(c, n_src));
     const float4 *src = reinterpret_cast<const float4 *>(src_xyzw);
-    DevCtl *d = ctl_of(c);
-    if (n_fallback_out) {
-        // fb_count is zero between searches; the correspond kernel counts this
-        // search's global queries and the fallback kernel clears it again.
-        TRY(run_localised(c, src, n_src, pose_dev, nn_out, d2_out, 0));
-        cudaError_t e = cudaMemcpyAsync(n_fallback_out, &d->fb_count, sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                                        c->stream);
-        if (e != cudaSuccess)
-            return cuda_fail(c, e, "fallback count copy");
-        TRY(launch(c, K_FALLBACK, [&] {
-            return launch_fallback(src, pose_dev, (const float4 *)c->bpts.p, (const float4 *)c->brick_box.p,
-                                   (const float4 *)c->sb_box.p, c->target, c->n_target, (const int *)c->outside.p,
-                                   (const int *)c->fb_list.p, (const int *)c->hv_list.p,
-                                   (const uint2 *)c->hv_range.p, (const float4 *)c->csr.p, d, nn_out, d2_out, n_src, 0,
-                                   c->stream);
-        }));
-        e = cudaEventRecord(c->ev_nns, c->stream);   // a later dilation waits for this search
-        return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
-    }
-    return run_nns(c, src, n_src, pose_dev, nn_out, d2_out, 0);
+    return run_nns(c, src, n_src, pose_dev, nn_out, d2_out, 0, n_fallback_out);
 }
 
 vicp_status vicp_step(vicp_ctx *c, const float *src_xyzw, int32_t n_src, double *pose_dev, double *rmse_dev)
@@ -1580,20 +1590,9 @@ vicp_status vicp_fixed_correspond(vicp_ctx *c, const float *src_xyzw, int32_t n_
                                        nn_out, d2_out, (int *)c->fb_list.p, (int *)c->hv_list.p,
                                        (uint2 *)c->hv_range.p, d, c->stream);
     }));
-    if (n_fallback_out) {
-        cudaError_t e = cudaMemcpyAsync(n_fallback_out, &d->fb_count, sizeof(int32_t), cudaMemcpyDeviceToDevice,
-                                        c->stream);
-        if (e != cudaSuccess)
-            return cuda_fail(c, e, "fallback count copy");
-    }
-    // global searches over the brick level of the CSR build; dense segments
-    // are scanned in the slots
-    TRY(launch(c, K_FALLBACK, [&] {
-        return launch_fallback(src, pose_dev, (const float4 *)c->bpts.p, (const float4 *)c->brick_box.p,
-                               (const float4 *)c->sb_box.p, c->target, c->n_target, (const int *)c->outside.p,
-                               (const int *)c->fb_list.p, (const int *)c->hv_list.p, (const uint2 *)c->hv_range.p,
-                               (const float4 *)c->fslots.p, d, nn_out, d2_out, n_src, 0, c->stream);
-    }));
+    // global searches over the CSR build's grid and brick level; dense
+    // segments are scanned in the slots
+    TRY(run_global(c, src, n_src, pose_dev, nn_out, d2_out, (const float4 *)c->fslots.p, 0, n_fallback_out));
     cudaError_t e = cudaEventRecord(c->ev_nns, c->stream);
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
 }

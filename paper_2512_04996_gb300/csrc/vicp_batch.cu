@@ -581,23 +581,13 @@ __device__ bool grid_barrier(DevCtl *ctl, int *s_flag)
     return *s_flag != 0;
 }
 
-// The float pose of a pair, on every lane of a warp (lanes 0..11 convert one
-// entry each).
-__device__ __forceinline__ PoseF pose_f_warp(const double *__restrict__ pose)
+// The float pose of a pair, as phase 1 stored it.
+__device__ __forceinline__ PoseF load_posef(const float *__restrict__ posef, int pair)
 {
-    const int lane = threadIdx.x & 31;
-    const float v = lane < 12 ? __double2float_rn(pose[lane]) : 0.0f;
-    PoseF P;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-        const float x = __shfl_sync(FULL_MASK, v, k);
-        const int a = k >> 2, b = k & 3;
-        if (b < 3)
-            P.r[3 * a + b] = x;
-        else
-            P.t[a] = x;
-    }
-    return P;
+    static_assert(sizeof(PoseF) == 48, "PoseF layout");
+    const float4 *p = reinterpret_cast<const float4 *>(posef + 12 * pair);
+    const float4 a = __ldcg(p), b = __ldcg(p + 1), c = __ldcg(p + 2);
+    return PoseF{{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x}, {c.y, c.z, c.w}};
 }
 
 // ---------------------------------------------------------------------------
@@ -750,7 +740,7 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
     __shared__ BatchItem s_item;
     __shared__ int s_skip, s_flag, s_last;
     __shared__ unsigned long long s_cand;
-    __shared__ int s_fb, s_fb_base, s_hv, s_hv_base;
+    __shared__ int s_fb, s_fb_base, s_nr, s_nr_base, s_hv, s_hv_base;
     __shared__ float s_whi[WARPS][N_SUMS], s_wlo[WARPS][N_SUMS];
     __shared__ dfl s_tot[N_SUMS];
     extern __shared__ float s_dyn[];   // [2][WARPS][N_SUMS][33]
@@ -770,7 +760,7 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
             s_item = a.items[itx];
             s_skip = *(volatile const int *)&a.state[s_item.pair].stop;
             s_cand = 0ull;
-            s_fb = s_hv = 0;
+            s_fb = s_nr = s_hv = 0;
         }
         __syncthreads();
         const BatchItem it = s_item;
@@ -783,47 +773,61 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
         const BatchPair *bp = a.pairs + it.pair;
         const GridGeom g = bp->g;
         const long long vb = bp->vbase;
-        bool fall[PPT], heavy[PPT];
+        if (it.l0 == 0 && tid < 12)   // the pair's first item
+            a.posef[12 * it.pair + tid] = reinterpret_cast<const float *>(&s_pose)[tid];
+        const bool seeds = a.state[it.pair].n_outside <= NEAR_OUTSIDE_MAX;
+        bool far[PPT], near[PPT], heavy[PPT];
         unsigned ra[PPT], rb[PPT];
         unsigned cand = 0u;
 #pragma unroll
         for (int u = 0; u < PPT; ++u) {
             const int i = it.i0 + tid + TH * u;
-            fall[u] = heavy[u] = false;
+            far[u] = near[u] = heavy[u] = false;
             ra[u] = rb[u] = 0u;
-            if (i < it.i1) {
+            if (i < it.i1) {   // (as k_correspond)
                 const float3 s = transform_pt(P, __ldg(a.src + i));
-                const int v = voxel_key(g, s.x, s.y, s.z);
-                const int r = (v >= 0) ? __ldg(a.root + vb + v) : -1;
+                bool inside;
+                const int v = nearest_voxel(g, s, inside);
+                const int r = v >= 0 ? __ldg(a.root + vb + v) : -1;
+                far[u] = true;
+                unsigned dense = 0u;
                 if (r >= 0) {
                     const unsigned x0 = __ldg(a.off + vb + r);
-                    const unsigned x1 = max(x0, min(__ldg(a.off + vb + r + 1), (unsigned)a.n_stored));
+                    unsigned x1 = max(x0, min(__ldg(a.off + vb + r + 1), (unsigned)a.n_stored));
+                    dense = x1 - x0;
+                    if (!inside)   // only a seed
+                        x1 = min(x1, x0 + (unsigned)NEAR_SEED);
                     ra[u] = x0;
                     rb[u] = x1;
-                    cand += x1 - x0;
-                    heavy[u] = x1 - x0 > HEAVY;
-                    if (!heavy[u]) {
-                        const unsigned long long best = segment_min(a.csr, x0, x1, s);
-                        a.nn[i] = (int)(unsigned)best;
-                        a.d2[i] = __uint_as_float((unsigned)(best >> 32));
-                    }
-                } else {
-                    fall[u] = true;
+                    cand += inside ? dense : 0u;
+                    heavy[u] = inside && dense > HEAVY;
+                    far[u] = !inside;
+                }
+                if (!heavy[u]) {
+                    const unsigned long long best = segment_min(a.csr, ra[u], rb[u], s);
+                    a.nn[i] = (int)(unsigned)best;
+                    a.d2[i] = __uint_as_float((unsigned)(best >> 32));
+                    near[u] = far[u] && dense && seeds &&
+                              near_seed(s, __uint_as_float((unsigned)(best >> 32)), g.inv_h, dense);
+                    far[u] = far[u] && !near[u];
                 }
             }
         }
         // list the queries for phase 2: warp slots by shared atomics, one
         // global atomic per list and block
-        unsigned fm[PPT], hm[PPT];
-        int fb_w[PPT], hv_w[PPT];
+        unsigned fm[PPT], nm[PPT], hm[PPT];
+        int fb_w[PPT], nr_w[PPT], hv_w[PPT];
 #pragma unroll
         for (int u = 0; u < PPT; ++u) {
-            fm[u] = __ballot_sync(FULL_MASK, fall[u]);
+            fm[u] = __ballot_sync(FULL_MASK, far[u]);
+            nm[u] = __ballot_sync(FULL_MASK, near[u]);
             hm[u] = __ballot_sync(FULL_MASK, heavy[u]);
-            fb_w[u] = hv_w[u] = 0;
+            fb_w[u] = nr_w[u] = hv_w[u] = 0;
             if (lane == 0) {
                 if (fm[u])
                     fb_w[u] = atomicAdd(&s_fb, __popc(fm[u]));
+                if (nm[u])
+                    nr_w[u] = atomicAdd(&s_nr, __popc(nm[u]));
                 if (hm[u])
                     hv_w[u] = atomicAdd(&s_hv, __popc(hm[u]));
             }
@@ -838,6 +842,8 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
             atomicAdd(&ctl->stat_queries, (unsigned long long)(it.i1 - it.i0));
             if (s_fb)
                 s_fb_base = atomicAdd(&ctl->fb_count, s_fb);
+            if (s_nr)
+                s_nr_base = atomicAdd(&ctl->nr_count, s_nr);
             if (s_hv)
                 s_hv_base = atomicAdd(&ctl->hv_count, s_hv);
         }
@@ -845,8 +851,16 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
 #pragma unroll
         for (int u = 0; u < PPT; ++u) {
             const int i = it.i0 + tid + TH * u;
-            const int fbw = __shfl_sync(FULL_MASK, fb_w[u], 0), hvw = __shfl_sync(FULL_MASK, hv_w[u], 0);
-            if (fall[u]) {
+            const int fbw = __shfl_sync(FULL_MASK, fb_w[u], 0), nrw = __shfl_sync(FULL_MASK, nr_w[u], 0),
+                      hvw = __shfl_sync(FULL_MASK, hv_w[u], 0);
+            if (near[u]) {
+                const int slot = s_nr_base + nrw + __popc(nm[u] & lanemask_lt());
+                if (slot < a.list_cap)
+                    a.fb_list[a.list_cap - 1 - slot] = make_int2(it.pair, i);
+                else
+                    atomicOr(&ctl->err, DEVERR_BOUNDS);
+            }
+            if (far[u]) {
                 const int slot = s_fb_base + fbw + __popc(fm[u] & lanemask_lt());
                 if (slot < a.list_cap)
                     a.fb_list[slot] = make_int2(it.pair, i);
@@ -869,67 +883,122 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
     // ---- phase 2: dense segments, then global searches, a warp each -------
     {
         const int F = min(*(volatile int *)&ctl->fb_count, a.list_cap);
+        const int N = min(*(volatile int *)&ctl->nr_count, a.list_cap - F);
         const int Hv = min(*(volatile int *)&ctl->hv_count, a.list_cap);
         const int n_warps = gridDim.x * WARPS, gw = blockIdx.x * WARPS + warp;
-        unsigned long long examined = 0ull;
-        for (int qi = n_warps - 1 - gw; qi < Hv; qi += n_warps) {
-            const int4 e = a.hv_list[qi];
-            if ((unsigned)e.x >= (unsigned)a.n_pairs || (unsigned)e.y >= (unsigned)a.list_cap || e.z > e.w ||
-                (unsigned)e.w > (unsigned)a.n_stored) {   // a stale entry: skip it, report it
-                if (lane == 0)
+        unsigned long long examined = 0ull;   // far queries: every lane counts the same
+        unsigned examined_near = 0u;          // near queries: each lane its own
+        const int lanes = n_warps * 32;
+        {   // dense segments, 8 to 32 lanes each
+            const int shift = group_shift(Hv, lanes, HEAVY_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
+            const int sub = lane & (G - 1);
+            for (int q0 = (n_warps - 1 - gw) * pack; q0 < Hv; q0 += n_warps * pack) {
+                const int q = q0 + (lane >> shift);
+                const int4 e = q < Hv ? a.hv_list[q] : make_int4(-1, -1, 0, 0);
+                const bool on = (unsigned)e.x < (unsigned)a.n_pairs && (unsigned)e.y < (unsigned)a.list_cap &&
+                                e.z <= e.w && (unsigned)e.w <= (unsigned)a.n_stored;
+                if (!on && q < Hv)   // a stale entry: skip it, report it
                     atomicOr(&ctl->err, DEVERR_BOUNDS);
-                continue;
-            }
-            const PoseF P = pose_f_warp(a.pose + 16 * e.x);
-            const float3 s = transform_pt(P, __ldg(a.src + e.y));
-            unsigned long long unused = 0ull;
-            const unsigned long long best = scan_run(a.csr, (unsigned)e.z, (unsigned)e.w, s, lane, ~0ull, unused);
-            if (lane == 0) {
-                a.nn[e.y] = (int)(unsigned)best;
-                a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
+                unsigned long long best = ~0ull;
+                if (on)
+                    best = group_scan(a.csr, (unsigned)e.z, (unsigned)e.w,
+                                      transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y)), sub, G);
+                best = group_min(best, G);
+                if (on && sub == 0) {
+                    a.nn[e.y] = (int)(unsigned)best;
+                    a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
+                }
             }
         }
-        // global queries in chunks of FB_CHUNK, each chunk to whichever warp is
+        // far queries: a first chunk per warp, then chunks to whichever warp is
         // free (a ticket per chunk): their costs vary widely, and a fixed share
         // per warp leaves the whole grid waiting at the barrier for the warp
         // that drew the slowest ones
-        constexpr int FB_CHUNK = 4;
-        for (;;) {
-            int q0 = 0;
-            if (lane == 0)
-                q0 = FB_CHUNK * (int)atomicAdd(&ctl->fb_next, 1u);
-            q0 = __shfl_sync(FULL_MASK, q0, 0);
-            if (q0 >= F)
+        const int far_chunk = min(max(F / (4 * n_warps), 1), 4);
+        for (int q0 = gw * far_chunk; q0 < F;) {
+            for (int qi = q0; qi < min(q0 + far_chunk, F); ++qi) {
+                const int2 e = a.fb_list[qi];
+                if ((unsigned)e.x >= (unsigned)a.n_pairs || (unsigned)e.y >= (unsigned)a.list_cap) {
+                    if (lane == 0)   // a stale entry: skip it, report it
+                        atomicOr(&ctl->err, DEVERR_BOUNDS);
+                    continue;
+                }
+                const BatchPair *bp = a.pairs + e.x;
+                const float3 s = transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y));
+                const int tbase = bp->tbase;
+                const unsigned long long best = global_search(
+                    s, a.bpts, a.bbox + 2 * bp->bbase, a.sb_box + 2 * bp->sbbase, a.state[e.x].n_super, a.tgt + tbase,
+                    bp->n_tgt, a.outside + tbase, a.state[e.x].n_outside, lane, examined,
+                    nn_key(__ldcg(a.d2 + e.y), __ldcg(a.nn + e.y)));
+                __syncwarp();   // every lane has read the seed
+                if (lane == 0) {
+                    a.nn[e.y] = (int)(unsigned)best;
+                    a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
+                }
+            }
+            if ((long long)n_warps * far_chunk >= F)
                 break;
-            for (int qi = q0; qi < min(q0 + FB_CHUNK, F); ++qi) {
-            const int2 e = a.fb_list[qi];
-            if ((unsigned)e.x >= (unsigned)a.n_pairs || (unsigned)e.y >= (unsigned)a.list_cap) {
-                if (lane == 0)   // a stale entry: skip it, report it
-                    atomicOr(&ctl->err, DEVERR_BOUNDS);
-                continue;
-            }
-            const BatchPair *bp = a.pairs + e.x;
-            const PoseF P = pose_f_warp(a.pose + 16 * e.x);
-            const float3 s = transform_pt(P, __ldg(a.src + e.y));
-            const int tbase = bp->tbase;
-            const unsigned long long best =
-                global_search(s, a.bpts, a.bbox + 2 * bp->bbase, a.sb_box + 2 * bp->sbbase, a.state[e.x].n_super,
-                              a.tgt + tbase, bp->n_tgt, a.outside + tbase, a.state[e.x].n_outside, lane, examined);
-            if (lane == 0) {
-                a.nn[e.y] = (int)(unsigned)best;
-                a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
-            }
+            if (lane == 0)
+                q0 = far_chunk * (n_warps + (int)atomicAdd(&ctl->fb_next, 1u));
+            q0 = __shfl_sync(FULL_MASK, q0, 0);
+        }
+        // near queries: 8 to 32 lanes each, a warp's worth at a time, in the
+        // same way
+        {
+            const int shift = group_shift(N, lanes, NEAR_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
+            const int sub = lane & (G - 1);
+            const int packs = (N + pack - 1) / pack, chunk = min(max(packs / (4 * n_warps), 1), 8);
+            for (int p0 = gw * chunk; p0 < packs;) {
+                for (int p = p0; p < min(p0 + chunk, packs); ++p) {
+                    const int q = p * pack + (lane >> shift);
+                    const int2 e = q < N ? a.fb_list[a.list_cap - 1 - q] : make_int2(-1, -1);
+                    const bool on = (unsigned)e.x < (unsigned)a.n_pairs && (unsigned)e.y < (unsigned)a.list_cap;
+                    if (!on && q < N)   // a stale entry: skip it, report it
+                        atomicOr(&ctl->err, DEVERR_BOUNDS);
+                    const BatchPair *bp = a.pairs + (on ? e.x : 0);
+                    const long long vb = bp->vbase;
+                    float3 s = make_float3(0.0f, 0.0f, 0.0f);
+                    unsigned long long best = ~0ull;
+                    int no = 0;
+                    if (on) {
+                        s = transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y));
+                        best = nn_key(__ldcg(a.d2 + e.y), __ldcg(a.nn + e.y));
+                        no = a.state[e.x].n_outside;
+                        const int tbase = bp->tbase;
+                        for (int o = sub; o < no; o += G) {   // target points outside the grid
+                            const int j = __ldg(a.outside + tbase + o);
+                            best = umin64(best, nn_key(dist2(s, __ldg(a.tgt + tbase + j)), j));
+                        }
+                        examined_near += sub == 0 ? (unsigned)no : 0u;
+                    }
+                    if (__any_sync(FULL_MASK, no > 0))
+                        best = group_min(best, G);
+                    best = near_search(bp->g, CsrRows{a.occ + (vb >> 5), a.off + vb, (unsigned)a.n_stored, a.csr}, s,
+                                       best, on, sub, G, examined_near);
+                    if (on && sub == 0) {
+                        a.nn[e.y] = (int)(unsigned)best;
+                        a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
+                    }
+                }
+                if ((long long)n_warps * chunk >= packs)
+                    break;
+                if (lane == 0)
+                    p0 = chunk * (n_warps + (int)atomicAdd(&ctl->nr_next, 1u));
+                p0 = __shfl_sync(FULL_MASK, p0, 0);
             }
         }
+        examined = warp_sum_u64((lane == 0 ? examined : 0ull) + examined_near);
         if (lane == 0 && examined)
             atomicAdd(&ctl->stat_global_cand, examined);
         if (!grid_barrier(ctl, &s_flag))
             return;
         if (blockIdx.x == 0 && tid == 0) {   // every block has read the list lengths
-            ctl->stat_fallbacks += (unsigned long long)F;
+            ctl->stat_fallbacks += (unsigned long long)(F + N);
             ctl->fb_count = 0;
+            ctl->nr_count = 0;
             ctl->hv_count = 0;
             ctl->fb_next = 0u;
+            ctl->nr_next = 0u;
         }
     }
     if (a.search_only)

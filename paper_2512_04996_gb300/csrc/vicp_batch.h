@@ -85,7 +85,10 @@ struct BatchIterArgs {
     const int *outside;         // pooled (at tbase) lists of target points outside each grid
     int *nn;                    // [M] pair-local target index of each source point
     float *d2;                  // [M] squared distance
-    int2 *fb_list;              // global-search queries (pair, pooled source index)
+    const unsigned *occ;        // pooled occupancy bits
+    float *posef;               // [P][12] the poses rounded to float (PoseF), written by phase 1 for phase 2
+    int2 *fb_list;              // global-search queries (pair, pooled source index): far ones from the
+                                // front, near ones (vicp_search.cuh) from the back
     int4 *hv_list;              // dense segments (pair, pooled source index, begin, end)
     int list_cap;               // capacity of each list (M)
     float2 *partials;           // [n_items][16] double-float sums per item

@@ -71,7 +71,7 @@ struct vicp_batch {
     BBuf counts, off, root, ring, inter, occ, desc, tile_sum, rows, dirty;
     BBuf bcounts, boff, blist, brange, bslot, boxord, bbox, sb_box;
     BBuf keys, ids, csr, bpts, outside;
-    BBuf nn, d2, fb_list, hv_list, partials, sitems;
+    BBuf nn, d2, fb_list, hv_list, partials, sitems, posef;
     BBuf pairs_d, state, pose, pose_save, titems, ustart_xy_d, ustart_z_d, bb, ctl;
     BBuf hsrc, htgt;
 };
@@ -445,6 +445,7 @@ vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
     BTRY(bensure(b, b->partials, items.size() * REDUCE_VALUES * sizeof(float2), "item sums"));
     BTRY(bensure(b, b->nn, (size_t)M * 4, "nn"));
     BTRY(bensure(b, b->d2, (size_t)M * 4, "d2"));
+    BTRY(bensure(b, b->posef, (size_t)P * sizeof(PoseF), "float poses"));
     BTRY(bensure(b, b->fb_list, (size_t)M * sizeof(int2), "global-search list"));
     BTRY(bensure(b, b->hv_list, (size_t)M * sizeof(int4), "dense segment list"));
     BCUDA(b, cudaMemcpyAsync(b->sitems.p, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice, st),
@@ -468,10 +469,8 @@ vicp_status reset_loop(vicp_batch *b)
                             sizeof(BatchState) - offsetof(BatchState, items_done), b->P, st),
           "loop state reset");
     DevCtl *d = bctl(b);
-    BCUDA(b, cudaMemsetAsync(&d->fb_count, 0, sizeof(int), st), "list reset");
-    BCUDA(b, cudaMemsetAsync(&d->hv_count, 0, sizeof(int), st), "list reset");
-    BCUDA(b, cudaMemsetAsync(&d->bar_count, 0, sizeof(unsigned), st), "barrier reset");
-    BCUDA(b, cudaMemsetAsync(&d->fb_next, 0, sizeof(unsigned), st), "ticket reset");
+    static_assert(offsetof(DevCtl, bar_count) - offsetof(DevCtl, fb_count) == 20, "list fields");
+    BCUDA(b, cudaMemsetAsync(&d->fb_count, 0, 24, st), "list, ticket and barrier reset");
     return VICP_OK;
 }
 
@@ -496,6 +495,8 @@ BatchIterArgs iter_args(vicp_batch *b, const float4 *src, double *pose, int *nn,
     a.outside = (const int *)b->outside.p;
     a.nn = nn;
     a.d2 = d2;
+    a.occ = (const unsigned *)b->occ.p;
+    a.posef = (float *)b->posef.p;
     a.fb_list = (int2 *)b->fb_list.p;
     a.hv_list = (int4 *)b->hv_list.p;
     a.list_cap = b->M;
@@ -692,7 +693,7 @@ void vicp_batch_destroy(vicp_batch *b)
     BBuf *all[] = {&b->counts, &b->off, &b->root, &b->ring, &b->inter, &b->occ, &b->desc, &b->tile_sum, &b->rows,
                    &b->dirty, &b->bcounts, &b->boff, &b->blist, &b->brange, &b->bslot, &b->boxord, &b->bbox,
                    &b->sb_box, &b->keys, &b->ids, &b->csr, &b->bpts, &b->outside, &b->nn, &b->d2, &b->fb_list,
-                   &b->hv_list, &b->partials, &b->sitems, &b->pairs_d, &b->state, &b->pose, &b->pose_save,
+                   &b->hv_list, &b->partials, &b->sitems, &b->posef, &b->pairs_d, &b->state, &b->pose, &b->pose_save,
                    &b->titems, &b->ustart_xy_d, &b->ustart_z_d, &b->bb, &b->ctl, &b->hsrc, &b->htgt};
     for (BBuf *x : all)
         bfree(b, *x);

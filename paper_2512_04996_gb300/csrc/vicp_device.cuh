@@ -58,20 +58,23 @@ constexpr unsigned DEVERR_CAPACITY = 8u;     // a hashed voxel table could not t
 // Per-context control block in device memory.  Kernels of one stream use it
 // in launch order; the comments say which kernel writes each field.
 struct DevCtl {
-    unsigned bar_count;     // batched iteration: blocks arrived at the grid barrier
     unsigned scan_epoch;    // scan: descriptor epoch; bumped by the histogram kernel
     int n_outside;          // scatter: target points outside the grid; reset by histogram
     int n_bricks;           // brick list length; reset by histogram
-    int fb_count;           // correspond: fallback queries; reset by the fallback kernel
-    unsigned fb_done;       // fallback: finished blocks (the last one resets fb_count)
+    int n_super;            // non-empty super-bricks; reset by the histogram
     unsigned err;           // DEVERR_* bits; cleared by the host
     unsigned max_count;     // memory report: largest voxel count
     unsigned occupied;      // memory report: occupied voxels
     unsigned red_done;      // reduction: finished blocks (the last one solves and resets it)
-    int hv_count;           // correspond: dense segments listed; reset by the fallback kernel
+    unsigned fb_done;       // fallback: finished blocks (the last one resets the list lengths)
     unsigned bar_gen;       // batched iteration: grid barrier generation
-    int n_super;            // non-empty super-bricks; reset by the histogram
-    unsigned fb_next;       // batched iteration: next chunk of listed global queries; reset with fb_count
+    // Search lists, reset together by the host before batched iterations.
+    int fb_count;           // correspond: far global queries listed; reset by the fallback kernel
+    int nr_count;           // correspond: near global queries listed; reset with fb_count
+    int hv_count;           // correspond: dense segments listed; reset with fb_count
+    unsigned fb_next;       // batched iteration: next chunk of far queries; reset with fb_count
+    unsigned nr_next;       // batched iteration: next chunk of near queries; reset with fb_count
+    unsigned bar_count;     // batched iteration: blocks arrived at the grid barrier
     // Work counters (added by the search kernels, read and cleared by the host).
     unsigned long long stat_queries;       // source points searched
     unsigned long long stat_fallbacks;     // of which took the global search
@@ -83,7 +86,7 @@ struct DevCtl {
     double prev_rmse;
     double last_rmse;
 };
-static_assert(sizeof(DevCtl) == 112, "DevCtl layout");
+static_assert(sizeof(DevCtl) == 120, "DevCtl layout");
 
 // Rigid transform rounded to float: R row-major, t.
 struct PoseF {

@@ -137,8 +137,10 @@ int dilate_hashed_blocks(const GridGeom &g, int L);
 long long dilate_units(const GridGeom &g);
 long long dilate_column_units(const GridGeom &g);
 // The localised search lists queries whose root segment is long (with the
-// segment) in hv_list / hv_range and queries without a root in fb_list; the
-// fallback kernel then answers both lists.
+// segment) in hv_list / hv_range, and queries without a root in fb_list: far
+// ones from its front, near ones (vicp_search.cuh) from its back, each with
+// a known point's key or all ones as the seed in its nn / d2 entries.  The
+// fallback kernel then answers the lists.
 cudaError_t launch_correspond(const float4 *src, int m, const double *pose, const GridGeom &g, const int *root,
                               const unsigned *off, const float4 *csr, int n_cap, int *nn, float *d2,
                               int *fb_list, int *hv_list, uint2 *hv_range, DevCtl *ctl, int honor_stop,
@@ -162,10 +164,28 @@ cudaError_t launch_correspond_fixed(const float4 *src, int m, const double *pose
 // (one word) is added to.
 cudaError_t launch_fixed_scatter(const float4 *pts, int n, const GridGeom &g, unsigned C, unsigned *count,
                                  float4 *slots, unsigned *overflow, cudaStream_t st);
-cudaError_t launch_fallback(const float4 *src, const double *pose, const float4 *bpts, const float4 *bbox,
-                            const float4 *sb_box, const float4 *tgt, int n_tgt, const int *outside, const int *fb_list,
-                            const int *hv_list, const uint2 *hv_range, const float4 *csr, DevCtl *ctl, int *nn,
-                            float *d2, int m, int honor_stop, cudaStream_t st);
+// The global searches and dense segments the localised search listed.
+struct FallbackArgs {
+    const float4 *src;
+    const double *pose;
+    GridGeom g;
+    const unsigned *occ, *off;   // voxel occupancy bits; offsets by voxel, or by slot of okeys
+    const float4 *csr;           // the CSR store they index
+    HashTable okeys;             // sparse grid: the occupied-voxel table; keys null: dense
+    const float4 *bpts, *bbox, *sb_box;   // brick level
+    const float4 *tgt;
+    int n_tgt;
+    const int *outside;
+    const int *fb_list, *hv_list;   // far queries from the front, near ones from the back; dense segments
+    const uint2 *hv_range;
+    const float4 *hv_store;      // the store the dense segments lie in (csr, or the fixed-capacity slots)
+    DevCtl *ctl;
+    int *nn;
+    float *d2;
+    int m, honor_stop;
+    int *n_global_out;           // may be null: receives the number of global searches
+};
+cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st);
 // Standalone voxel histogram (vicp_hist.cu): method 0 warp-aggregated,
 // 1 per-block shared-memory hash; adds to counts.
 cudaError_t launch_voxel_histogram(const float4 *pts, int n, const GridGeom &g, int method, int *keys,

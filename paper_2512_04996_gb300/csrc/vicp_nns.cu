@@ -17,6 +17,10 @@ namespace vicp {
 // for it.  Both lists get one global atomic per block.
 // ---------------------------------------------------------------------------
 constexpr int CORR_THREADS = 512;
+// Up to this many source points the global queries are so few that each has
+// a warp of its own, and the brick search (with the seed) is the shorter
+// chain: one step of 1,000 points on a 4k object 22.2 us against 24.6.
+constexpr int NEAR_MIN_QUERIES = 16384;
 
 // Segment of a root voxel in the CSR store: [off[r], off[r + 1]) (clamped to
 // the store's length).
@@ -93,60 +97,90 @@ __global__ void __launch_bounds__(CORR_THREADS) k_correspond(const float4 *__res
         return;
     __shared__ PoseF sp;
     __shared__ unsigned long long s_cand;   // block totals: one global atomic each
-    __shared__ int s_fb, s_fb_base, s_hv, s_hv_base;
-    if (threadIdx.x == 0) {
+    __shared__ int s_fb, s_fb_base, s_nr, s_nr_base, s_hv, s_hv_base, s_no;
+    if (threadIdx.x == 32) {   // (not the warp that loads the pose: the round trips overlap)
         s_cand = 0ull;
-        s_fb = s_hv = 0;
+        s_fb = s_nr = s_hv = 0;
+        s_no = __ldcg(&ctl->n_outside);
     }
     load_pose_f_block(pose, sp);   // also orders the initialisation above
     const PoseF P = sp;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
-    bool fall = false, heavy = false;
+    bool far = false, near = false, heavy = false;
     unsigned cand = 0u, a = 0u, b = 0u;
     if (i < m) {
         const float3 s = transform_pt(P, __ldg(src + i));
-        const int v = voxel_key(g, s.x, s.y, s.z);
-        const int r = (v >= 0) ? root(v) : -1;
+        bool inside;
+        const int v = nearest_voxel(g, s, inside);
+        const int r = v >= 0 ? root(v) : -1;
+        far = true;
+        unsigned dense = 0u;
         if (r >= 0) {
             seg.range(r, a, b);
-            cand = b - a;
+            dense = b - a;
+            if (!inside)   // only a seed
+                b = min(b, a + (unsigned)NEAR_SEED);
+            cand = inside ? dense : 0u;
             heavy = cand > HEAVY;
-            if (!heavy) {
-                const unsigned long long best = segment_min(csr, a, b, s);
-                nn[i] = (int)(unsigned)best;
-                d2[i] = __uint_as_float((unsigned)(best >> 32));
-            }
-        } else {
-            fall = true;
+            far = !inside;
+        }
+        if (!heavy) {   // (far without a label: an empty run, no seed)
+            const unsigned long long best = segment_min(csr, a, b, s);
+            nn[i] = (int)(unsigned)best;
+            d2[i] = __uint_as_float((unsigned)(best >> 32));
+            near = far && dense && m > NEAR_MIN_QUERIES && s_no <= NEAR_OUTSIDE_MAX &&
+                   near_seed(s, __uint_as_float((unsigned)(best >> 32)), g.inv_h, dense);
+            far = far && !near;
         }
     }
-    const unsigned fm = __ballot_sync(FULL_MASK, fall), hm = __ballot_sync(FULL_MASK, heavy);
     const unsigned long long wc = warp_sum_u64(cand);
-    int fb_base = 0, hv_base = 0;
+    unsigned fm = 0u, nm = 0u, hm = 0u;
+    int fb_base = 0, nr_base = 0, hv_base = 0;
+    const bool lists = __any_sync(FULL_MASK, far || near || heavy);
+    if (lists) {
+        fm = __ballot_sync(FULL_MASK, far);
+        nm = __ballot_sync(FULL_MASK, near);
+        hm = __ballot_sync(FULL_MASK, heavy);
+    }
     if (lane == 0) {
         if (wc)
             atomicAdd(&s_cand, wc);
         if (fm)
             fb_base = atomicAdd(&s_fb, __popc(fm));
+        if (nm)
+            nr_base = atomicAdd(&s_nr, __popc(nm));
         if (hm)
             hv_base = atomicAdd(&s_hv, __popc(hm));
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    // a thread of another warp for each counter: the round trips overlap
+    if (threadIdx.x == 0 && s_fb)
+        s_fb_base = atomicAdd(&ctl->fb_count, s_fb);
+    if (threadIdx.x == 32 && s_nr)
+        s_nr_base = atomicAdd(&ctl->nr_count, s_nr);
+    if (threadIdx.x == 64 && s_hv)
+        s_hv_base = atomicAdd(&ctl->hv_count, s_hv);
+    if (threadIdx.x == 96) {
         if (s_cand)
             atomicAdd(&ctl->stat_local_cand, s_cand);
         if (blockIdx.x == 0)
             atomicAdd(&ctl->stat_queries, (unsigned long long)m);
-        if (s_fb)
-            s_fb_base = atomicAdd(&ctl->fb_count, s_fb);
-        if (s_hv)
-            s_hv_base = atomicAdd(&ctl->hv_count, s_hv);
     }
     __syncthreads();
+    if (!lists)
+        return;
     fb_base = __shfl_sync(FULL_MASK, fb_base, 0);
+    nr_base = __shfl_sync(FULL_MASK, nr_base, 0);
     hv_base = __shfl_sync(FULL_MASK, hv_base, 0);
-    if (fall) {
+    if (near) {   // from the list's end: a query is in one of the two at most
+        const int slot = s_nr_base + nr_base + __popc(nm & lanemask_lt());
+        if (slot < m)
+            fb_list[m - 1 - slot] = i;
+        else
+            atomicOr(&ctl->err, DEVERR_BOUNDS);
+    }
+    if (far) {
         const int slot = s_fb_base + fb_base + __popc(fm & lanemask_lt());
         if (slot < m)
             fb_list[slot] = i;
@@ -199,13 +233,15 @@ cudaError_t launch_correspond_fixed(const float4 *src, int m, const double *pose
 // ---------------------------------------------------------------------------
 // Global search ("Globalsearch" of Alg. 4) of the queries the localised
 // search listed (global_search: a warp per query over the brick levels), and
-// the dense root segments it left (all lanes of a warp scan one).
+// the near queries and dense root segments it listed (a group of 8 to 32
+// lanes each).
 //
-// Scheduling without global atomics: block b takes the list entries b,
-// b + B, b + 2B, ... of both lists (B blocks; strided, so that a block's
-// share mixes the regions of the source cloud and the shares cost about the
-// same), global queries first and dense segments after them, and its warps
-// take these items one at a time from a shared-memory counter.  Per-query
+// Scheduling without global atomics: block b takes the items b, b + B,
+// b + 2B, ... of every list (B blocks; strided, so that a block's share
+// mixes the regions of the source cloud and the shares cost about the
+// same), far queries first, then a warp's worth of near queries or of dense
+// segments at a time, and its warps take these items one at a time from a
+// shared-memory counter.  Per-query
 // costs vary several-fold, so the warps of a block balance each other; the
 // shares balance the blocks.  (A single global ticket counter would put one
 // same-address atomic per item, plus one per warp at the end, into the L2
@@ -214,13 +250,17 @@ cudaError_t launch_correspond_fixed(const float4 *src, int m, const double *pose
 // kernel's duration.)
 // ---------------------------------------------------------------------------
 constexpr int FB_THREADS = 256;
-constexpr int FB_WARPS = FB_THREADS / 32;
 
-// Entries b, b + B, ... below n: how many.
-__device__ __forceinline__ int strided_share(int n, int b, int B) { return n > b ? (n - 1 - b) / B + 1 : 0; }
+// Entries b, b + B, ... below n: how many (without a division while the
+// blocks' shares are at most one).
+__device__ __forceinline__ int strided_share(int n, int b, int B)
+{
+    return n <= b ? 0 : (n - b <= B ? 1 : (n - 1 - b) / B + 1);
+}
 
+template <class Rows>
 __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__restrict__ src,
-                                                         const double *__restrict__ pose,
+                                                         const double *__restrict__ pose, GridGeom g, Rows rows,
                                                          const float4 *__restrict__ bpts,
                                                          const float4 *__restrict__ bbox,
                                                          const float4 *__restrict__ sb_box,
@@ -231,39 +271,47 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
                                                          const uint2 *__restrict__ hv_range,
                                                          const float4 *__restrict__ csr,
                                                          DevCtl *__restrict__ ctl, int *__restrict__ nn,
-                                                         float *__restrict__ d2, int m, int honor_stop)
+                                                         float *__restrict__ d2, int m, int honor_stop,
+                                                         int *__restrict__ n_global_out)
 {
     pdl_begin();
     if (honor_stop && *(volatile int *)&ctl->stop)
         return;   // the correspond kernel appended nothing either
     __shared__ PoseF sp;
     __shared__ unsigned long long s_examined;   // block total: one global atomic
-    __shared__ int s_F, s_Hv, s_ns, s_no;
+    __shared__ int s_n[5];                      // far, near, dense segments listed; super-bricks; targets outside
     __shared__ unsigned s_next;                 // next item of this block's share
-    if (threadIdx.x == 0) {
+    if (threadIdx.x >= 32 && threadIdx.x < 37) {   // (not the warp that loads the pose: the round trips overlap)
+        const int k = threadIdx.x - 32;
+        s_n[k] = __ldcg(k == 0 ? &ctl->fb_count : (k == 1 ? &ctl->nr_count : (k == 2 ? &ctl->hv_count :
+                        (k == 3 ? &ctl->n_super : &ctl->n_outside))));
+    }
+    if (threadIdx.x == 64) {
         s_examined = 0ull;
-        s_F = min(*(volatile int *)&ctl->fb_count, m);
-        s_Hv = min(*(volatile int *)&ctl->hv_count, m);
-        s_ns = *(volatile int *)&ctl->n_super;
-        s_no = *(volatile int *)&ctl->n_outside;
         s_next = 0u;
     }
     load_pose_f_block(pose, sp);   // also orders the initialisation above
     const PoseF P = sp;
     const int lane = threadIdx.x & 31;
-    const int F = s_F, Hv = s_Hv, ns = s_ns, no = s_no;
+    const int F = min(s_n[0], m), N = min(s_n[1], m - F), Hv = min(s_n[2], m), ns = s_n[3], no = s_n[4];
     const int B = (int)gridDim.x, b = (int)blockIdx.x;
-    const int nG = strided_share(F, b, B), nH = strided_share(Hv, b, B);
-    unsigned long long examined = 0ull;   // every lane counts the same; lane 0 reports
+    // lanes a near query and a dense segment get (2^...), and how many of
+    // them a warp takes at a time (2^...)
+    const int gN = group_shift(N, B * FB_THREADS, NEAR_SHIFT_MIN), gH = group_shift(Hv, B * FB_THREADS, HEAVY_SHIFT_MIN);
+    const int packN = 5 - gN, packH = 5 - gH;
+    const int nG = strided_share(F, b, B), nN = strided_share((N + (1 << packN) - 1) >> packN, b, B),
+              nH = strided_share((Hv + (1 << packH) - 1) >> packH, b, B);
+    unsigned long long examined = 0ull;   // far queries: every lane counts the same; lane 0 reports
+    unsigned examined_near = 0u;          // near queries: each lane its own
 
     for (;;) {
         int k = 0;
         if (lane == 0)
             k = (int)atomicAdd(&s_next, 1u);
         k = __shfl_sync(FULL_MASK, k, 0);
-        if (k >= nG + nH)
+        if (k >= nG + nN + nH)
             break;
-        if (k < nG) {   // a global query
+        if (k < nG) {   // a far query
             const int i = __ldg(fb_list + b + k * B);
             if ((unsigned)i >= (unsigned)m) {   // a stale entry: skip it, report it
                 if (lane == 0)
@@ -271,25 +319,50 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
                 continue;
             }
             const float3 s = transform_pt(P, __ldg(src + i));
-            const unsigned long long best =
-                global_search(s, bpts, bbox, sb_box, ns, tgt, n_tgt, outside, no, lane, examined);
+            const unsigned long long best = global_search(s, bpts, bbox, sb_box, ns, tgt, n_tgt, outside, no, lane,
+                                                          examined, nn_key(d2[i], nn[i]));
+            __syncwarp();   // every lane has read the seed
             if (lane == 0) {
                 nn[i] = (int)(unsigned)best;
                 d2[i] = __uint_as_float((unsigned)(best >> 32));
             }
-        } else {        // a dense root segment: all lanes scan it
-            const int qi = b + (k - nG) * B;
-            const int i = __ldg(hv_list + qi);
-            const uint2 r = __ldg(hv_range + qi);
-            if ((unsigned)i >= (unsigned)m) {
-                if (lane == 0)
-                    atomicOr(&ctl->err, DEVERR_BOUNDS);
-                continue;
+        } else if (k < nG + nN) {   // near queries
+            const int G = 1 << gN, q = ((b + (k - nG) * B) << packN) + (lane >> gN), sub = lane & (G - 1);
+            const int i = q < N ? __ldg(fb_list + m - 1 - q) : -1;
+            const bool on = (unsigned)i < (unsigned)m;
+            if (!on && q < N)   // a stale entry: skip it, report it
+                atomicOr(&ctl->err, DEVERR_BOUNDS);
+            float3 s = make_float3(0.0f, 0.0f, 0.0f);
+            unsigned long long best = ~0ull;
+            if (on) {
+                s = transform_pt(P, __ldg(src + i));
+                best = nn_key(d2[i], nn[i]);
+                for (int o = sub; o < no; o += G) {   // target points outside the grid
+                    const int j = __ldg(outside + o);
+                    best = umin64(best, nn_key(dist2(s, __ldg(tgt + j)), j));
+                }
+                examined_near += sub == 0 ? (unsigned)no : 0u;
             }
-            const float3 s = transform_pt(P, __ldg(src + i));
-            unsigned long long unused = 0ull;
-            const unsigned long long best = scan_run(csr, r.x, r.y, s, lane, ~0ull, unused);
-            if (lane == 0) {
+            if (no > 0)
+                best = group_min(best, G);
+            best = near_search(g, rows, s, best, on, sub, G, examined_near);
+            if (on && sub == 0) {
+                nn[i] = (int)(unsigned)best;
+                d2[i] = __uint_as_float((unsigned)(best >> 32));
+            }
+        } else {        // dense root segments
+            const int G = 1 << gH, q = ((b + (k - nG - nN) * B) << packH) + (lane >> gH), sub = lane & (G - 1);
+            const int i = q < Hv ? __ldg(hv_list + q) : -1;
+            const bool on = (unsigned)i < (unsigned)m;
+            if (!on && q < Hv)
+                atomicOr(&ctl->err, DEVERR_BOUNDS);
+            unsigned long long best = ~0ull;
+            if (on) {
+                const uint2 r = __ldg(hv_range + q);
+                best = group_scan(csr, r.x, r.y, transform_pt(P, __ldg(src + i)), sub, G);
+            }
+            best = group_min(best, G);
+            if (on && sub == 0) {
                 nn[i] = (int)(unsigned)best;
                 d2[i] = __uint_as_float((unsigned)(best >> 32));
             }
@@ -297,6 +370,8 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
     }
     // work counter: one global atomic per block; the last block to finish
     // clears the list lengths for the next search
+    examined = (lane == 0 ? examined : 0ull) + examined_near;
+    examined = warp_sum_u64(examined);
     if (lane == 0 && examined)
         atomicAdd(&s_examined, examined);
     __syncthreads();
@@ -306,31 +381,42 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
         __threadfence();
         const unsigned done = atomicAdd(&ctl->fb_done, 1u);
         if (done == gridDim.x - 1) {
-            ctl->stat_fallbacks += (unsigned long long)F;
+            ctl->stat_fallbacks += (unsigned long long)(F + N);
+            if (n_global_out)
+                *n_global_out = F + N;
             ctl->fb_count = 0;
+            ctl->nr_count = 0;
             ctl->hv_count = 0;
             ctl->fb_done = 0u;
         }
     }
 }
 
-cudaError_t launch_fallback(const float4 *src, const double *pose, const float4 *bpts, const float4 *bbox,
-                            const float4 *sb_box, const float4 *tgt, int n_tgt, const int *outside, const int *fb_list,
-                            const int *hv_list, const uint2 *hv_range, const float4 *csr, DevCtl *ctl, int *nn,
-                            float *d2, int m, int honor_stop, cudaStream_t st)
+template <class Rows>
+static cudaError_t run_fallback(const FallbackArgs &a, const Rows &rows, cudaStream_t st)
 {
-    // as many warps as can be resident
+    // as many warps as can be resident, and no more than there are queries
     static int per_sm = 0;
     if (per_sm == 0) {
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fallback, FB_THREADS, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fallback<Rows>, FB_THREADS, 0);
         if (e != cudaSuccess || per_sm < 1)
             per_sm = 1;
     }
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return launch_kernel(k_fallback, dim3(sms * per_sm), dim3(FB_THREADS), 0, st, src, pose, bpts, bbox, sb_box, tgt,
-                         n_tgt, outside, fb_list, hv_list, hv_range, csr, ctl, nn, d2, m, honor_stop);
+    const int blocks = min(sms * per_sm, (a.m + FB_THREADS / 32 - 1) / (FB_THREADS / 32));
+    return launch_kernel(k_fallback<Rows>, dim3(blocks), dim3(FB_THREADS), 0, st, a.src, a.pose, a.g, rows, a.bpts,
+                         a.bbox, a.sb_box, a.tgt, a.n_tgt, a.outside, a.fb_list, a.hv_list, a.hv_range, a.hv_store,
+                         a.ctl, a.nn, a.d2, a.m, a.honor_stop, a.n_global_out);
+}
+
+cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st)
+{
+    if (a.okeys.keys)
+        return run_fallback(a, HashedRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr, a.okeys.keys, a.okeys.mask,
+                                          a.okeys.shift}, st);
+    return run_fallback(a, CsrRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr}, st);
 }
 
 }  // namespace vicp

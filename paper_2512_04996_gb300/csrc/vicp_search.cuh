@@ -15,12 +15,14 @@ namespace vicp {
 constexpr unsigned HEAVY = 48;
 
 // Nearest point of the CSR run [a, b) to s by one thread: 16-byte loads of
-// (x, y, z, index), eight in flight.  Returns the (distance bits, index) key;
-// ~0 for an empty run.
+// (x, y, z, index), eight in flight, then four, then the last three at once
+// with the index held at the run's last point (a point examined twice changes
+// no minimum), so that a short run is one round of loads and not one round
+// trip a point.  Returns the smaller of `best` and the run's (distance bits,
+// index) key; ~0 when both are empty.
 __device__ __forceinline__ unsigned long long segment_min(const float4 *__restrict__ csr, unsigned a, unsigned b,
-                                                          float3 s)
+                                                          float3 s, unsigned long long best = ~0ull)
 {
-    unsigned long long best = ~0ull;
     unsigned k = a;
     for (; k + 8 <= b; k += 8) {
         float4 q[8];
@@ -31,9 +33,310 @@ __device__ __forceinline__ unsigned long long segment_min(const float4 *__restri
         for (int u = 0; u < 8; ++u)
             best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
     }
-    for (; k < b; ++k) {
-        const float4 q = __ldg(csr + k);
-        best = umin64(best, nn_key(dist2(s, q), __float_as_int(q.w)));
+    if (k + 4 <= b) {
+        float4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            q[u] = __ldg(csr + k + u);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
+        k += 4;
+    }
+    if (k < b) {
+        float4 q[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            q[u] = __ldg(csr + min(k + u, b - 1u));
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+            best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
+    }
+    return best;
+}
+
+// ---------------------------------------------------------------------------
+// Near global queries.  Most points that take the global search lie just
+// outside the grid (the grid is the target's bounding box, so a flat side of
+// the target lies on its face and noise alone puts half of the matching
+// points outside): on the scenes and objects measured, 60-99% of them, half
+// of those within three voxels of their nearest point.  For them the grid
+// itself bounds the answer: the voxel nearest to the point has a root label,
+// and any point of that root's segment is at a distance D the nearest point
+// cannot exceed.  The localised search reads that segment anyway (the same
+// loads as for a point inside), so it leaves the seed (D, index) in the
+// query's own nn / d2 entries, and where the voxels that can hold a point
+// within D are few rows, the query is listed as near.  A group of 1 to 32
+// lanes then takes those rows (all voxels of one y and z, at most 32 along
+// x), a row a lane, the rows nearest to the query first: one window of
+// occupancy bits, and the occupied voxels of the window are one run of the
+// CSR store.  There is no chain from box to box as in the brick search
+// below, and many queries share a warp.  (Where a voxel holds many points
+// the rows would hold hundreds, and the brick search, which narrows D brick
+// by brick, is the better one.  On 256 pairs of objects, 14.7% of whose
+// queries are global, a batch of 40 iterations went from 47.5 to 25.2 ms;
+// NEAR_WORK 96: 27.7, 512: 24.5, but the 226k scene's registration 2% longer.)
+//
+// Exactness.  A point p with computed squared distance <= D2 is, in exact
+// arithmetic, within sqrt(D2) (1 + 2^-22) of s (rounding is monotone; below
+// 1e-18 a difference's square underflows, hence the floor at 1e-36).  Rows
+// and window ends are those of the ball of that radius in voxel units,
+// widened by a margin that covers the rounding of scaled coordinates (three
+// operations, 2^-24 of their size each, where the margin takes 1e-6 of it).
+// Every candidate's distance is computed as everywhere else, so the
+// (distance, index) minimum is that of a scan of all target points.
+// ---------------------------------------------------------------------------
+constexpr int NEAR_SHIFT_MIN = 0;     // a near query gets one lane at least
+constexpr int HEAVY_SHIFT_MIN = 2;    // a dense segment four
+constexpr float NEAR_R2 = 15.9f;      // squared distance of the seed in voxels, at most: beyond it the brick search
+constexpr int NEAR_WORK = 256;        // ... which also takes what has more rows times points a voxel than this
+constexpr int NEAR_SEED = 16;         // points of a root segment examined for the seed
+constexpr int NEAR_OUTSIDE_MAX = 64;  // with more target points outside the grid: the brick search
+
+// Whether a query s with a seed at squared distance d2, from a root segment
+// of `dense` points, is near: at most 3 voxels, so at most 8 voxels along
+// every axis, and few points expected ((2r + 1)^2 <= 8 r^2 + 2 rows of
+// `dense`).  A coordinate of 2^20 voxels and more has too few bits for that
+// count of voxels.
+__device__ __forceinline__ bool near_seed(float3 s, float d2, float inv_h, unsigned dense)
+{
+    const float r2 = d2 * (inv_h * inv_h);   // (not a number, or infinite: far)
+    return r2 <= NEAR_R2 && (8.0f * r2 + 2.0f) * (float)dense <= (float)NEAR_WORK &&
+           fmaxf(fmaxf(fabsf(s.x), fabsf(s.y)), fabsf(s.z)) * inv_h <= 1048576.0f;
+}
+
+// Square root to 2^-22 (what it is used for has a margin of 1e-3 voxels).
+__device__ __forceinline__ float near_sqrt(float x)
+{
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+struct NearBox {
+    int x0, x1, y0, y1, z0, z1;   // voxels, inclusive
+};
+
+__device__ __forceinline__ int near_voxel(float c, float o, float inv_h, int n)
+{
+    const float f = __fmul_rn(__fsub_rn(c, o), inv_h);
+    return min((int)fminf(fmaxf(f, 0.0f), 2147483520.0f), n - 1);
+}
+
+// The grid voxel nearest to s (its own voxel when s lies inside); `inside`
+// as voxel_coords.  -1 for a point with a non-finite coordinate.
+__device__ __forceinline__ int nearest_voxel(const GridGeom &g, float3 s, bool &inside)
+{
+    int ix, iy, iz;
+    inside = voxel_coords(g, s.x, s.y, s.z, ix, iy, iz);
+    if (!inside) {
+        if (!(isfinite(s.x) && isfinite(s.y) && isfinite(s.z)))
+            return -1;
+        ix = near_voxel(s.x, g.ox, g.inv_h, g.nx);
+        iy = near_voxel(s.y, g.oy, g.inv_h, g.ny);
+        iz = near_voxel(s.z, g.oz, g.inv_h, g.nz);
+    }
+    return ix + g.nx * (iy + g.ny * iz);
+}
+
+// Lanes each of n near queries or dense segments gets, as a power of two: as
+// many as `lanes` resident lanes allow, 2^least to 32 (few queries: one short
+// round trip each; many: several to a warp, whose chains of loads overlap).
+__device__ __forceinline__ int group_shift(int n, int lanes, int least)
+{
+    if (n <= 0 || n <= lanes >> 5)
+        return 5;
+    return max(least, 31 - __clz(max(lanes / n, 1)));
+}
+
+// Warp minimum of (distance bits, index) keys: the smallest distance, then
+// the smallest index at it -- two single-instruction warp reductions.
+__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v)
+{
+    const unsigned d = __reduce_min_sync(FULL_MASK, (unsigned)(v >> 32));
+    const unsigned i = __reduce_min_sync(FULL_MASK, (unsigned)(v >> 32) == d ? (unsigned)v : 0xffffffffu);
+    return ((unsigned long long)d << 32) | i;
+}
+
+// Minimum key over each aligned group of G lanes (the whole warp calls it).
+__device__ __forceinline__ unsigned long long group_min(unsigned long long v, int G)
+{
+    if (G == 32)
+        return warp_min_key(v);
+    for (int o = G / 2; o > 0; o >>= 1)
+        v = umin64(v, __shfl_xor_sync(FULL_MASK, v, o));
+    return v;
+}
+
+// The points of occupied voxels (bits, at `key` on) of a row as runs of the
+// store: next() takes some of the bits and gives their run.  In the CSR store
+// a row is one run, from the first occupied voxel's offset to the one past
+// the last's (both of which the build writes).
+struct CsrRows {
+    const unsigned *occ, *off;
+    unsigned cap;
+    const float4 *csr;
+    __device__ __forceinline__ void next(int key, unsigned &bits, unsigned &a, unsigned &e) const
+    {
+        a = __ldg(off + key + (__ffs(bits) - 1));
+        e = min(__ldg(off + key + (32 - __clz(bits))), cap);
+        bits = 0u;
+    }
+};
+
+// On the sparse grid, whose segments lie in slot order: a lookup and a run
+// an occupied voxel.
+struct HashedRows {
+    const unsigned *occ, *off;
+    unsigned cap;
+    const float4 *csr;
+    const unsigned *okeys;
+    unsigned omask;
+    int oshift;
+    __device__ __forceinline__ void next(int key, unsigned &bits, unsigned &a, unsigned &e) const
+    {
+        const int slot = hash_find(okeys, omask, oshift, (unsigned)(key + __ffs(bits) - 1));
+        bits &= bits - 1u;
+        a = e = 0u;
+        if (slot >= 0) {
+            a = __ldg(off + slot);
+            e = min(__ldg(off + slot + 1), cap);
+        }
+    }
+};
+
+// The runs [a, a + c) of the lanes of each aligned group of G lanes, scanned
+// by the group.  Runs of at most RUN_OWN points are scanned by their own
+// lanes; where a run of the warp is longer (a dense voxel holds hundreds of
+// points, and one lane would keep the others waiting) the groups deal all
+// points of their runs out over their lanes: point t of the concatenated
+// runs belongs to the first lane whose inclusive count exceeds t, found by
+// bisection over the lanes.
+constexpr unsigned RUN_OWN = 8;
+
+__device__ __forceinline__ unsigned long long scan_runs(const float4 *__restrict__ csr, unsigned a, unsigned c,
+                                                        float3 s, unsigned long long best, int sub, int G)
+{
+    if (G == 1 || !__any_sync(FULL_MASK, c > RUN_OWN))
+        return c ? segment_min(csr, a, a + c, s, best) : best;
+    unsigned incl = c;
+    for (int d = 1; d < G; d <<= 1) {
+        const unsigned y = __shfl_up_sync(FULL_MASK, incl, d, G);
+        if (sub >= d)
+            incl += y;
+    }
+    const unsigned total = __shfl_sync(FULL_MASK, incl, G - 1, G);
+    const unsigned base = a + c - incl;   // point t of the group is point base + t of the store
+    const unsigned most = __reduce_max_sync(FULL_MASK, total);
+    for (unsigned t0 = 0u; t0 < most; t0 += 4u * G) {
+        float4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const unsigned t = t0 + (unsigned)(u * G + sub);
+            int own = 0;
+            for (int step = G >> 1; step > 0; step >>= 1)
+                if (__shfl_sync(FULL_MASK, incl, own + step - 1, G) <= t)
+                    own += step;
+            const unsigned p = __shfl_sync(FULL_MASK, base, own, G) + t;
+            q[u].w = 0.0f;
+            if (t < total)
+                q[u] = __ldg(csr + p);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (t0 + (unsigned)(u * G + sub) < total)
+                best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
+    }
+    return best;
+}
+
+// The k-th index of [a, b] in the order of distance from c (a <= c <= b).
+__device__ __forceinline__ int outward(int k, int a, int b, int c)
+{
+    const int t = min(c - a, b - c);
+    if (k <= 2 * t)
+        return c + ((k & 1) ? (k + 1) / 2 : -(k / 2));
+    return c - a > b - c ? c - (k - t) : c + (k - t);
+}
+
+// One near query by an aligned group of G lanes (lane `sub` of them), from
+// the seed `best` on; on = false: a group without a query.  The whole warp
+// calls it.  Returns the group's minimum on each of its lanes.  The next
+// row's occupancy words are loaded while a row is scanned, and the best
+// distance is shared after every round of G rows.
+template <class Rows>
+__device__ __forceinline__ unsigned long long near_search(const GridGeom &g, const Rows &rows, float3 s,
+                                                          unsigned long long best, bool on, int sub, int G,
+                                                          unsigned &examined)
+{
+    const float sx = __fmul_rn(__fsub_rn(s.x, g.ox), g.inv_h), sy = __fmul_rn(__fsub_rn(s.y, g.oy), g.inv_h),
+                sz = __fmul_rn(__fsub_rn(s.z, g.oz), g.inv_h);
+    const float m = 1e-3f + 1e-6f * (fmaxf(fmaxf(fabsf(sx), fabsf(sy)), fabsf(sz)) +
+                                     (float)max(max(g.nx, g.ny), g.nz));
+    const float scale = 1.0002f * g.inv_h * g.inv_h;
+    const float r2s = fmaxf(__uint_as_float((unsigned)(best >> 32)), 1e-36f) * scale;
+    NearBox b{0, 0, 0, 0, 0, 0};
+    int ny = 1, n = 0;
+    if (on && r2s <= 1.001f * NEAR_R2) {   // (any other seed would be a stale entry)
+        const float r = near_sqrt(r2s) + m;
+        b.x0 = max((int)floorf(sx - r), 0);
+        b.x1 = min((int)floorf(sx + r), g.nx - 1);
+        b.y0 = max((int)floorf(sy - r), 0);
+        b.y1 = min((int)floorf(sy + r), g.ny - 1);
+        b.z0 = max((int)floorf(sz - r), 0);
+        b.z1 = min((int)floorf(sz + r), g.nz - 1);
+        ny = b.y1 - b.y0 + 1;
+        n = b.x0 <= b.x1 && ny > 0 && b.z0 <= b.z1 ? ny * (b.z1 - b.z0 + 1) : 0;
+    }
+    const int yc = min(max((int)floorf(sy), b.y0), b.y1), zc = min(max((int)floorf(sz), b.z0), b.z1);
+    const float inv_ny = __fdividef(1.0f, (float)ny);   // (rows of at most 10 x 10: (row + 1/2) / ny is never near an integer)
+    auto locate = [&](int row, int &iy, int &iz) {
+        const int kz = (int)(((float)row + 0.5f) * inv_ny);
+        iy = outward(row - kz * ny, b.y0, b.y1, yc);
+        iz = outward(kz, b.z0, b.z1, zc);
+        return b.x0 + g.nx * (iy + g.ny * iz);
+    };
+    int row = sub, iy = 0, iz = 0, key = 0;
+    unsigned lo = 0u, hi = 0u;
+    if (row < n) {
+        key = locate(row, iy, iz);
+        lo = __ldg(rows.occ + (key >> 5));
+        hi = __ldg(rows.occ + (key >> 5) + 1);   // (the bits have two words past the last voxel's)
+    }
+    const int rounds = __reduce_max_sync(FULL_MASK, (n + G - 1) / G);
+    for (int r = 0; r < rounds; ++r, row += G) {
+        const int jy = iy, jz = iz, jkey = key;
+        const unsigned window = __funnelshift_r(lo, hi, jkey & 31);
+        if (row + G < n) {
+            key = locate(row + G, iy, iz);
+            lo = __ldg(rows.occ + (key >> 5));
+            hi = __ldg(rows.occ + (key >> 5) + 1);
+        }
+        unsigned bits = 0u;
+        if (row < n && window) {
+            const float fy = (float)jy, fz = (float)jz;
+            const float gy = fmaxf(fmaxf(fy - sy, sy - (fy + 1.0f)) - m, 0.0f);
+            const float gz = fmaxf(fmaxf(fz - sz, sz - (fz + 1.0f)) - m, 0.0f);
+            const float r2 = fmaxf(__uint_as_float((unsigned)(best >> 32)), 1e-36f) * scale;
+            const float t = r2 - gy * gy - gz * gz;
+            if (t >= 0.0f) {
+                const float w = near_sqrt(t) + m;
+                const int xa = max(b.x0, (int)floorf(sx - w)) - b.x0, xb = min(b.x1, (int)floorf(sx + w)) - b.x0;
+                if (xa <= xb)
+                    bits = window & (0xffffffffu << xa) & (0xffffffffu >> (31 - xb));
+            }
+        }
+        if (!__any_sync(FULL_MASK, bits != 0u))
+            continue;
+        do {
+            unsigned a = 0u, e = 0u;
+            if (bits)
+                rows.next(jkey, bits, a, e);
+            const unsigned c = e > a ? e - a : 0u;
+            examined += c;
+            best = scan_runs(rows.csr, a, c, s, best, sub, G);
+        } while (__any_sync(FULL_MASK, bits != 0u));
+        best = group_min(best, G);
     }
     return best;
 }
@@ -77,15 +380,6 @@ __device__ __forceinline__ int warp_argmin(unsigned lb, int k)
 {
     const unsigned mn = __reduce_min_sync(FULL_MASK, lb);
     return __shfl_sync(FULL_MASK, k, __ffs(__ballot_sync(FULL_MASK, lb == mn)) - 1);
-}
-
-// Warp minimum of (distance bits, index) keys: the smallest distance, then
-// the smallest index at it -- two single-instruction warp reductions.
-__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long v)
-{
-    const unsigned d = __reduce_min_sync(FULL_MASK, (unsigned)(v >> 32));
-    const unsigned i = __reduce_min_sync(FULL_MASK, (unsigned)(v >> 32) == d ? (unsigned)v : 0xffffffffu);
-    return ((unsigned long long)d << 32) | i;
 }
 
 // Bound of box record k (as order-preserving bits), and its index range
@@ -152,6 +446,24 @@ __device__ __forceinline__ unsigned long long scan_chunk(const float4 *__restric
     return best;
 }
 
+// Lane `sub` of a group of G lanes: its part of the run [a, b) (four loads in
+// flight); the group's minimum is the run's.
+__device__ __forceinline__ unsigned long long group_scan(const float4 *__restrict__ pts, unsigned a, unsigned b,
+                                                         float3 s, int sub, int G)
+{
+    unsigned long long best = ~0ull;
+    for (unsigned i = a + (unsigned)sub; i < b; i += 4u * G) {
+        float4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)   // (past the end: the run's last point again)
+            q[u] = __ldg(pts + min(i + (unsigned)(u * G), b - 1u));
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
+    }
+    return best;
+}
+
 constexpr int SB_CACHED = 4;   // super-brick records kept in registers: 32 per chunk
 
 // The global search of one query s by the whole warp (every lane calls it
@@ -160,14 +472,15 @@ constexpr int SB_CACHED = 4;   // super-brick records kept in registers: 32 per 
 // super-brick records sb_box (w fields: brick-record ranges), and the `no`
 // target points outside the grid (indices into tgt); tgt holds all n_tgt
 // target points.  `examined` counts the candidates (the same on every lane).
+// `best` (the same on every lane): a known point's key, or ~0.
 __device__ __forceinline__ unsigned long long global_search(float3 s, const float4 *__restrict__ bpts,
                                                             const float4 *__restrict__ bbox,
                                                             const float4 *__restrict__ sb_box, int ns,
                                                             const float4 *__restrict__ tgt, int n_tgt,
                                                             const int *__restrict__ outside, int no, int lane,
-                                                            unsigned long long &examined)
+                                                            unsigned long long &examined,
+                                                            unsigned long long best = ~0ull)
 {
-    unsigned long long best = ~0ull;
     if (!(isfinite(s.x) && isfinite(s.y) && isfinite(s.z))) {
         for (int j = lane; j < n_tgt; j += 32)
             best = umin64(best, nn_key(dist2(s, __ldg(tgt + j)), j));
@@ -218,7 +531,8 @@ __device__ __forceinline__ unsigned long long global_search(float3 s, const floa
         int k0 = min(warp_argmin(bmin, bk), (int)(r0.y - r0.x) - 1);
         {
             const uint2 pr = box_range(bbox, (int)r0.x + k0);
-            best = scan_run(bpts, pr.x, pr.y, s, lane, best, examined);
+            if (box_bound(bbox, (int)r0.x + k0, s) <= (unsigned)(best >> 32))   // (a seed may rule it out)
+                best = scan_run(bpts, pr.x, pr.y, s, lane, best, examined);
         }
         // (2) best first: the unvisited super-brick of smallest bound
         //     while that bound is <= D, and in it the unvisited brick
