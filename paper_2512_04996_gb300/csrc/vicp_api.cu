@@ -67,7 +67,7 @@ struct vicp_ctx {
     bool off_dense = false;   // the build writes sparse offsets; vicp_get_grid completes them
     long long cap_V = -1;
     // brick level (V / 512)
-    Buf bcounts, boff, brick_list, brick_range, brick_box, bslot, sb_box, sb_left;
+    Buf bcounts, bsums, boff, brick_list, brick_range, brick_box, bslot, sb_box, sb_left;
     Buf boxk[2];      // brick bounds by key: the current build's, and the next build's (kept all ones)
     long long cap_bricks = -1;
     // N-sized
@@ -323,6 +323,7 @@ vicp_status ensure_voxel_buffers(vicp_ctx *c, long long V, long long n_bricks)
     if (n_bricks > c->cap_bricks) {
         TRY(buf_alloc(c, c->bcounts, (size_t)n_bricks * 4, "brick counts"));
         TRY(buf_zero(c, c->bcounts, "zero brick counts"));   // kept at zero between builds
+        TRY(buf_alloc(c, c->bsums, (size_t)brick_tiles(n_bricks) * 8, "brick tile sums"));
         TRY(buf_alloc(c, c->boff, (size_t)(n_bricks + 1) * 4, "brick offsets"));
         TRY(buf_alloc(c, c->brick_list, (size_t)n_bricks * 4, "brick list"));
         TRY(buf_alloc(c, c->brick_range, (size_t)n_bricks * 8, "brick ranges"));
@@ -658,8 +659,10 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
     c->off_dense = false;
     TRY(launch(c, K_BRICK_SCAN, [&] {
         return launch_brick_scan((const unsigned *)c->bcounts.p, g, (unsigned *)c->boff.p, (int *)c->brick_list.p,
-                                 (uint2 *)c->brick_range.p, (int *)c->bslot.p, d, c->stream);
+                                 (uint2 *)c->brick_range.p, (int *)c->bslot.p, (unsigned long long *)c->bsums.p, d,
+                                 c->stream);
     }));
+    c->launches += brick_slots(g) > BM_MAX_BRICKS ? 1 : 0;
     TRY(launch(c, K_SCATTER, [&] {
         const int *idx = (const int *)(sparse ? c->pslot.p : c->keys.p);   // what indexes the counts
         return launch_scatter(tgt, idx, n, g, off, counts, (const unsigned *)c->boff.p, (unsigned *)c->bcounts.p,
@@ -1253,7 +1256,7 @@ void vicp_destroy(vicp_ctx *c)
         cudaStreamSynchronize(c->side);
     Buf *all[] = {&c->counts,  &c->off,      &c->root,       &c->ring,       &c->occ[0],    &c->occ[1], &c->desc, &c->tile_sum,
                   &c->inter,       &c->uflag,      &c->zdirty,
-                  &c->bcounts, &c->boff,     &c->brick_list, &c->brick_range, &c->brick_box, &c->bslot,
+                  &c->bcounts, &c->bsums, &c->boff,     &c->brick_list, &c->brick_range, &c->brick_box, &c->bslot,
                   &c->boxk[0], &c->boxk[1], &c->sb_box,     &c->sb_left,    &c->keys,
                   &c->ids,     &c->csr,      &c->bpts,       &c->outside,    &c->nn,        &c->d2,
                   &c->fb_list, &c->hv_list, &c->hv_range, &c->partials, &c->rmse,       &c->ctl,       &c->bbox,

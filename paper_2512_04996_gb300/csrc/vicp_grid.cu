@@ -212,106 +212,21 @@ cudaError_t launch_histogram(const float4 *pts, int n, const GridGeom &g, int *k
 }
 
 // ---------------------------------------------------------------------------
-// Brick offsets: one CTA scans the per-brick counts (few: V / 512) into
-// brick offsets, and lists the non-empty bricks in ascending order with their
-// point ranges and slot numbers.  The
-// count and the non-empty flag are scanned together as one 64-bit value
-// (flag count in the high half).  The counts are staged in shared memory with
-// coalesced loads; each thread sums a contiguous run of bricks, one
-// block-wide scan offsets the runs, and a second pass writes them.
+// Brick offsets: the per-brick counts (few: V / 512) scanned into brick
+// offsets, and the non-empty bricks listed in ascending order with their
+// point ranges and slot numbers.  The count and the non-empty flag are
+// scanned together as one 64-bit value (flag count in the high half).
 // ---------------------------------------------------------------------------
-constexpr int BS_THREADS = 1024;
-
 __device__ __forceinline__ unsigned long long brick_pair(unsigned c)
 {
     return (unsigned long long)c | ((unsigned long long)(c != 0u) << 32);
 }
 
-constexpr int BS_CHUNK = 24576;   // bricks staged in shared memory per pass (96 KB)
-
-__global__ void __launch_bounds__(BS_THREADS) k_brick_scan(const unsigned *__restrict__ bcounts, int nbt,
-                                                           unsigned *__restrict__ boff, int *__restrict__ list,
-                                                           uint2 *__restrict__ range, int *__restrict__ bslot,
-                                                           DevCtl *__restrict__ ctl)
-{
-    pdl_begin();
-    extern __shared__ unsigned s_c[];   // [BS_CHUNK]
-    __shared__ unsigned long long s_w[BS_THREADS / 32];
-    __shared__ unsigned long long s_carry;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (tid == 0)
-        s_carry = 0ull;
-    for (int c0 = 0; c0 < nbt; c0 += BS_CHUNK) {
-        const int cn = min(BS_CHUNK, nbt - c0);
-        for (int i0 = tid; i0 < cn; i0 += 8 * BS_THREADS) {   // coalesced, eight loads in flight
-            unsigned v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                v[k] = (i0 + k * BS_THREADS < cn) ? __ldg(bcounts + c0 + i0 + k * BS_THREADS) : 0u;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (i0 + k * BS_THREADS < cn)
-                    s_c[i0 + k * BS_THREADS] = v[k];
-        }
-        __syncthreads();
-        // thread t owns the contiguous bricks [t*per, (t+1)*per) of the chunk
-        const int per = (cn + BS_THREADS - 1) / BS_THREADS;
-        const int i0 = min(tid * per, cn), i1 = min(i0 + per, cn);
-        unsigned long long sum = 0ull;
-        for (int i = i0; i < i1; ++i)
-            sum += brick_pair(s_c[i]);
-        unsigned long long incl = sum;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const unsigned long long y = __shfl_up_sync(FULL_MASK, incl, d);
-            if (lane >= d)
-                incl += y;
-        }
-        if (lane == 31)
-            s_w[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned long long w = s_w[lane];
-            unsigned long long wi = w;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned long long y = __shfl_up_sync(FULL_MASK, wi, d);
-                if (lane >= d)
-                    wi += y;
-            }
-            s_w[lane] = wi - w;
-        }
-        __syncthreads();
-        unsigned long long run = s_carry + s_w[warp] + (incl - sum);
-        for (int i = i0; i < i1; ++i) {
-            const unsigned c = s_c[i];
-            const int bi = c0 + i;
-            const unsigned start = (unsigned)run;
-            boff[bi] = start;
-            if (c) {
-                const int slot = (int)(run >> 32);
-                list[slot] = bi;
-                range[slot] = make_uint2(start, start + c);
-                bslot[bi] = slot;
-            }
-            run += brick_pair(c);
-        }
-        __syncthreads();
-        if (tid == BS_THREADS - 1)
-            s_carry = run;
-        __syncthreads();
-    }
-    if (tid == 0) {
-        boff[nbt] = (unsigned)s_carry;
-        ctl->n_bricks = (int)(s_carry >> 32);
-    }
-}
-
-// Many bricks per CTA in parallel: CTA b owns bricks [1024 b, 1024 b + 1024)
-// and finds its starting offset and slot by summing the counts of all
-// earlier bricks itself (cheap while bricks are few: at most 64 CTAs).
+// Up to BM_MAX_BRICKS: CTA b owns bricks [1024 b, 1024 b + 1024) and finds
+// its starting offset and slot by summing the counts of all earlier bricks
+// itself (cheap while bricks are few: at most 64 CTAs).
 constexpr int BM_THREADS = 1024;
-constexpr int BM_MAX_BRICKS = 64 * BM_THREADS;
+static_assert(BM_MAX_BRICKS == 64 * BM_THREADS, "CTAs of the one-launch brick scan");
 
 __device__ __forceinline__ unsigned long long block_sum_u64(unsigned long long v, unsigned long long *s_w)
 {
@@ -394,20 +309,114 @@ __global__ void __launch_bounds__(BM_THREADS) k_brick_scan_multi(const unsigned 
     }
 }
 
+// More bricks than that (grids past about 30 million voxels): tiles of 4096
+// bricks, a CTA each, in two launches.  The first adds up every tile, the
+// second's CTAs add the earlier tiles' sums (a few loads a thread) and scan
+// their own tile.  Bound by latency, as the form above; a single CTA passing
+// over all bricks took 195 us of the 715 us that a frame of 1.5 million
+// points on 111 million voxels (233k bricks) takes to build and match, the
+// two launches 9 us.
+constexpr int BT_PER = 4;
+constexpr int BT_TILE = BM_THREADS * BT_PER;
+static_assert(BT_TILE == BRICK_TILE, "tile sums buffer");
+
+__device__ __forceinline__ void brick_tile_counts(const unsigned *__restrict__ bcounts, int nbt, unsigned (&c)[BT_PER])
+{
+    const long long i = (long long)blockIdx.x * BT_TILE + BT_PER * threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < BT_PER; ++k)
+        c[k] = 0u;
+    if (i + BT_PER <= nbt) {   // (nbt and i are multiples of 4, the buffer is 256-byte aligned)
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(bcounts + i));
+        c[0] = v.x;
+        c[1] = v.y;
+        c[2] = v.z;
+        c[3] = v.w;
+    }
+}
+
+__global__ void __launch_bounds__(BM_THREADS) k_brick_tile_sums(const unsigned *__restrict__ bcounts, int nbt,
+                                                                unsigned long long *__restrict__ sums)
+{
+    pdl_begin();
+    __shared__ unsigned long long s_w[BM_THREADS / 32];
+    unsigned c[BT_PER];
+    brick_tile_counts(bcounts, nbt, c);
+    unsigned long long v = 0ull;
+#pragma unroll
+    for (int k = 0; k < BT_PER; ++k)
+        v += brick_pair(c[k]);
+    v = block_sum_u64(v, s_w);
+    if (threadIdx.x == 0)
+        sums[blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(BM_THREADS) k_brick_scan_tiles(const unsigned *__restrict__ bcounts, int nbt,
+                                                                 const unsigned long long *__restrict__ sums,
+                                                                 unsigned *__restrict__ boff, int *__restrict__ list,
+                                                                 uint2 *__restrict__ range, int *__restrict__ bslot,
+                                                                 DevCtl *__restrict__ ctl)
+{
+    pdl_begin();
+    __shared__ unsigned long long s_w[BM_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned c[BT_PER];
+    brick_tile_counts(bcounts, nbt, c);
+    unsigned long long before = 0ull;
+    for (int t = tid; t < (int)blockIdx.x; t += BM_THREADS)
+        before += __ldg(sums + t);
+    before = block_sum_u64(before, s_w);
+    unsigned long long own = 0ull;
+#pragma unroll
+    for (int k = 0; k < BT_PER; ++k)
+        own += brick_pair(c[k]);
+    unsigned long long incl = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long y = __shfl_up_sync(FULL_MASK, incl, d);
+        if (lane >= d)
+            incl += y;
+    }
+    if (lane == 31)
+        s_w[warp] = incl;
+    __syncthreads();
+    unsigned long long run = before + (incl - own);
+    for (int w = 0; w < warp; ++w)
+        run += s_w[w];
+    const long long i = (long long)blockIdx.x * BT_TILE + BT_PER * tid;
+    if (i >= nbt)
+        return;
+#pragma unroll
+    for (int k = 0; k < BT_PER; ++k) {
+        boff[i + k] = (unsigned)run;
+        if (c[k]) {
+            const int slot = (int)(run >> 32);
+            list[slot] = (int)(i + k);
+            range[slot] = make_uint2((unsigned)run, (unsigned)run + c[k]);
+            bslot[i + k] = slot;
+        }
+        run += brick_pair(c[k]);
+    }
+    if (i + BT_PER == nbt) {
+        boff[nbt] = (unsigned)run;
+        ctl->n_bricks = (int)(run >> 32);
+    }
+}
+
 cudaError_t launch_brick_scan(const unsigned *bcounts, const GridGeom &g, unsigned *boff, int *list, uint2 *range,
-                              int *bslot, DevCtl *ctl, cudaStream_t st)
+                              int *bslot, unsigned long long *sums, DevCtl *ctl, cudaStream_t st)
 {
     const int nbt = brick_slots(g);
     if (nbt <= BM_MAX_BRICKS) {
         return launch_kernel(k_brick_scan_multi, dim3((nbt + BM_THREADS - 1) / BM_THREADS), dim3(BM_THREADS), 0, st,
                              bcounts, nbt, boff, list, range, bslot, ctl);
     }
-    const size_t smem = BS_CHUNK * sizeof(unsigned);
-    cudaError_t e = cudaFuncSetAttribute(k_brick_scan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const dim3 tiles((nbt + BT_TILE - 1) / BT_TILE);
+    const cudaError_t e = launch_kernel(k_brick_tile_sums, tiles, dim3(BM_THREADS), 0, st, bcounts, nbt, sums);
     if (e != cudaSuccess)
         return e;
-    return launch_kernel(k_brick_scan, dim3(1), dim3(BS_THREADS), smem, st, bcounts, nbt, boff, list, range, bslot,
-                         ctl);
+    return launch_kernel(k_brick_scan_tiles, tiles, dim3(BM_THREADS), 0, st, bcounts, nbt,
+                         (const unsigned long long *)sums, boff, list, range, bslot, ctl);
 }
 
 // ---------------------------------------------------------------------------

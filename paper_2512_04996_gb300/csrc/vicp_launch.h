@@ -90,8 +90,12 @@ cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off
                         const unsigned *tile_sum, unsigned long long *desc, const DevCtl *ctl, cudaStream_t st,
                         bool dense);
 cudaError_t launch_offsets_fill(unsigned *off, const unsigned *occ, long long V, cudaStream_t st);
+// sums: brick_tiles(slots) words of scratch (used by large grids).
+constexpr int BM_MAX_BRICKS = 65536;   // up to this many slots one launch, past it two
+constexpr int BRICK_TILE = 4096;
+inline long long brick_tiles(long long slots) { return (slots + BRICK_TILE - 1) / BRICK_TILE; }
 cudaError_t launch_brick_scan(const unsigned *bcounts, const GridGeom &g, unsigned *boff, int *list, uint2 *range,
-                              int *bslot, DevCtl *ctl, cudaStream_t st);
+                              int *bslot, unsigned long long *sums, DevCtl *ctl, cudaStream_t st);
 // The scatter also zeroes the tile totals and the occupancy buffer of the
 // next build (occ_next, occ_next_words words), writes the brick and
 // super-brick float boxes from the histogram's bounds (boxk) and sets the
