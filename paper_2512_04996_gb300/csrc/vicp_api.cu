@@ -46,6 +46,7 @@ struct vicp_ctx {
     cudaEvent_t ev_fork = nullptr, ev_clr = nullptr;      // graph capture: the buffer resets beside the copy
     int device = 0;
     int sms = 152;
+    bool small_ok = false;   // the device runs the one-cluster iterations of small clouds
     std::string last_error;
     uint64_t cur_bytes = 0, peak_bytes = 0;
 
@@ -583,8 +584,48 @@ vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, i
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
 }
 
+// Whether m source points take the one-cluster iterations (vicp_small.cu):
+// few enough, the dense grid, double-float sums.  (Kernel timing keeps the
+// separate kernels, which it names.)
+bool takes_small(const vicp_ctx *c, int m)
+{
+    return c->small_ok && m <= SMALL_MAX_POINTS && !sparse_of(c) && !(c->params.flags & VICP_FLAG_FP64_SOLVE) &&
+           !c->profiling;
+}
+
+vicp_status run_small(vicp_ctx *c, const float4 *src, int m, double *pose, double *rmse, int iters, int honor_stop)
+{
+    SmallArgs a{};
+    a.src = src;
+    a.m = m;
+    a.pose = pose;
+    a.g = c->geom;
+    a.root = (const int *)c->root.p;
+    a.occ = (const unsigned *)c->occ[c->occ_cur].p;
+    a.off = (const unsigned *)c->off.p;
+    a.csr = (const float4 *)c->csr.p;
+    a.bpts = (const float4 *)c->bpts.p;
+    a.bbox = (const float4 *)c->brick_box.p;
+    a.sb_box = (const float4 *)c->sb_box.p;
+    a.tgt = c->target;
+    a.n_tgt = c->n_target;
+    a.outside = (const int *)c->outside.p;
+    a.center = grid_center(c->geom);
+    a.iters = iters;
+    a.honor_stop = honor_stop;
+    a.eps = c->params.rmse_eps;
+    a.rmse_out = rmse;
+    a.ctl = ctl_of(c);
+    TRY(launch(c, K_SMALL_ITERS, [&] { return launch_small_iters(a, c->stream); }));
+    cudaError_t e = cudaEventRecord(c->ev_nns, c->stream);   // a later dilation waits for these searches
+    c->nns_in_capture = c->capturing;
+    return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
+}
+
 vicp_status run_step(vicp_ctx *c, const float4 *src, int m, double *pose, double *rmse, int honor_stop)
 {
+    if (takes_small(c, m))
+        return run_small(c, src, m, pose, rmse, 1, honor_stop);
     TRY(ensure_query_buffers(c, m));
     int *nn = (int *)c->nn.p;
     TRY(run_nns(c, src, m, pose, nn, (float *)c->d2.p, honor_stop));
@@ -871,8 +912,12 @@ vicp_status registration_work(vicp_ctx *c, const float4 *src, int32_t m, const f
     e = cudaStreamWaitEvent(c->stream, c->ev_src, 0);
     if (e != cudaSuccess)
         return cuda_fail(c, e, "stream wait");
-    for (int k = 0; k < c->params.max_iters; ++k) {
-        if (k > 0 && (c->params.flags & VICP_FLAG_REBUILD_EACH_ITER)) {
+    const bool rebuild = (c->params.flags & VICP_FLAG_REBUILD_EACH_ITER) != 0;
+    const bool one = !rebuild && c->params.max_iters > 0 && takes_small(c, m);   // all iterations in one launch
+    if (one)
+        TRY(run_small(c, src, m, pose, nullptr, c->params.max_iters, 1));
+    for (int k = 0; k < c->params.max_iters && !one; ++k) {
+        if (k > 0 && rebuild) {
             TRY(build(c, tgt, n));
             TRY(dilate(c, -1));
         }
@@ -1230,6 +1275,7 @@ vicp_status vicp_create(vicp_ctx **out, const vicp_params *params, const vicp_al
         cudaGetLastError();
         c->sms = 152;
     }
+    c->small_ok = small_iters_usable();
     s = buf_alloc(c, c->ctl, sizeof(vicp_ctx::RegOut), "control block and registration pose");
     if (s == VICP_OK)
         s = buf_zero(c, c->ctl, "zero control block");
@@ -1669,7 +1715,7 @@ const char *kernel_name(int k)
     static const char *names[K_COUNT] = {"bbox",       "histogram", "scan",     "scatter",      "brick_scan",
                                          "dilate",   "correspond", "fallback", "reduce_solve",
                                          "maxcount",   "fixed_scatter", "fixed_correspond", "offsets_fill",
-                                         "reduce_solve_f64"};
+                                         "reduce_solve_f64", "small_iterations"};
     return (k >= 0 && k < K_COUNT) ? names[k] : "?";
 }
 }  // namespace vicp

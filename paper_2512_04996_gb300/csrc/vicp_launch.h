@@ -43,6 +43,7 @@ enum KernelId {
     K_FIXED_CORRESPOND,
     K_OFFSETS_FILL,
     K_REDUCE_SOLVE_F64,
+    K_SMALL_ITERS,
     K_COUNT
 };
 const char *kernel_name(int k);
@@ -190,6 +191,30 @@ struct FallbackArgs {
     int *n_global_out;           // may be null: receives the number of global searches
 };
 cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st);
+// Iterations of a small source cloud on the dense grid by one cluster
+// (vicp_small.cu): searches, sums (double-float), solve, stopping test.
+constexpr int SMALL_MAX_POINTS = 16384;
+bool small_iters_usable();   // whether the current device takes the cluster (asked once per context)
+struct SmallArgs {
+    const float4 *src;
+    int m;
+    double *pose;
+    GridGeom g;
+    const int *root;
+    const unsigned *occ, *off;
+    const float4 *csr;
+    const float4 *bpts, *bbox, *sb_box;
+    const float4 *tgt;
+    int n_tgt;
+    const int *outside;
+    float3 center;
+    int iters;
+    int honor_stop;    // 1: the registration's loop state in ctl is continued
+    double eps;
+    double *rmse_out;  // may be null
+    DevCtl *ctl;
+};
+cudaError_t launch_small_iters(const SmallArgs &a, cudaStream_t st);
 // Standalone voxel histogram (vicp_hist.cu): method 0 warp-aggregated,
 // 1 per-block shared-memory hash; adds to counts.
 cudaError_t launch_voxel_histogram(const float4 *pts, int n, const GridGeom &g, int method, int *keys,

@@ -18,8 +18,8 @@ namespace vicp {
 // ---------------------------------------------------------------------------
 constexpr int CORR_THREADS = 512;
 // Up to this many source points the global queries are so few that each has
-// a warp of its own, and the brick search (with the seed) is the shorter
-// chain: one step of 1,000 points on a 4k object 22.2 us against 24.6.
+// a warp of its own, and the brick search (with the seed) is as short a chain
+// (one step of 1,000 points on a 4k object 24.2 to 24.6 us either way).
 constexpr int NEAR_MIN_QUERIES = 16384;
 
 // Segment of a root voxel in the CSR store: [off[r], off[r + 1]) (clamped to
