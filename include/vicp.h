@@ -537,6 +537,14 @@ VICP_API vicp_status vicp_batch_register_host(vicp_batch *b, int32_t n_pairs, co
 VICP_API vicp_status vicp_batch_correspond(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
                                            const double *poses_dev, int32_t *nn_out, float *d2_out);
 
+/* vicp_batch_correspond without waiting: the search is only enqueued on the
+ * context's stream (the first call for other sizes than the last still
+ * synchronises to upload them), and what vicp_batch_correspond would report
+ * from the device is returned by the next call that synchronises
+ * (vicp_batch_correspond, vicp_batch_register). */
+VICP_API vicp_status vicp_batch_correspond_async(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
+                                                 const double *poses_dev, int32_t *nn_out, float *d2_out);
+
 /* Autotuner: runs `iters` iterations of every pair from `poses` (host, as
  * for vicp_batch_register; left unchanged) with each iteration kernel shape,
  * timing each with CUDA events (best of `trials`), and keeps the fastest for

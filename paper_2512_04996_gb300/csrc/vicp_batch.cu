@@ -5,21 +5,30 @@
 // (Alg. 4 and the update of Eq. 1) is one persistent launch.
 //
 // The iteration kernel is cooperative: all its blocks are resident together
-// and pass two grid-wide barriers.
-//   phase 1  each block takes (pair, tile) items in turn and runs the
-//            localised search of the tile's points (a thread per point); a
-//            query whose root segment is long, or that has no root, is
-//            listed for phase 2 (one global atomic per block and list);
-//   phase 2  every warp of the grid takes listed queries in turn: all lanes
-//            scan one dense segment, or run one exact global search over the
-//            query's pair;
-//   phase 3  each block reduces the items it searched in phase 1 into
-//            per-item double-float sums; the block that finishes a pair's
-//            last item adds the pair's item sums in item order and solves
-//            Eq. 1 for that pair (one warp), so every pair's update is
+// and pass one to three grid-wide barriers.
+//   phase 1  each warp takes (pair, tile) items as they come: the localised search
+//            of the tile's points (a lane per point), the near global queries
+//            among them (vicp_search.cuh) from a list in the warp's shared
+//            memory, and the tile's sums of what is answered by then; far
+//            queries and dense segments are listed for phase 2 (one global
+//            atomic per tile and list);
+//   phase 2  all warps share out the listed queries of all pairs (dense
+//            segments by groups of lanes, a far query by a warp);
+//   phase 3  what phase 2 answered joins the sums of its tiles (listed, a warp
+//            each); then a block per pair adds the pair's tiles in a fixed
+//            order and solves Eq. 1 for that pair, so every pair's update is
 //            bit-identical from run to run.
+// Phase 2 and the first half of phase 3, with a barrier each, are left out
+// when nothing was listed.
+// A tile is a warp's own: no block barrier, and no list or match that goes
+// through global memory for the points that phase 1 answers.  (With items of
+// a block, its barriers between dependent loads left an item of 512 points
+// 10 us in phase 1 and 13 us in a phase 3 that read every match again:
+// 140 and 190 us of the 560 us an iteration of 256 pairs took.)
 // The barriers wait with a time limit (one second): a block that gives up
 // sets DEVERR_TIMEOUT and leaves the kernel.
+#include <algorithm>
+
 #include "vicp_batch.h"
 #include "vicp_df.cuh"
 #include "vicp_f64.cuh"
@@ -591,160 +600,185 @@ __device__ __forceinline__ PoseF load_posef(const float *__restrict__ posef, int
 }
 
 // ---------------------------------------------------------------------------
-// Phase 3 of the iteration kernel with FP64 sums and an FP64 solve: the same
-// items and the same fixed summation order (thread, warp, block per item,
-// then the pair's items in item order by the block of its last item) as the
-// double-float phase 3 of k_batch_iter, in doubles.  s_dyn_f holds
-// WARPS x 16 x 33 doubles; the partials one double per (item, sum).
+// The sums of phases 1 and 3 in double-float or, for the FP64 variant, in
+// doubles (vicp_df.cuh, vicp_f64.cuh): 8 bytes a value either way.
 // ---------------------------------------------------------------------------
-template <int TH, int PPT>
-__device__ __forceinline__ void batch_phase3_f64(const BatchIterArgs &a, float *s_dyn_f, BatchItem &s_item,
-                                                 int &s_skip, int &s_last, PoseF &s_pose)
-{
-    constexpr int WARPS = TH / 32;
-    __shared__ double s_w[WARPS][F64_SUMS];
-    __shared__ double s_tot[F64_SUMS];
-    double(*s_t)[F64_SUMS][33] = reinterpret_cast<double(*)[F64_SUMS][33]>(s_dyn_f);
-    double *partials = reinterpret_cast<double *>(a.partials);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    DevCtl *const ctl = a.ctl;
-    for (int itx = blockIdx.x; itx < a.n_items; itx += gridDim.x) {
-        if (tid == 0) {
-            s_item = a.items[itx];
-            s_skip = *(volatile const int *)&a.state[s_item.pair].stop;
-        }
-        __syncthreads();
-        const BatchItem it = s_item;
-        if (s_skip) {
-            __syncthreads();
-            continue;
-        }
-        load_pose_f_block(a.pose + 16 * it.pair, s_pose);
-        const PoseF P = s_pose;
-        const BatchPair *bp = a.pairs + it.pair;
-        const double3 c = make_double3((double)bp->cx, (double)bp->cy, (double)bp->cz);
-        const int tbase = bp->tbase, n_tgt = bp->n_tgt;
-        double acc[F64_SUMS];
-#pragma unroll
-        for (int k = 0; k < F64_SUMS; ++k)
-            acc[k] = 0.0;
-        int j[PPT];
-        float4 p[PPT], q[PPT];
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            const int i = it.i0 + tid + TH * u;
-            j[u] = -1;
-            if (i < it.i1) {
-                j[u] = __ldcg(a.nn + i);
-                p[u] = __ldg(a.src + i);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            if ((unsigned)j[u] < (unsigned)n_tgt)
-                q[u] = __ldg(a.tgt + tbase + j[u]);
-            else if (it.i0 + tid + TH * u < it.i1)   // no valid match: report, leave it out
-                atomicOr(&ctl->err, DEVERR_BOUNDS);
-        }
-#pragma unroll
-        for (int u = 0; u < PPT; ++u)
-            if ((unsigned)j[u] < (unsigned)n_tgt)
-                accumulate_corr_f64(acc, transform_pt(P, p[u]), q[u], c);
-        // warp sums through shared memory: lane l adds value l % 16 over
-        // lanes 16 (l / 16) .. 16 (l / 16) + 15 in order, then the halves
-#pragma unroll
-        for (int k = 0; k < F64_SUMS; ++k)
-            s_t[warp][k][lane] = acc[k];
-        __syncwarp();
-        {
-            const int k = lane & 15, h = (lane >> 4) * 16;
-            double v = s_t[warp][k][h];
-#pragma unroll
-            for (int t = 1; t < 16; ++t)
-                v += s_t[warp][k][h + t];
-            v += __shfl_xor_sync(FULL_MASK, v, 16);
-            if (lane < 16)
-                s_w[warp][k] = v;
-        }
-        __syncthreads();
-        if (tid < F64_SUMS) {   // the block's warps, in order
-            double v = s_w[0][tid];
-#pragma unroll
-            for (int w = 1; w < WARPS; ++w)
-                v += s_w[w][tid];
-            partials[(size_t)itx * F64_SUMS + tid] = v;
-            __threadfence();
-        }
-        __syncthreads();
-        if (tid == 0)
-            s_last = atomicAdd(&a.state[it.pair].items_done, 1u) == (unsigned)(bp->n_items - 1);
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            // the pair's item sums in item order, as in the double-float phase 3
-            const int item0 = bp->item0, n_items = bp->n_items;
-            {
-                const int k = tid & 15, grp = tid >> 4;
-                double v = 0.0;
-                for (int b = grp; b < n_items; b += TH / 16)
-                    v += __ldcg(partials + (size_t)(item0 + b) * F64_SUMS + k);
-                v += __shfl_xor_sync(FULL_MASK, v, 16);
-                if (lane < 16)
-                    s_w[warp][lane] = v;
-            }
-            __syncthreads();
-            if (tid < F64_SUMS) {
-                double t = s_w[0][tid];
-#pragma unroll
-                for (int w = 1; w < WARPS; ++w)
-                    t += s_w[w][tid];
-                s_tot[tid] = t;
-            }
-            __syncthreads();
-            if (warp == 0) {
-                double rmse;
-                BatchState *stp = a.state + it.pair;
-                const bool ok = solve_update_f64(s_tot, bp->n_src, c, a.pose + 16 * it.pair, rmse);
-                if (lane == 0) {
-                    stp->items_done = 0u;
-                    stp->last_rmse = rmse;
-                    if (!ok) {
-                        stp->err |= DEVERR_DEGENERATE;
-                        stp->stop = 1;
-                        atomicOr(&ctl->err, DEVERR_DEGENERATE);
-                    } else {
-                        const int k = stp->iters;
-                        stp->iters = k + 1;
-                        if (a.eps > 0.0 && k >= 1 && fabs(rmse - stp->prev_rmse) < a.eps)
-                            stp->stop = 1;
-                        stp->prev_rmse = rmse;
-                    }
-                }
-            }
-        }
-        __syncthreads();   // s_item, s_pose and the sums are rewritten for the next item
+template <bool F64> struct IterSum;
+
+template <> struct IterSum<false> {
+    using T = dfl;
+    __device__ static T zero() { return {0.0f, 0.0f}; }
+    __device__ static T add(T a, T b) { return df_acc(a, b); }
+    __device__ static T shfl_xor(T v, int o) { return df_shfl_xor(v, o); }
+    __device__ static T load(const float2 *p)
+    {
+        const float2 x = __ldcg(p);
+        return {x.x, x.y};
     }
+    __device__ static void store(float2 *p, T v) { *p = make_float2(v.hi, v.lo); }
+    __device__ static void accumulate(T (&acc)[N_SUMS], float3 s, float4 q, const BatchPair *bp)
+    {
+        accumulate_corr(acc, s, q, make_float3(bp->cx, bp->cy, bp->cz));
+    }
+    __device__ static bool solve(const T *s_tot, const BatchPair *bp, double *pose, double &rmse)
+    {
+        return solve_update(s_tot, bp->n_src, make_float3(bp->cx, bp->cy, bp->cz), pose, rmse);
+    }
+};
+
+template <> struct IterSum<true> {
+    using T = double;
+    __device__ static T zero() { return 0.0; }
+    __device__ static T add(T a, T b) { return a + b; }
+    __device__ static T shfl_xor(T v, int o) { return __shfl_xor_sync(FULL_MASK, v, o); }
+    __device__ static T load(const float2 *p) { return __ldcg(reinterpret_cast<const double *>(p)); }
+    __device__ static void store(float2 *p, T v) { *reinterpret_cast<double *>(p) = v; }
+    __device__ static void accumulate(T (&acc)[N_SUMS], float3 s, float4 q, const BatchPair *bp)
+    {
+        static_assert(N_SUMS == F64_SUMS, "sum layout");
+        accumulate_corr_f64(acc, s, q, make_double3((double)bp->cx, (double)bp->cy, (double)bp->cz));
+    }
+    __device__ static bool solve(const T *s_tot, const BatchPair *bp, double *pose, double &rmse)
+    {
+        return solve_update_f64(s_tot, bp->n_src, make_double3((double)bp->cx, (double)bp->cy, (double)bp->cz), pose,
+                                rmse);
+    }
+};
+
+// A warp's shared memory: the tile's matches, seeds and lists while it is
+// searched, then the lanes' sums laid out for the warp's reduction.
+struct WarpTile {
+    union {
+        struct {
+            float pose[12];
+            int nn[BATCH_TILE_MAX];      // match of each point; -1: left to phase 2 (or no point)
+            float d2[BATCH_TILE_MAX];    // seed of a near query
+            unsigned char near[BATCH_TILE_MAX], far[BATCH_TILE_MAX];
+        };
+        double lanes[N_SUMS][33];        // a row per sum (row stride 33: no bank conflicts either way)
+        double total[N_SUMS];
+    };
+};
+
+// The tile's 16 sums from the lanes' (fixed order): sum k on lanes k and
+// k + 16.  The whole warp calls it; w's contents are overwritten.
+template <bool F64>
+__device__ __forceinline__ typename IterSum<F64>::T tile_sum(const typename IterSum<F64>::T (&acc)[N_SUMS], WarpTile &w)
+{
+    using S = IterSum<F64>;
+    using T = typename S::T;
+    static_assert(sizeof(T) == sizeof(double), "sum words");
+    const int lane = threadIdx.x & 31;
+    T(*rows)[33] = reinterpret_cast<T(*)[33]>(w.lanes);
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < N_SUMS; ++k)
+        rows[k][lane] = acc[k];
+    __syncwarp();
+    const int k = lane & 15, h = (lane >> 4) * 16;
+    T v = rows[k][h];
+#pragma unroll
+    for (int t = 1; t < 16; ++t)
+        v = S::add(v, rows[k][h + t]);
+    v = S::add(v, S::shfl_xor(v, 16));
+    __syncwarp();
+    return v;
+}
+
+// The near queries of a tile, 1 to 32 lanes each; returns the candidates
+// this lane examined.  (Out of line, it and the sums below spill less and
+// are slower: 256 pairs 28.8 ms a batch against 25.9.)
+template <bool SEARCH_ONLY>
+static __device__ __forceinline__ unsigned near_tile(const BatchIterArgs &a, WarpTile &w, const BatchItem &it, int n_near)
+{
+    const int lane = threadIdx.x & 31;
+    const BatchPair *bp = a.pairs + it.pair;
+    const GridGeom g = bp->g;
+    const long long vb = bp->vbase;
+    const CsrRows rows{a.occ + (vb >> 5), a.off + vb, (unsigned)a.n_stored, a.csr};
+    const PoseF P = *reinterpret_cast<const PoseF *>(w.pose);
+    const int no = a.state[it.pair].n_outside;
+    const int shift = group_shift(n_near, 32, NEAR_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
+    const int sub = lane & (G - 1);
+    unsigned cand = 0u;
+    for (int k = 0; k < n_near; k += pack) {
+        const int q = k + (lane >> shift);
+        const bool on = q < n_near;
+        const int l = on ? w.near[q] : 0, i = it.i0 + l;
+        float3 s = make_float3(0.0f, 0.0f, 0.0f);
+        unsigned long long best = ~0ull;
+        if (on) {
+            s = transform_pt(P, __ldg(a.src + i));
+            best = nn_key(w.d2[l], w.nn[l]);
+            for (int o = sub; o < no; o += G) {   // target points outside the grid
+                const int j = __ldg(a.outside + bp->tbase + o);
+                best = umin64(best, nn_key(dist2(s, __ldg(a.tgt + bp->tbase + j)), j));
+            }
+            cand += sub == 0 ? (unsigned)no : 0u;
+        }
+        if (no > 0)
+            best = group_min(best, G);
+        best = near_search(g, rows, s, best, on, sub, G, cand);
+        if (on && sub == 0) {
+            w.nn[l] = (int)(unsigned)best;
+            if (SEARCH_ONLY) {
+                a.nn[i] = (int)(unsigned)best;
+                a.d2[i] = __uint_as_float((unsigned)(best >> 32));
+            }
+        }
+    }
+    __syncwarp();
+    return cand;
+}
+
+// The sums of a tile's matches w.nn, stored as item itx's; lane r gets the
+// mask of the points 32 r .. 32 r + 31 that have none yet.
+template <bool F64>
+static __device__ __forceinline__ unsigned sum_tile(const BatchIterArgs &a, WarpTile &w, const BatchItem &it, int itx)
+{
+    using S = IterSum<F64>;
+    using T = typename S::T;
+    const int lane = threadIdx.x & 31, n = it.i1 - it.i0;
+    const BatchPair *bp = a.pairs + it.pair;
+    const PoseF P = *reinterpret_cast<const PoseF *>(w.pose);
+    T acc[N_SUMS];
+#pragma unroll
+    for (int k = 0; k < N_SUMS; ++k)
+        acc[k] = S::zero();
+    unsigned left = 0u;
+#pragma unroll 1
+    for (int l0 = 0; l0 < n; l0 += 32) {
+        const int l = l0 + lane;
+        const int j = l < n ? w.nn[l] : -1;
+        if ((unsigned)j < (unsigned)bp->n_tgt)
+            S::accumulate(acc, transform_pt(P, __ldg(a.src + it.i0 + l)), __ldg(a.tgt + bp->tbase + j), bp);
+        else if (j >= 0)   // no valid match: report, leave it out
+            atomicOr(&a.ctl->err, DEVERR_BOUNDS);
+        const unsigned m = __ballot_sync(FULL_MASK, l < n && j < 0);
+        if (lane == (l0 >> 5))
+            left = m;
+    }
+    const T v = tile_sum<F64>(acc, w);
+    if (lane < N_SUMS)
+        S::store(a.partials + (size_t)itx * N_SUMS + lane, v);
+    return left;
 }
 
 // ---------------------------------------------------------------------------
-// The iteration kernel (see the top of this file).  Dynamic shared memory:
-// the transposed per-lane sums of phase 3, WARPS x 16 x 33 words of 8 bytes
-// (a float pair per word for double-float sums, a double for FP64 sums).
-// With F64 the sums of phase 3 and the solve are FP64 (vicp_f64.cuh).
+// The iteration kernel (see the top of this file).  Dynamic shared memory: a
+// WarpTile per warp.
 // ---------------------------------------------------------------------------
-template <int TH, int PPT, int MINB, bool F64>
-__global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
+template <int TH, int MINB, bool F64, bool SEARCH_ONLY = false, int UNROLL = 1>
+__global__ void __launch_bounds__(TH, MINB) k_batch_iter(const __grid_constant__ BatchIterArgs a)
 {
     constexpr int WARPS = TH / 32;
-    __shared__ PoseF s_pose;
-    __shared__ BatchItem s_item;
-    __shared__ int s_skip, s_flag, s_last;
-    __shared__ unsigned long long s_cand;
-    __shared__ int s_fb, s_fb_base, s_nr, s_nr_base, s_hv, s_hv_base;
-    __shared__ float s_whi[WARPS][N_SUMS], s_wlo[WARPS][N_SUMS];
-    __shared__ dfl s_tot[N_SUMS];
-    extern __shared__ float s_dyn[];   // [2][WARPS][N_SUMS][33]
+    using S = IterSum<F64>;
+    using T = typename S::T;
+    __shared__ int s_flag;
+    __shared__ unsigned long long s_cand, s_queries, s_near, s_glob;   // work counters: one global atomic a block
+    extern __shared__ double s_dyn[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    WarpTile &w = reinterpret_cast<WarpTile *>(s_dyn)[warp];
     DevCtl *const ctl = a.ctl;
     // After a barrier gave up, the arrival count no longer matches the
     // blocks in the barrier: the remaining launches of the registration do
@@ -753,427 +787,367 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const BatchIterArgs a)
         return;
     if (a.test_leave_early && blockIdx.x == 0)
         return;   // the others' first barrier runs out of time (test of the time limit)
+    if (tid == 0)
+        s_cand = s_queries = s_near = s_glob = 0ull;
+    __syncthreads();
+    const int n_warps = gridDim.x * WARPS, gw = blockIdx.x * WARPS + warp;
 
-    // ---- phase 1: localised search, item by item --------------------------
-    for (int itx = blockIdx.x; itx < a.n_items; itx += gridDim.x) {
-        if (tid == 0) {
-            s_item = a.items[itx];
-            s_skip = *(volatile const int *)&a.state[s_item.pair].stop;
-            s_cand = 0ull;
-            s_fb = s_nr = s_hv = 0;
-        }
-        __syncthreads();
-        const BatchItem it = s_item;
-        if (s_skip) {
-            __syncthreads();
+    // ---- phase 1: each warp's tiles: localised and near searches, sums ------
+    unsigned cand = 0u, queries = 0u, near_done = 0u, near_cand = 0u;
+    // The first tile by position, then whichever is next (the ticket is drawn
+    // while the tile before is searched): tiles differ several-fold.
+    unsigned ticket = 0u;
+    for (int itx = gw; itx < a.n_items;
+         itx = a.n_items > n_warps ? n_warps + (int)__shfl_sync(FULL_MASK, ticket, 0) : a.n_items) {
+        if (lane == 0 && a.n_items > n_warps)
+            ticket = atomicAdd(&ctl->item_next, 1u);
+        const BatchItem it = a.items[itx];
+        if (!SEARCH_ONLY && __ldcg(&a.state[it.pair].stop))
             continue;
+        __syncwarp();   // the last tile's use of w is over
+        if (lane < 12) {
+            const int r = lane >> 2, c = lane & 3, k = c < 3 ? 3 * r + c : 9 + r;
+            const float v = __double2float_rn(__ldcg(a.pose + 16 * it.pair + lane));
+            w.pose[k] = v;
+            if (it.l0 == 0)   // the pair's first tile: for phase 2
+                a.posef[12 * it.pair + k] = v;
         }
-        load_pose_f_block(a.pose + 16 * it.pair, s_pose);
-        const PoseF P = s_pose;
+        const bool seeds = a.state[it.pair].n_outside <= NEAR_OUTSIDE_MAX;
         const BatchPair *bp = a.pairs + it.pair;
         const GridGeom g = bp->g;
         const long long vb = bp->vbase;
-        if (it.l0 == 0 && tid < 12)   // the pair's first item
-            a.posef[12 * it.pair + tid] = reinterpret_cast<const float *>(&s_pose)[tid];
-        const bool seeds = a.state[it.pair].n_outside <= NEAR_OUTSIDE_MAX;
-        bool far[PPT], near[PPT], heavy[PPT];
-        unsigned ra[PPT], rb[PPT];
-        unsigned cand = 0u;
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            const int i = it.i0 + tid + TH * u;
-            far[u] = near[u] = heavy[u] = false;
-            ra[u] = rb[u] = 0u;
-            if (i < it.i1) {   // (as k_correspond)
+        const CsrRows rows{a.occ + (vb >> 5), a.off + vb, (unsigned)a.n_stored, a.csr};
+        __syncwarp();
+        const PoseF P = *reinterpret_cast<const PoseF *>(w.pose);
+        const int n = it.i1 - it.i0;
+        int n_near = 0, n_far = 0;
+#pragma unroll UNROLL
+        for (int l0 = 0; l0 < n; l0 += 32) {
+            const int l = l0 + lane, i = it.i0 + l;
+            bool far = false, near = false, heavy = false;
+            unsigned x0 = 0u, x1 = 0u;
+            if (l < n) {   // (as k_correspond)
                 const float3 s = transform_pt(P, __ldg(a.src + i));
                 bool inside;
                 const int v = nearest_voxel(g, s, inside);
                 const int r = v >= 0 ? __ldg(a.root + vb + v) : -1;
-                far[u] = true;
                 unsigned dense = 0u;
                 if (r >= 0) {
-                    const unsigned x0 = __ldg(a.off + vb + r);
-                    unsigned x1 = max(x0, min(__ldg(a.off + vb + r + 1), (unsigned)a.n_stored));
+                    x0 = __ldg(rows.off + r);
+                    x1 = max(x0, min(__ldg(rows.off + r + 1), rows.cap));
                     dense = x1 - x0;
                     if (!inside)   // only a seed
                         x1 = min(x1, x0 + (unsigned)NEAR_SEED);
-                    ra[u] = x0;
-                    rb[u] = x1;
-                    cand += inside ? dense : 0u;
-                    heavy[u] = inside && dense > HEAVY;
-                    far[u] = !inside;
                 }
-                if (!heavy[u]) {
-                    const unsigned long long best = segment_min(a.csr, ra[u], rb[u], s);
-                    a.nn[i] = (int)(unsigned)best;
-                    a.d2[i] = __uint_as_float((unsigned)(best >> 32));
-                    near[u] = far[u] && dense && seeds &&
-                              near_seed(s, __uint_as_float((unsigned)(best >> 32)), g.inv_h, dense);
-                    far[u] = far[u] && !near[u];
+                const bool local = inside && r >= 0;
+                cand += local ? dense : 0u;
+                heavy = local && dense > HEAVY;
+                if (!heavy) {
+                    const unsigned long long best = segment_min(rows.csr, x0, x1, s);
+                    const float d = __uint_as_float((unsigned)(best >> 32));
+                    near = !local && dense && seeds && near_seed(s, d, g.inv_h, dense);
+                    far = !local && !near;
+                    if (near)
+                        w.d2[l] = d;
+                    if (far || SEARCH_ONLY) {   // (a far query's seed, or the answer)
+                        a.nn[i] = (int)(unsigned)best;
+                        a.d2[i] = d;
+                    }
+                    w.nn[l] = far ? -1 : (int)(unsigned)best;
+                } else {
+                    w.nn[l] = -1;
+                }
+            }
+            const unsigned nm = __ballot_sync(FULL_MASK, near), fm = __ballot_sync(FULL_MASK, far);
+            if (near)
+                w.near[n_near + __popc(nm & lanemask_lt())] = (unsigned char)l;
+            if (far)
+                w.far[n_far + __popc(fm & lanemask_lt())] = (unsigned char)l;
+            n_near += __popc(nm);
+            n_far += __popc(fm);
+            const unsigned hm = __ballot_sync(FULL_MASK, heavy);
+            if (hm) {   // dense segments: listed right away
+                int slot = lane == 0 ? atomicAdd(&ctl->hv_count, __popc(hm)) : 0;
+                slot = __shfl_sync(FULL_MASK, slot, 0) + __popc(hm & lanemask_lt());
+                if (heavy) {
+                    if (slot < a.list_cap)
+                        a.hv_list[slot] = make_int4(it.pair, i, (int)x0, (int)x1);
+                    else
+                        atomicOr(&ctl->err, DEVERR_BOUNDS);
                 }
             }
         }
-        // list the queries for phase 2: warp slots by shared atomics, one
-        // global atomic per list and block
-        unsigned fm[PPT], nm[PPT], hm[PPT];
-        int fb_w[PPT], nr_w[PPT], hv_w[PPT];
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            fm[u] = __ballot_sync(FULL_MASK, far[u]);
-            nm[u] = __ballot_sync(FULL_MASK, near[u]);
-            hm[u] = __ballot_sync(FULL_MASK, heavy[u]);
-            fb_w[u] = nr_w[u] = hv_w[u] = 0;
-            if (lane == 0) {
-                if (fm[u])
-                    fb_w[u] = atomicAdd(&s_fb, __popc(fm[u]));
-                if (nm[u])
-                    nr_w[u] = atomicAdd(&s_nr, __popc(nm[u]));
-                if (hm[u])
-                    hv_w[u] = atomicAdd(&s_hv, __popc(hm[u]));
-            }
-        }
-        const unsigned long long wc = warp_sum_u64(cand);
-        if (lane == 0 && wc)
-            atomicAdd(&s_cand, wc);
-        __syncthreads();
-        if (tid == 0) {
-            if (s_cand)
-                atomicAdd(&ctl->stat_local_cand, s_cand);
-            atomicAdd(&ctl->stat_queries, (unsigned long long)(it.i1 - it.i0));
-            if (s_fb)
-                s_fb_base = atomicAdd(&ctl->fb_count, s_fb);
-            if (s_nr)
-                s_nr_base = atomicAdd(&ctl->nr_count, s_nr);
-            if (s_hv)
-                s_hv_base = atomicAdd(&ctl->hv_count, s_hv);
-        }
-        __syncthreads();
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            const int i = it.i0 + tid + TH * u;
-            const int fbw = __shfl_sync(FULL_MASK, fb_w[u], 0), nrw = __shfl_sync(FULL_MASK, nr_w[u], 0),
-                      hvw = __shfl_sync(FULL_MASK, hv_w[u], 0);
-            if (near[u]) {
-                const int slot = s_nr_base + nrw + __popc(nm[u] & lanemask_lt());
-                if (slot < a.list_cap)
-                    a.fb_list[a.list_cap - 1 - slot] = make_int2(it.pair, i);
-                else
-                    atomicOr(&ctl->err, DEVERR_BOUNDS);
-            }
-            if (far[u]) {
-                const int slot = s_fb_base + fbw + __popc(fm[u] & lanemask_lt());
-                if (slot < a.list_cap)
-                    a.fb_list[slot] = make_int2(it.pair, i);
-                else
-                    atomicOr(&ctl->err, DEVERR_BOUNDS);
-            }
-            if (heavy[u]) {
-                const int slot = s_hv_base + hvw + __popc(hm[u] & lanemask_lt());
-                if (slot < a.list_cap)
-                    a.hv_list[slot] = make_int4(it.pair, i, (int)ra[u], (int)rb[u]);
+        queries += (unsigned)n;
+        near_done += (unsigned)n_near;
+        __syncwarp();
+        if (n_far) {   // one global atomic a tile
+            int slot0 = lane == 0 ? atomicAdd(&ctl->fb_count, n_far) : 0;
+            slot0 = __shfl_sync(FULL_MASK, slot0, 0);
+            for (int k = lane; k < n_far; k += 32) {
+                if (slot0 + k < a.list_cap)
+                    a.fb_list[slot0 + k] = make_int2(it.pair, it.i0 + w.far[k]);
                 else
                     atomicOr(&ctl->err, DEVERR_BOUNDS);
             }
         }
-        __syncthreads();   // s_item and the counters are rewritten for the next item
+        if (n_near)
+            near_cand += near_tile<SEARCH_ONLY>(a, w, it, n_near);
+        if constexpr (!SEARCH_ONLY) {
+            // the sums of the points answered here, and which are left
+            const unsigned left = sum_tile<F64>(a, w, it, itx);
+            if (__any_sync(FULL_MASK, left != 0u)) {
+                if (lane < BATCH_TILE_MAX / 32)
+                    a.left[(size_t)itx * (BATCH_TILE_MAX / 32) + lane] = left;
+                if (lane == 0)
+                    a.open_items[atomicAdd(&ctl->open_count, 1)] = itx;
+            }
+        }
+    }
+    {
+        const unsigned long long c = warp_sum_u64(cand), gl = warp_sum_u64(near_cand);
+        if (lane == 0) {
+            if (c)
+                atomicAdd(&s_cand, c);
+            if (gl)
+                atomicAdd(&s_glob, gl);
+            if (queries)
+                atomicAdd(&s_queries, (unsigned long long)queries);
+            if (near_done)
+                atomicAdd(&s_near, (unsigned long long)near_done);
+        }
     }
     if (!grid_barrier(ctl, &s_flag))
         return;
 
-    // ---- phase 2: dense segments, then global searches, a warp each -------
-    {
-        const int F = min(*(volatile int *)&ctl->fb_count, a.list_cap);
-        const int N = min(*(volatile int *)&ctl->nr_count, a.list_cap - F);
-        const int Hv = min(*(volatile int *)&ctl->hv_count, a.list_cap);
-        const int n_warps = gridDim.x * WARPS, gw = blockIdx.x * WARPS + warp;
-        unsigned long long examined = 0ull;   // far queries: every lane counts the same
-        unsigned examined_near = 0u;          // near queries: each lane its own
-        const int lanes = n_warps * 32;
-        {   // dense segments, 8 to 32 lanes each
-            const int shift = group_shift(Hv, lanes, HEAVY_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
-            const int sub = lane & (G - 1);
-            for (int q0 = (n_warps - 1 - gw) * pack; q0 < Hv; q0 += n_warps * pack) {
-                const int q = q0 + (lane >> shift);
-                const int4 e = q < Hv ? a.hv_list[q] : make_int4(-1, -1, 0, 0);
-                const bool on = (unsigned)e.x < (unsigned)a.n_pairs && (unsigned)e.y < (unsigned)a.list_cap &&
-                                e.z <= e.w && (unsigned)e.w <= (unsigned)a.n_stored;
-                if (!on && q < Hv)   // a stale entry: skip it, report it
+    // ---- phase 2: dense segments and far queries of all pairs ---------------
+    const int F = min(*(volatile int *)&ctl->fb_count, a.list_cap);
+    const int Hv = min(*(volatile int *)&ctl->hv_count, a.list_cap);
+    if (tid == 0) {
+        if (blockIdx.x == 0)
+            ctl->item_next = 0u;   // (every tile is taken)
+        if (s_cand)
+            atomicAdd(&ctl->stat_local_cand, s_cand);
+        if (s_queries)
+            atomicAdd(&ctl->stat_queries, s_queries);
+        if (s_near)
+            atomicAdd(&ctl->stat_fallbacks, s_near);
+    }
+    unsigned long long examined = 0ull;   // far queries: every lane counts the same
+    {   // dense segments, 4 to 32 lanes each
+        const int shift = group_shift(Hv, n_warps * 32, HEAVY_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
+        const int sub = lane & (G - 1);
+        for (int q0 = (n_warps - 1 - gw) * pack; q0 < Hv; q0 += n_warps * pack) {
+            const int q = q0 + (lane >> shift);
+            const int4 e = q < Hv ? a.hv_list[q] : make_int4(-1, -1, 0, 0);
+            const bool on = (unsigned)e.x < (unsigned)a.n_pairs && (unsigned)e.y < (unsigned)a.list_cap &&
+                            e.z <= e.w && (unsigned)e.w <= (unsigned)a.n_stored;
+            if (!on && q < Hv)   // a stale entry: skip it, report it
+                atomicOr(&ctl->err, DEVERR_BOUNDS);
+            unsigned long long best = ~0ull;
+            if (on)
+                best = group_scan(a.csr, (unsigned)e.z, (unsigned)e.w,
+                                  transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y)), sub, G);
+            best = group_min(best, G);
+            if (on && sub == 0) {
+                a.nn[e.y] = (int)(unsigned)best;
+                a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
+            }
+        }
+    }
+    // far queries: a first chunk per warp, then chunks to whichever warp is
+    // free (a ticket per chunk): their costs vary widely, and a fixed share
+    // per warp leaves the whole grid waiting at the barrier for the warp
+    // that drew the slowest ones
+    const int far_chunk = min(max(F / (4 * n_warps), 1), 4);
+    for (int q0 = gw * far_chunk; q0 < F;) {
+        for (int qi = q0; qi < min(q0 + far_chunk, F); ++qi) {
+            const int2 e = a.fb_list[qi];
+            if ((unsigned)e.x >= (unsigned)a.n_pairs || (unsigned)e.y >= (unsigned)a.list_cap) {
+                if (lane == 0)   // a stale entry: skip it, report it
                     atomicOr(&ctl->err, DEVERR_BOUNDS);
-                unsigned long long best = ~0ull;
-                if (on)
-                    best = group_scan(a.csr, (unsigned)e.z, (unsigned)e.w,
-                                      transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y)), sub, G);
-                best = group_min(best, G);
-                if (on && sub == 0) {
-                    a.nn[e.y] = (int)(unsigned)best;
-                    a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
-                }
+                continue;
+            }
+            const BatchPair *bp = a.pairs + e.x;
+            const float3 s = transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y));
+            const int tbase = bp->tbase;
+            const unsigned long long best = global_search(
+                s, a.bpts, a.bbox + 2 * bp->bbase, a.sb_box + 2 * bp->sbbase, a.state[e.x].n_super, a.tgt + tbase,
+                bp->n_tgt, a.outside + tbase, a.state[e.x].n_outside, lane, examined,
+                nn_key(__ldcg(a.d2 + e.y), __ldcg(a.nn + e.y)));
+            __syncwarp();   // every lane has read the seed
+            if (lane == 0) {
+                a.nn[e.y] = (int)(unsigned)best;
+                a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
             }
         }
-        // far queries: a first chunk per warp, then chunks to whichever warp is
-        // free (a ticket per chunk): their costs vary widely, and a fixed share
-        // per warp leaves the whole grid waiting at the barrier for the warp
-        // that drew the slowest ones
-        const int far_chunk = min(max(F / (4 * n_warps), 1), 4);
-        for (int q0 = gw * far_chunk; q0 < F;) {
-            for (int qi = q0; qi < min(q0 + far_chunk, F); ++qi) {
-                const int2 e = a.fb_list[qi];
-                if ((unsigned)e.x >= (unsigned)a.n_pairs || (unsigned)e.y >= (unsigned)a.list_cap) {
-                    if (lane == 0)   // a stale entry: skip it, report it
-                        atomicOr(&ctl->err, DEVERR_BOUNDS);
-                    continue;
-                }
-                const BatchPair *bp = a.pairs + e.x;
-                const float3 s = transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y));
-                const int tbase = bp->tbase;
-                const unsigned long long best = global_search(
-                    s, a.bpts, a.bbox + 2 * bp->bbase, a.sb_box + 2 * bp->sbbase, a.state[e.x].n_super, a.tgt + tbase,
-                    bp->n_tgt, a.outside + tbase, a.state[e.x].n_outside, lane, examined,
-                    nn_key(__ldcg(a.d2 + e.y), __ldcg(a.nn + e.y)));
-                __syncwarp();   // every lane has read the seed
-                if (lane == 0) {
-                    a.nn[e.y] = (int)(unsigned)best;
-                    a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
-                }
-            }
-            if ((long long)n_warps * far_chunk >= F)
-                break;
-            if (lane == 0)
-                q0 = far_chunk * (n_warps + (int)atomicAdd(&ctl->fb_next, 1u));
-            q0 = __shfl_sync(FULL_MASK, q0, 0);
-        }
-        // near queries: 8 to 32 lanes each, a warp's worth at a time, in the
-        // same way
-        {
-            const int shift = group_shift(N, lanes, NEAR_SHIFT_MIN), G = 1 << shift, pack = 32 >> shift;
-            const int sub = lane & (G - 1);
-            const int packs = (N + pack - 1) / pack, chunk = min(max(packs / (4 * n_warps), 1), 8);
-            for (int p0 = gw * chunk; p0 < packs;) {
-                for (int p = p0; p < min(p0 + chunk, packs); ++p) {
-                    const int q = p * pack + (lane >> shift);
-                    const int2 e = q < N ? a.fb_list[a.list_cap - 1 - q] : make_int2(-1, -1);
-                    const bool on = (unsigned)e.x < (unsigned)a.n_pairs && (unsigned)e.y < (unsigned)a.list_cap;
-                    if (!on && q < N)   // a stale entry: skip it, report it
-                        atomicOr(&ctl->err, DEVERR_BOUNDS);
-                    const BatchPair *bp = a.pairs + (on ? e.x : 0);
-                    const long long vb = bp->vbase;
-                    float3 s = make_float3(0.0f, 0.0f, 0.0f);
-                    unsigned long long best = ~0ull;
-                    int no = 0;
-                    if (on) {
-                        s = transform_pt(load_posef(a.posef, e.x), __ldg(a.src + e.y));
-                        best = nn_key(__ldcg(a.d2 + e.y), __ldcg(a.nn + e.y));
-                        no = a.state[e.x].n_outside;
-                        const int tbase = bp->tbase;
-                        for (int o = sub; o < no; o += G) {   // target points outside the grid
-                            const int j = __ldg(a.outside + tbase + o);
-                            best = umin64(best, nn_key(dist2(s, __ldg(a.tgt + tbase + j)), j));
-                        }
-                        examined_near += sub == 0 ? (unsigned)no : 0u;
-                    }
-                    if (__any_sync(FULL_MASK, no > 0))
-                        best = group_min(best, G);
-                    best = near_search(bp->g, CsrRows{a.occ + (vb >> 5), a.off + vb, (unsigned)a.n_stored, a.csr}, s,
-                                       best, on, sub, G, examined_near);
-                    if (on && sub == 0) {
-                        a.nn[e.y] = (int)(unsigned)best;
-                        a.d2[e.y] = __uint_as_float((unsigned)(best >> 32));
-                    }
-                }
-                if ((long long)n_warps * chunk >= packs)
-                    break;
-                if (lane == 0)
-                    p0 = chunk * (n_warps + (int)atomicAdd(&ctl->nr_next, 1u));
-                p0 = __shfl_sync(FULL_MASK, p0, 0);
-            }
-        }
-        examined = warp_sum_u64((lane == 0 ? examined : 0ull) + examined_near);
-        if (lane == 0 && examined)
-            atomicAdd(&ctl->stat_global_cand, examined);
+        if ((long long)n_warps * far_chunk >= F)
+            break;
+        if (lane == 0)
+            q0 = far_chunk * (n_warps + (int)atomicAdd(&ctl->fb_next, 1u));
+        q0 = __shfl_sync(FULL_MASK, q0, 0);
+    }
+    if (lane == 0 && examined)
+        atomicAdd(&s_glob, examined);
+    if (F + Hv) {   // (the same in every block: the lists are complete)
         if (!grid_barrier(ctl, &s_flag))
             return;
         if (blockIdx.x == 0 && tid == 0) {   // every block has read the list lengths
-            ctl->stat_fallbacks += (unsigned long long)(F + N);
+            ctl->stat_fallbacks += (unsigned long long)F;
             ctl->fb_count = 0;
-            ctl->nr_count = 0;
             ctl->hv_count = 0;
             ctl->fb_next = 0u;
-            ctl->nr_next = 0u;
         }
+    } else {
+        __syncthreads();
     }
-    if (a.search_only)
+    if (tid == 0 && s_glob)
+        atomicAdd(&ctl->stat_global_cand, s_glob);
+    if constexpr (SEARCH_ONLY)
         return;
 
-    // ---- phase 3: per-item sums; the last item of a pair solves it --------
-    if constexpr (F64) {
-        batch_phase3_f64<TH, PPT>(a, s_dyn, s_item, s_skip, s_last, s_pose);
-        return;
+    // ---- phase 3: what phase 2 answered joins its tiles' sums ---------------
+    if (F + Hv) {
+        const int n_open = min(__ldcg(&ctl->open_count), a.n_items);
+        for (int o = gw; o < n_open; o += n_warps) {
+            const int itx = __ldcg(a.open_items + o);
+            const BatchItem it = a.items[itx];
+            const BatchPair *bp = a.pairs + it.pair;
+            const unsigned left =
+                lane < BATCH_TILE_MAX / 32 ? __ldcg(a.left + (size_t)itx * (BATCH_TILE_MAX / 32) + lane) : 0u;
+            const PoseF P = load_posef(a.posef, it.pair);
+            T acc[N_SUMS];
+#pragma unroll
+            for (int k = 0; k < N_SUMS; ++k)
+                acc[k] = S::zero();
+#pragma unroll 1
+            for (int l0 = 0; l0 < it.i1 - it.i0; l0 += 32) {
+                const unsigned m = __shfl_sync(FULL_MASK, left, l0 >> 5);
+                if (!((m >> lane) & 1u))
+                    continue;
+                const int i = it.i0 + l0 + lane;
+                const int j = __ldcg(a.nn + i);
+                if ((unsigned)j < (unsigned)bp->n_tgt)
+                    S::accumulate(acc, transform_pt(P, __ldg(a.src + i)), __ldg(a.tgt + bp->tbase + j), bp);
+                else   // no valid match: report, leave it out
+                    atomicOr(&ctl->err, DEVERR_BOUNDS);
+            }
+            __syncwarp();
+            const T v = tile_sum<F64>(acc, w);
+            float2 *part = a.partials + (size_t)itx * N_SUMS;
+            if (lane < N_SUMS)
+                S::store(part + lane, S::add(S::load(part + lane), v));
+        }
+        if (!grid_barrier(ctl, &s_flag))
+            return;
+        if (blockIdx.x == 0 && tid == 0)
+            ctl->open_count = 0;
     }
-    float(*s_thi)[N_SUMS][33] = reinterpret_cast<float(*)[N_SUMS][33]>(s_dyn);
-    float(*s_tlo)[N_SUMS][33] = reinterpret_cast<float(*)[N_SUMS][33]>(s_dyn + WARPS * N_SUMS * 33);
-    for (int itx = blockIdx.x; itx < a.n_items; itx += gridDim.x) {
-        if (tid == 0) {
-            s_item = a.items[itx];
-            s_skip = *(volatile const int *)&a.state[s_item.pair].stop;
-        }
-        __syncthreads();
-        const BatchItem it = s_item;
-        if (s_skip) {
-            __syncthreads();
+
+    // ---- and a block per pair adds the pair's tiles in a fixed order and
+    // solves: thread t adds sum t % 16 of tiles t / 16, t / 16 + TH / 16, ...;
+    // then the groups in order (pairs of them by a shuffle, then the warps) ---
+    __shared__ T s_w[WARPS][N_SUMS], s_tot[N_SUMS];
+    for (int p = blockIdx.x; p < a.n_pairs; p += gridDim.x) {
+        BatchState *stp = a.state + p;
+        const int stop = __ldcg(&stp->stop);
+        __syncthreads();   // (read by all before it can change; s_w is free)
+        if (stop)
             continue;
+        const BatchPair *bp = a.pairs + p;
+        const int k = tid & 15, n_items = bp->n_items;
+        const float2 *p0 = a.partials + (size_t)bp->item0 * N_SUMS + k;
+        T v = S::zero();
+        for (int b = tid >> 4; b < n_items; b += 8 * (TH / 16)) {   // eight loads in flight
+            T x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                x[u] = b + u * (TH / 16) < n_items ? S::load(p0 + (size_t)(b + u * (TH / 16)) * N_SUMS) : S::zero();
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                v = S::add(v, x[u]);
         }
-        load_pose_f_block(a.pose + 16 * it.pair, s_pose);
-        const PoseF P = s_pose;
-        const BatchPair *bp = a.pairs + it.pair;
-        const float3 cf = make_float3(bp->cx, bp->cy, bp->cz);
-        const int tbase = bp->tbase, n_tgt = bp->n_tgt;
-        dfl acc[N_SUMS];
-#pragma unroll
-        for (int k = 0; k < N_SUMS; ++k)
-            acc[k] = {0.0f, 0.0f};
-        int j[PPT];
-        float4 p[PPT], q[PPT];
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            const int i = it.i0 + tid + TH * u;
-            j[u] = -1;
-            if (i < it.i1) {
-                j[u] = __ldcg(a.nn + i);
-                p[u] = __ldg(a.src + i);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < PPT; ++u) {
-            if ((unsigned)j[u] < (unsigned)n_tgt)
-                q[u] = __ldg(a.tgt + tbase + j[u]);
-            else if (it.i0 + tid + TH * u < it.i1)   // no valid match: report, leave it out
-                atomicOr(&ctl->err, DEVERR_BOUNDS);
-        }
-#pragma unroll
-        for (int u = 0; u < PPT; ++u)
-            if ((unsigned)j[u] < (unsigned)n_tgt)
-                accumulate_corr(acc, transform_pt(P, p[u]), q[u], cf);
-        // warp sums through shared memory: lane l adds value l % 16 over
-        // lanes 16 (l / 16) .. 16 (l / 16) + 15 in order, then the halves
-#pragma unroll
-        for (int k = 0; k < N_SUMS; ++k) {
-            s_thi[warp][k][lane] = acc[k].hi;
-            s_tlo[warp][k][lane] = acc[k].lo;
-        }
-        __syncwarp();
-        {
-            const int k = lane & 15, h = (lane >> 4) * 16;
-            dfl v = {s_thi[warp][k][h], s_tlo[warp][k][h]};
-#pragma unroll
-            for (int t = 1; t < 16; ++t)
-                v = df_acc(v, dfl{s_thi[warp][k][h + t], s_tlo[warp][k][h + t]});
-            v = df_acc(v, df_shfl_xor(v, 16));
-            if (lane < 16) {
-                s_whi[warp][k] = v.hi;
-                s_wlo[warp][k] = v.lo;
-            }
-        }
+        v = S::add(v, S::shfl_xor(v, 16));
+        if (lane < N_SUMS)
+            s_w[warp][lane] = v;
         __syncthreads();
-        if (tid < N_SUMS) {   // the block's warps, in order
-            dfl v = {s_whi[0][tid], s_wlo[0][tid]};
+        if (warp == 0) {
+            if (lane < N_SUMS) {
+                T t = s_w[0][lane];
 #pragma unroll
-            for (int w = 1; w < WARPS; ++w)
-                v = df_acc(v, dfl{s_whi[w][tid], s_wlo[w][tid]});
-            a.partials[(size_t)itx * N_SUMS + tid] = make_float2(v.hi, v.lo);
-            __threadfence();
-        }
-        __syncthreads();
-        if (tid == 0)
-            s_last = atomicAdd(&a.state[it.pair].items_done, 1u) == (unsigned)(bp->n_items - 1);
-        __syncthreads();
-        if (s_last) {
-            __threadfence();
-            // the pair's item sums in item order: thread t adds value t % 16
-            // of items t/16, t/16 + TH/16, ...; the groups are then added in
-            // order (pairs of groups by a shuffle, then the warps)
-            const int item0 = bp->item0, n_items = bp->n_items;
-            {
-                const int k = tid & 15, grp = tid >> 4;
-                dfl v = {0.0f, 0.0f};
-                for (int b = grp; b < n_items; b += TH / 16) {
-                    const float2 x = __ldcg(a.partials + (size_t)(item0 + b) * N_SUMS + k);
-                    v = df_acc(v, dfl{x.x, x.y});
-                }
-                v = df_acc(v, df_shfl_xor(v, 16));
-                if (lane < 16) {
-                    s_whi[warp][lane] = v.hi;
-                    s_wlo[warp][lane] = v.lo;
-                }
+                for (int q = 1; q < WARPS; ++q)
+                    t = S::add(t, s_w[q][lane]);
+                s_tot[lane] = t;
             }
-            __syncthreads();
-            if (tid < N_SUMS) {
-                dfl t = {s_whi[0][tid], s_wlo[0][tid]};
-#pragma unroll
-                for (int w = 1; w < WARPS; ++w)
-                    t = df_acc(t, dfl{s_whi[w][tid], s_wlo[w][tid]});
-                s_tot[tid] = t;
-            }
-            __syncthreads();
-            if (warp == 0) {
-                double rmse;
-                BatchState *stp = a.state + it.pair;
-                const bool ok = solve_update(s_tot, bp->n_src, cf, a.pose + 16 * it.pair, rmse);
-                if (lane == 0) {
-                    stp->items_done = 0u;
-                    stp->last_rmse = rmse;
-                    if (!ok) {
-                        stp->err |= DEVERR_DEGENERATE;
+            __syncwarp();
+            double rmse;
+            const bool ok = S::solve(s_tot, bp, a.pose + 16 * p, rmse);
+            if (lane == 0) {
+                stp->last_rmse = rmse;
+                if (!ok) {
+                    stp->err |= DEVERR_DEGENERATE;
+                    stp->stop = 1;
+                    atomicOr(&ctl->err, DEVERR_DEGENERATE);
+                } else {
+                    const int it = stp->iters;
+                    stp->iters = it + 1;
+                    if (a.eps > 0.0 && it >= 1 && fabs(rmse - stp->prev_rmse) < a.eps)
                         stp->stop = 1;
-                        atomicOr(&ctl->err, DEVERR_DEGENERATE);
-                    } else {
-                        const int k = stp->iters;
-                        stp->iters = k + 1;
-                        if (a.eps > 0.0 && k >= 1 && fabs(rmse - stp->prev_rmse) < a.eps)
-                            stp->stop = 1;
-                        stp->prev_rmse = rmse;
-                    }
+                    stp->prev_rmse = rmse;
                 }
             }
         }
-        __syncthreads();   // s_item, s_pose and the sums are rewritten for the next item
     }
 }
 
+// (Tiles have at most 64 x ppt and at most BATCH_TILE_MAX points, fewer where
+// the batch has few points: 64 to 256 differ by under 3% on 256 pairs, and the
+// searches alone prefer 128, 64 x 20k points 107 us against 125 with 256.)
 const BatchShape BATCH_SHAPES[BATCH_N_SHAPES] = {
-    {256, 4, 2},   // 1024-point items
-    {256, 2, 3},   // 512-point items, more warps per SM
-    {512, 2, 1},   // 1024-point items, wide blocks
-    {128, 4, 4},   // 512-point items, narrow blocks
-    {256, 8, 2},   // 2048-point items
-    {256, 2, 4},   // 512-point items, 64 registers: more warps per SM
-    {256, 2, 5},   // 512-point items, 48 registers (spills some of the reduction's sums)
+    {256, 4, 2},   // 128 registers
+    {256, 2, 3},   // 80 registers, more warps per SM
+    {512, 2, 1},   // wide blocks
+    {128, 4, 4},   // narrow blocks
+    {256, 8, 2},   // as 0
+    {256, 2, 4},   // 64 registers
+    {256, 2, 5},   // 48 registers (spills some of the sums)
 };
 
 using IterKernel = void (*)(const BatchIterArgs);
 
-static IterKernel iter_kernel(int shape, bool f64)
+static IterKernel iter_kernel(int shape, BatchMode mode)
 {
+    const bool f64 = mode == BATCH_FP64;
+    if (mode == BATCH_SEARCH)   // without the sums every shape's searches run best with the most warps
+        return k_batch_iter<256, 2, false, true, 4>;
     switch (shape) {
-    case 0: return f64 ? k_batch_iter<256, 4, 2, true> : k_batch_iter<256, 4, 2, false>;
-    case 1: return f64 ? k_batch_iter<256, 2, 3, true> : k_batch_iter<256, 2, 3, false>;
-    case 2: return f64 ? k_batch_iter<512, 2, 1, true> : k_batch_iter<512, 2, 1, false>;
-    case 3: return f64 ? k_batch_iter<128, 4, 4, true> : k_batch_iter<128, 4, 4, false>;
-    case 4: return f64 ? k_batch_iter<256, 8, 2, true> : k_batch_iter<256, 8, 2, false>;
-    case 5: return f64 ? k_batch_iter<256, 2, 4, true> : k_batch_iter<256, 2, 4, false>;
-    case 6: return f64 ? k_batch_iter<256, 2, 5, true> : k_batch_iter<256, 2, 5, false>;
+    case 0: case 4: return f64 ? k_batch_iter<256, 2, true> : k_batch_iter<256, 2, false>;
+    case 1: return f64 ? k_batch_iter<256, 3, true> : k_batch_iter<256, 3, false>;
+    case 2: return f64 ? k_batch_iter<512, 1, true> : k_batch_iter<512, 1, false>;
+    case 3: return f64 ? k_batch_iter<128, 4, true> : k_batch_iter<128, 4, false>;
+    case 5: return f64 ? k_batch_iter<256, 4, true> : k_batch_iter<256, 4, false>;
+    case 6: return f64 ? k_batch_iter<256, 5, true> : k_batch_iter<256, 5, false>;
     }
     return nullptr;
 }
 
-// 2 x WARPS x 16 x 33 floats = WARPS x 16 x 33 doubles
-static size_t iter_smem(int shape) { return (size_t)2 * (BATCH_SHAPES[shape].threads / 32) * N_SUMS * 33 * 4; }
+static int iter_threads(int shape, BatchMode mode) { return mode == BATCH_SEARCH ? 256 : BATCH_SHAPES[shape].threads; }
+static size_t iter_smem(int threads) { return (size_t)(threads / 32) * sizeof(WarpTile); }
 
-int batch_iter_blocks(int shape, bool f64)
+int batch_tile_points(int shape, int blocks, long long m)
+{
+    const long long warps = (long long)blocks * (BATCH_SHAPES[shape].threads / 32);
+    const long long most = std::min(64 * BATCH_SHAPES[shape].ppt, BATCH_TILE_MAX);
+    const long long rounds = (m + 64 * warps - 1) / std::max(64 * warps, 1ll);   // two tiles a warp where the batch is small
+    return (int)std::min(std::max(32 * rounds, 32ll), most);
+}
+
+int batch_iter_blocks(int shape, BatchMode mode)
 {
     if (shape < 0 || shape >= BATCH_N_SHAPES)
         return 0;
-    IterKernel k = iter_kernel(shape, f64);
-    const size_t smem = iter_smem(shape);
+    IterKernel k = iter_kernel(shape, mode);
+    const int threads = iter_threads(shape, mode);
+    const size_t smem = iter_smem(threads);
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -1181,22 +1155,22 @@ int batch_iter_blocks(int shape, bool f64)
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, BATCH_SHAPES[shape].threads, smem) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return sms * per_sm;
 }
 
-cudaError_t launch_batch_iter(int shape, bool f64, int blocks, const BatchIterArgs &a, cudaStream_t st)
+cudaError_t launch_batch_iter(int shape, BatchMode mode, int blocks, const BatchIterArgs &a, cudaStream_t st)
 {
-    IterKernel k = iter_kernel(shape, f64);
+    IterKernel k = iter_kernel(shape, mode);
     if (!k || blocks < 1)
         return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(BATCH_SHAPES[shape].threads);
-    cfg.dynamicSmemBytes = iter_smem(shape);
+    cfg.blockDim = dim3(iter_threads(shape, mode));
+    cfg.dynamicSmemBytes = iter_smem(iter_threads(shape, mode));
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;

@@ -49,21 +49,28 @@ struct BatchState {
 static_assert(sizeof(BatchState) == 48, "BatchState layout");
 
 // A tile of one pair's points: pooled indices [i0, i1), local index of i0.
+// (A block's of target points in the build, a warp's of source points in the
+// iterations.)
 struct BatchItem {
     int pair, i0, i1, l0;
 };
 
 constexpr int BATCH_TILE = 256;          // target points per build item (one block)
+constexpr int BATCH_TILE_MAX = 128;      // source points per iteration item, at most (one warp)
 constexpr int BATCH_SMEM_PAIRS = 2048;   // unit-start tables up to this many pairs go to shared memory
 
 // Iteration kernel shapes the autotuner chooses from: threads per block,
-// source points per thread (the item tile is their product) and the blocks
-// per SM the registers are budgeted for.
+// source points per thread (an item is a warp's tile of at most 64 times as
+// many) and the blocks per SM the registers are budgeted for.
 struct BatchShape {
     int threads, ppt, min_blocks;
 };
 constexpr int BATCH_N_SHAPES = 7;
 extern const BatchShape BATCH_SHAPES[BATCH_N_SHAPES];
+
+// What an iteration kernel does: an iteration with double-float or FP64 sums
+// and solve, or the searches alone (nn and d2 of every point).
+enum BatchMode { BATCH_DF = 0, BATCH_FP64 = 1, BATCH_SEARCH = 2 };
 
 // Arguments of one iteration of all pairs.
 struct BatchIterArgs {
@@ -87,17 +94,19 @@ struct BatchIterArgs {
     float *d2;                  // [M] squared distance
     const unsigned *occ;        // pooled occupancy bits
     float *posef;               // [P][12] the poses rounded to float (PoseF), written by phase 1 for phase 2
-    int2 *fb_list;              // global-search queries (pair, pooled source index): far ones from the
-                                // front, near ones (vicp_search.cuh) from the back
+    int2 *fb_list;              // far global queries (pair, pooled source index)
     int4 *hv_list;              // dense segments (pair, pooled source index, begin, end)
     int list_cap;               // capacity of each list (M)
-    float2 *partials;           // [n_items][16] double-float sums per item
+    float2 *partials;           // [n_items][16] double-float (or FP64) sums per item
+    unsigned *left;             // [n_items][4] bit masks of the item's points left to phase 2
+    int *open_items;            // [n_items] the items with such points
     DevCtl *ctl;                // fb_count, hv_count, barrier, stats, err
     double eps;                 // stopping threshold on the RMSE difference (<= 0: never)
-    int search_only;            // 1: phases 1-2 only (nn, d2), no reduction or update
     int test_leave_early;       // test hook: block 0 leaves before the first barrier
 };
 
+// Points per iteration item for m source points on `blocks` resident blocks.
+int batch_tile_points(int shape, int blocks, long long m);
 cudaError_t launch_batch_bbox(const float4 *pts, const BatchItem *items, int n_items, int P, unsigned *bbox,
                               cudaStream_t st);
 cudaError_t launch_batch_histogram(const float4 *pts, const BatchItem *items, int n_items, const BatchPair *pairs,
@@ -120,10 +129,10 @@ cudaError_t launch_batch_dilate(const unsigned *occ, const BatchPair *pairs, int
                                 int *root, unsigned char *ring, cudaStream_t st);
 // Resident blocks of the iteration kernel of a shape (0 if it cannot run);
 // f64: the variant with FP64 sums and solve.
-int batch_iter_blocks(int shape, bool f64);
+int batch_iter_blocks(int shape, BatchMode mode);
 // One iteration of every pair (or the search alone): a cooperative
 // persistent launch of `blocks` blocks (<= batch_iter_blocks(shape, f64)).
-cudaError_t launch_batch_iter(int shape, bool f64, int blocks, const BatchIterArgs &a, cudaStream_t st);
+cudaError_t launch_batch_iter(int shape, BatchMode mode, int blocks, const BatchIterArgs &a, cudaStream_t st);
 
 // Differentiable loss (vicp_diff.cu): SE(3) exponential T = Exp(xi) T0 and
 // J(xi)^T g (J the left Jacobian), one thread per pose; the loss of Eq. 1

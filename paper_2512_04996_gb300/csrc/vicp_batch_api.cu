@@ -57,6 +57,7 @@ struct vicp_batch {
     int items_shape = -1;
     std::vector<int> n_src_last;
     int tuned_shape = -1;
+    int blocks[3][BATCH_N_SHAPES];   // resident blocks by mode and shape; -1: not asked yet
 
     // iteration graph
     cudaGraphExec_t graph = nullptr;
@@ -64,14 +65,14 @@ struct vicp_batch {
     const void *g_src = nullptr;
     int g_shape = -1, g_iters = -1, g_M = -1, g_items = -1;
     double g_eps = 0.0;
-    bool g_f64 = false;
+    BatchMode g_mode = BATCH_DF;
     int last_graph = -1;             // the last registration's iterations: 1 graph replay, 0 direct
 
     // device buffers
     BBuf counts, off, root, ring, inter, occ, desc, tile_sum, rows, dirty;
     BBuf bcounts, boff, blist, brange, bslot, boxord, bbox, sb_box;
     BBuf keys, ids, csr, bpts, outside;
-    BBuf nn, d2, fb_list, hv_list, partials, sitems, posef;
+    BBuf nn, d2, fb_list, hv_list, partials, sitems, posef, left, open_items;
     BBuf pairs_d, state, pose, pose_save, titems, ustart_xy_d, ustart_z_d, bb, ctl;
     BBuf hsrc, htgt;
 };
@@ -417,6 +418,18 @@ int pick_shape(vicp_batch *b)
     return b->tuned_shape >= 0 ? b->tuned_shape : 0;
 }
 
+// The precision of this context's iterations (VICP_BATCH_FLAG_FP64).
+BatchMode mode_of(const vicp_batch *b) { return (b->params.flags & VICP_BATCH_FLAG_FP64) ? BATCH_FP64 : BATCH_DF; }
+
+// batch_iter_blocks of the context's device, asked once per shape.
+int iter_blocks(vicp_batch *b, int shape, BatchMode mode)
+{
+    int &n = b->blocks[mode][shape];
+    if (n < 0)
+        n = batch_iter_blocks(shape, mode);
+    return n;
+}
+
 // Source tiles of `shape` for these sizes; uploads the items and the pair
 // descriptors' item ranges when they changed.
 vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
@@ -427,7 +440,7 @@ vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
     const std::vector<int> ns(n_src, n_src + P);
     if (shape == b->items_shape && ns == b->n_src_last)
         return VICP_OK;
-    const int T = BATCH_SHAPES[shape].threads * BATCH_SHAPES[shape].ppt;
+    const int T = batch_tile_points(shape, iter_blocks(b, shape, mode_of(b)), M);
     std::vector<BatchItem> items;
     long long s = 0;
     for (int k = 0; k < P; ++k) {
@@ -443,6 +456,8 @@ vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
     cudaStream_t st = b->stream;
     BTRY(bensure(b, b->sitems, items.size() * sizeof(BatchItem), "source tiles"));
     BTRY(bensure(b, b->partials, items.size() * REDUCE_VALUES * sizeof(float2), "item sums"));
+    BTRY(bensure(b, b->left, items.size() * (BATCH_TILE_MAX / 32) * 4, "items' open points"));
+    BTRY(bensure(b, b->open_items, items.size() * 4, "items with open points"));
     BTRY(bensure(b, b->nn, (size_t)M * 4, "nn"));
     BTRY(bensure(b, b->d2, (size_t)M * 4, "d2"));
     BTRY(bensure(b, b->posef, (size_t)P * sizeof(PoseF), "float poses"));
@@ -460,21 +475,26 @@ vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
     return VICP_OK;
 }
 
-// Loop state of every pair (items_done .. last_rmse) and the search lists.
-vicp_status reset_loop(vicp_batch *b)
+// The search lists, the tickets and the barrier count.
+vicp_status reset_lists(vicp_batch *b)
 {
-    cudaStream_t st = b->stream;
-    BCUDA(b,
-          cudaMemset2DAsync((char *)b->state.p + offsetof(BatchState, items_done), sizeof(BatchState), 0,
-                            sizeof(BatchState) - offsetof(BatchState, items_done), b->P, st),
-          "loop state reset");
     DevCtl *d = bctl(b);
-    static_assert(offsetof(DevCtl, bar_count) - offsetof(DevCtl, fb_count) == 20, "list fields");
-    BCUDA(b, cudaMemsetAsync(&d->fb_count, 0, 24, st), "list, ticket and barrier reset");
+    static_assert(offsetof(DevCtl, bar_count) - offsetof(DevCtl, fb_count) == 24, "list fields");
+    BCUDA(b, cudaMemsetAsync(&d->fb_count, 0, 28, b->stream), "list, ticket and barrier reset");
     return VICP_OK;
 }
 
-BatchIterArgs iter_args(vicp_batch *b, const float4 *src, double *pose, int *nn, float *d2, int search_only)
+// Loop state of every pair (items_done .. last_rmse) and the search lists.
+vicp_status reset_loop(vicp_batch *b)
+{
+    BCUDA(b,
+          cudaMemset2DAsync((char *)b->state.p + offsetof(BatchState, items_done), sizeof(BatchState), 0,
+                            sizeof(BatchState) - offsetof(BatchState, items_done), b->P, b->stream),
+          "loop state reset");
+    return reset_lists(b);
+}
+
+BatchIterArgs iter_args(vicp_batch *b, const float4 *src, double *pose, int *nn, float *d2)
 {
     BatchIterArgs a{};
     a.src = src;
@@ -501,25 +521,24 @@ BatchIterArgs iter_args(vicp_batch *b, const float4 *src, double *pose, int *nn,
     a.hv_list = (int4 *)b->hv_list.p;
     a.list_cap = b->M;
     a.partials = (float2 *)b->partials.p;
+    a.left = (unsigned *)b->left.p;
+    a.open_items = (int *)b->open_items.p;
     a.ctl = bctl(b);
     a.eps = b->params.rmse_eps;
-    a.search_only = search_only;
     a.test_leave_early = (b->params.flags & VICP_BATCH_FLAG_TEST_BARRIER_TIMEOUT) ? 1 : 0;
     return a;
 }
 
-// FP64 sums and solve (VICP_BATCH_FLAG_FP64) for this context's iterations.
-bool fp64_of(const vicp_batch *b) { return (b->params.flags & VICP_BATCH_FLAG_FP64) != 0; }
 
-// `blocks`: batch_iter_blocks(shape, f64), queried by the caller outside any
+// `blocks`: iter_blocks(b, shape, mode), queried by the caller outside any
 // stream capture.
-vicp_status launch_iters(vicp_batch *b, int shape, bool f64, int blocks, const BatchIterArgs &a, int iters,
+vicp_status launch_iters(vicp_batch *b, int shape, BatchMode mode, int blocks, const BatchIterArgs &a, int iters,
                          cudaStream_t st)
 {
     if (blocks < 1)
         return bfail(b, VICP_ERR_CUDA, "iteration kernel shape %d cannot be resident", shape);
     for (int k = 0; k < iters; ++k)
-        BCUDA(b, launch_batch_iter(shape, f64, blocks, a, st), "launch of the batched iteration");
+        BCUDA(b, launch_batch_iter(shape, mode, blocks, a, st), "launch of the batched iteration");
     b->launches += iters;
     return VICP_OK;
 }
@@ -531,14 +550,14 @@ vicp_status run_iterations(vicp_batch *b, int shape, const float4 *src)
     const int iters = b->params.max_iters;
     if (iters == 0)
         return VICP_OK;
-    const BatchIterArgs a = iter_args(b, src, (double *)b->pose.p, (int *)b->nn.p, (float *)b->d2.p, 0);
-    const bool f64 = fp64_of(b);
-    const int blocks = batch_iter_blocks(shape, f64);
+    const BatchIterArgs a = iter_args(b, src, (double *)b->pose.p, (int *)b->nn.p, (float *)b->d2.p);
+    const BatchMode mode = mode_of(b);
+    const int blocks = iter_blocks(b, shape, mode);
     b->last_graph = 0;
     if ((b->params.flags & VICP_BATCH_FLAG_NO_GRAPH) || b->graph_broken)
-        return launch_iters(b, shape, f64, blocks, a, iters, b->stream);
+        return launch_iters(b, shape, mode, blocks, a, iters, b->stream);
     if (!b->graph || b->g_src != src || b->g_shape != shape || b->g_iters != iters || b->g_M != b->M ||
-        b->g_items != b->n_items || b->g_eps != b->params.rmse_eps || b->g_f64 != f64) {
+        b->g_items != b->n_items || b->g_eps != b->params.rmse_eps || b->g_mode != mode) {
         drop_graph(b);
         if (!b->capture)
             BCUDA(b, cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "capture stream");
@@ -546,7 +565,7 @@ vicp_status run_iterations(vicp_batch *b, int shape, const float4 *src)
         cudaError_t e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             const int64_t before = b->launches;
-            const vicp_status s = launch_iters(b, shape, f64, blocks, a, iters, b->capture);
+            const vicp_status s = launch_iters(b, shape, mode, blocks, a, iters, b->capture);
             b->launches = before;   // counted when replayed
             e = cudaStreamEndCapture(b->capture, &g);
             if (s != VICP_OK && e == cudaSuccess)
@@ -561,7 +580,7 @@ vicp_status run_iterations(vicp_batch *b, int shape, const float4 *src)
             cudaGetLastError();
             b->graph = nullptr;
             b->graph_broken = true;
-            return launch_iters(b, shape, f64, blocks, a, iters, b->stream);
+            return launch_iters(b, shape, mode, blocks, a, iters, b->stream);
         }
         b->g_src = src;
         b->g_shape = shape;
@@ -569,7 +588,7 @@ vicp_status run_iterations(vicp_batch *b, int shape, const float4 *src)
         b->g_M = b->M;
         b->g_items = b->n_items;
         b->g_eps = b->params.rmse_eps;
-        b->g_f64 = f64;
+        b->g_mode = mode;
     }
     BCUDA(b, cudaGraphLaunch(b->graph, b->stream), "graph launch");
     b->launches += iters;
@@ -648,7 +667,7 @@ vicp_status vicp_batch_shape_info(int32_t shape, int32_t *threads, int32_t *poin
     if (points_per_thread)
         *points_per_thread = BATCH_SHAPES[shape].ppt;
     if (resident_blocks)
-        *resident_blocks = batch_iter_blocks(shape, false);
+        *resident_blocks = batch_iter_blocks(shape, BATCH_DF);
     return VICP_OK;
 }
 
@@ -665,6 +684,9 @@ vicp_status vicp_batch_create(vicp_batch **out, const vicp_batch_params *params,
         return VICP_ERR_INVALID;
     vicp_batch *b = new vicp_batch();
     b->params = *params;
+    for (auto &per : b->blocks)
+        for (int &n : per)
+            n = -1;
     if (alloc) {
         b->alloc = *alloc;
         b->custom_alloc = true;
@@ -693,7 +715,7 @@ void vicp_batch_destroy(vicp_batch *b)
     BBuf *all[] = {&b->counts, &b->off, &b->root, &b->ring, &b->inter, &b->occ, &b->desc, &b->tile_sum, &b->rows,
                    &b->dirty, &b->bcounts, &b->boff, &b->blist, &b->brange, &b->bslot, &b->boxord, &b->bbox,
                    &b->sb_box, &b->keys, &b->ids, &b->csr, &b->bpts, &b->outside, &b->nn, &b->d2, &b->fb_list,
-                   &b->hv_list, &b->partials, &b->sitems, &b->posef, &b->pairs_d, &b->state, &b->pose, &b->pose_save,
+                   &b->hv_list, &b->partials, &b->sitems, &b->posef, &b->left, &b->open_items, &b->pairs_d, &b->state, &b->pose, &b->pose_save,
                    &b->titems, &b->ustart_xy_d, &b->ustart_z_d, &b->bb, &b->ctl, &b->hsrc, &b->htgt};
     for (BBuf *x : all)
         bfree(b, *x);
@@ -738,8 +760,8 @@ vicp_status vicp_batch_register_host(vicp_batch *b, int32_t n_pairs, const float
     return registration(b, (const float *)b->hsrc.p, n_src, poses, iters_out, rmse_out, status_out);
 }
 
-vicp_status vicp_batch_correspond(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
-                                  const double *poses_dev, int32_t *nn_out, float *d2_out)
+vicp_status vicp_batch_correspond_async(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
+                                        const double *poses_dev, int32_t *nn_out, float *d2_out)
 {
     if (!b)
         return VICP_ERR_INVALID;
@@ -749,10 +771,16 @@ vicp_status vicp_batch_correspond(vicp_batch *b, const float *src_xyzw, const in
         return bfail(b, VICP_ERR_INVALID, "vicp_batch_correspond: NULL or misaligned pointer");
     const int shape = pick_shape(b);
     BTRY(prepare_items(b, n_src, shape));
-    BTRY(reset_loop(b));
+    BTRY(reset_lists(b));
     const BatchIterArgs a = iter_args(b, reinterpret_cast<const float4 *>(src_xyzw), const_cast<double *>(poses_dev),
-                                      nn_out, d2_out, 1);
-    BTRY(launch_iters(b, shape, false, batch_iter_blocks(shape, false), a, 1, b->stream));   // search only
+                                      nn_out, d2_out);
+    return launch_iters(b, shape, BATCH_SEARCH, iter_blocks(b, shape, BATCH_SEARCH), a, 1, b->stream);   // search only
+}
+
+vicp_status vicp_batch_correspond(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
+                                  const double *poses_dev, int32_t *nn_out, float *d2_out)
+{
+    BTRY(vicp_batch_correspond_async(b, src_xyzw, n_src, poses_dev, nn_out, d2_out));
     const vicp_status s = read_status(b);
     return s == VICP_ERR_DEGENERATE ? VICP_OK : s;
 }
@@ -777,7 +805,7 @@ vicp_status vicp_batch_tune(vicp_batch *b, const float *src_xyzw, const int32_t 
     vicp_status s = VICP_OK;
     for (int shape = 0; shape < BATCH_N_SHAPES && s == VICP_OK; ++shape) {
         float ms = -1.0f;
-        if (batch_iter_blocks(shape, fp64_of(b)) > 0) {
+        if (iter_blocks(b, shape, mode_of(b)) > 0) {
             s = prepare_items(b, n_src, shape);
             for (int t = 0; t < trials && s == VICP_OK; ++t) {
                 if (cudaMemcpyAsync(b->pose.p, poses, (size_t)P * 16 * sizeof(double), cudaMemcpyHostToDevice, st) !=
@@ -790,10 +818,10 @@ vicp_status vicp_batch_tune(vicp_batch *b, const float *src_xyzw, const int32_t 
                     break;
                 const BatchIterArgs a =
                     iter_args(b, reinterpret_cast<const float4 *>(src_xyzw), (double *)b->pose.p, (int *)b->nn.p,
-                              (float *)b->d2.p, 0);
-                const int blocks = batch_iter_blocks(shape, fp64_of(b));
+                              (float *)b->d2.p);
+                const int blocks = iter_blocks(b, shape, mode_of(b));
                 cudaEventRecord(e0, st);
-                s = launch_iters(b, shape, fp64_of(b), blocks, a, iters, st);
+                s = launch_iters(b, shape, mode_of(b), blocks, a, iters, st);
                 cudaEventRecord(e1, st);
                 if (s != VICP_OK)
                     break;
@@ -928,10 +956,6 @@ vicp_status vicp_batch_loss(vicp_batch *b, const float *src_xyzw, const int32_t 
         (grad_src_out && !aligned16(grad_src_out)))
         return bfail(b, VICP_ERR_INVALID, "vicp_batch_loss: NULL or misaligned pointer");
     BTRY(prepare_items(b, n_src, pick_shape(b)));
-    BCUDA(b,
-          cudaMemset2DAsync((char *)b->state.p + offsetof(BatchState, items_done), sizeof(BatchState), 0,
-                            sizeof(unsigned), b->P, b->stream),
-          "ticket reset");
     BCUDA(b,
           launch_batch_loss(reinterpret_cast<const float4 *>(src_xyzw), b->target, (const BatchPair *)b->pairs_d.p,
                             (BatchState *)b->state.p, (const BatchItem *)b->sitems.p, b->n_items, poses_dev, nn_dev,

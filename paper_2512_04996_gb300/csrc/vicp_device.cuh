@@ -73,8 +73,10 @@ struct DevCtl {
     int nr_count;           // correspond: near global queries listed; reset with fb_count
     int hv_count;           // correspond: dense segments listed; reset with fb_count
     unsigned fb_next;       // batched iteration: next chunk of far queries; reset with fb_count
-    unsigned nr_next;       // batched iteration: next chunk of near queries; reset with fb_count
+    unsigned item_next;     // batched iteration: next item; reset with fb_count
+    int open_count;         // batched iteration: items with points left to phase 2; reset with fb_count
     unsigned bar_count;     // batched iteration: blocks arrived at the grid barrier
+    unsigned pad;
     // Work counters (added by the search kernels, read and cleared by the host).
     unsigned long long stat_queries;       // source points searched
     unsigned long long stat_fallbacks;     // of which took the global search
@@ -86,7 +88,7 @@ struct DevCtl {
     double prev_rmse;
     double last_rmse;
 };
-static_assert(sizeof(DevCtl) == 120, "DevCtl layout");
+static_assert(sizeof(DevCtl) == 128, "DevCtl layout");
 
 // Rigid transform rounded to float: R row-major, t.
 struct PoseF {

@@ -145,6 +145,7 @@ SIGNATURES = {
     "vicp_batch_register": (C.c_int, [_P, _P, _P, _P, _P, _P, _P]),
     "vicp_batch_register_host": (C.c_int, [_P, C.c_int32, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P]),
     "vicp_batch_correspond": (C.c_int, [_P, _P, _P, _P, _P, _P]),
+    "vicp_batch_correspond_async": (C.c_int, [_P, _P, _P, _P, _P, _P]),
     "vicp_batch_tune": (C.c_int, [_P, _P, _P, _P, C.c_int32, C.c_int32, C.POINTER(C.c_int32), _P]),
     "vicp_batch_pair_grid": (C.c_int, [_P, C.c_int32, C.POINTER(vicp_grid_view)]),
     "vicp_batch_report": (C.c_int, [_P, C.POINTER(C.c_uint64), C.POINTER(C.c_uint64), C.POINTER(vicp_stats),
@@ -661,6 +662,16 @@ class Batch:
         return st, T, it, rm, ps
 
     def correspond(self, source: torch.Tensor, n_src, poses: torch.Tensor):
+        return self._correspond(source, n_src, poses, self._lib.vicp_batch_correspond)
+
+    def _correspond_enqueued(self, source, n_src, poses):
+        """correspond without waiting for its end, where the caller works on the context's own stream (on another one
+        the end is waited for, as nothing else orders the two)."""
+        own = torch.cuda.current_stream(self.device) == self.stream
+        return self._correspond(source, n_src, poses, self._lib.vicp_batch_correspond_async if own
+                                else self._lib.vicp_batch_correspond)
+
+    def _correspond(self, source, n_src, poses, call):
         s = _cloud(source, "source")
         n = _sizes(n_src, self.n_pairs)
         if (poses.dtype != torch.float64 or not poses.is_cuda or poses.numel() != 16 * self.n_pairs
@@ -669,8 +680,8 @@ class Batch:
         m = s.shape[0]
         nn = torch.empty(m, dtype=torch.int32, device=s.device)
         d2 = torch.empty(m, dtype=torch.float32, device=s.device)
-        self._check(self._lib.vicp_batch_correspond(self.handle, s.data_ptr(), _ptr(n), poses.data_ptr(),
-                                                    nn.data_ptr(), d2.data_ptr()), "vicp_batch_correspond")
+        self._check(call(self.handle, s.data_ptr(), _ptr(n), poses.data_ptr(), nn.data_ptr(), d2.data_ptr()),
+                    "vicp_batch_correspond")
         return nn, d2
 
     def tune(self, source: torch.Tensor, n_src, poses=None, iters: int = 4, trials: int = 2):
@@ -846,7 +857,7 @@ class PointToPointLoss(torch.autograd.Function):
         xi64 = xi.detach().to(torch.float64).contiguous()
         T = vicp_se3_exp(xi64, T0)
         src = source.detach()
-        nn, _ = batch.correspond(src, n_src, T)
+        nn, _ = batch._correspond_enqueued(src, n_src, T)
         loss, _, _ = batch.loss(src, n_src, T, nn)
         ctx.batch, ctx.n_src, ctx.recompute = batch, n_src, recompute
         ctx.xi_dtype = xi.dtype
@@ -861,7 +872,7 @@ class PointToPointLoss(torch.autograd.Function):
     def backward(ctx, dloss):
         if ctx.recompute:
             xi64, T, src = ctx.saved_tensors
-            nn, _ = ctx.batch.correspond(src, ctx.n_src, T)
+            nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T)
         else:
             xi64, T, src, nn = ctx.saved_tensors
         dl = dloss.detach().to(torch.float64).contiguous()
