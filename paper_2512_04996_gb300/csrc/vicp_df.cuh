@@ -188,107 +188,12 @@ __device__ __forceinline__ void accumulate_corr(dfl (&acc)[N_SUMS], float3 s, fl
     acc[15] = df_acc(acc[15], df_acc(df_acc(df_mul(ex, ex), df_mul(ey, ey)), df_mul(ez, ez)));
 }
 
-// ---------------------------------------------------------------------------
-// The rigid update of Eq. 1 from the sums s_tot (shared memory) of m
-// correspondences, by one warp, every lane holding one entry of the
-// matrices involved so that the whole solve is one short stream of
-// instructions (a solve is latency-bound, and its code is fetched cold once
-// per iteration):
-//  * lanes 0..8: H = sum (s - sbar)(q - qbar)^T, entry (k / 3, k % 3), and
-//    its cofactors (rank test, det H); H, |H|_F^2 and the centred residual E
-//    are scaled by one power of two to |H|_F ~ 1, which changes neither the
-//    rotation nor any rounding.
-//  * Horn's closed form: the rotation minimising Eq. 1 is the unit
-//    quaternion (w, x, y, z) of the largest eigenvalue of the symmetric,
-//    traceless 4x4
-//      [ Sxx+Syy+Szz  Syz-Szy      Szx-Sxz      Sxy-Syx     ]
-//      [ Syz-Szy      Sxx-Syy-Szz  Sxy+Syx      Szx+Sxz     ]
-//      [ Szx-Sxz      Sxy+Syx     -Sxx+Syy-Szz  Syz+Szy     ]
-//      [ Sxy-Syx      Szx+Sxz      Syz+Szy     -Sxx-Syy+Szz ]
-//    (S = H), entry (k / 4, k % 4) on lane k < 16.  Its characteristic
-//    polynomial is l^4 + c2 l^2 + c1 l + c0, c2 = -2 |S|_F^2, c1 = -8 det S,
-//    c0 = det N (Laplace expansion over the 2x2 minors of rows 0-1 and 2-3,
-//    one column pair per lane).  The largest root: Newton's method from the
-//    upper bound (Ga + Gb) / 2 = E/2 + tr S, which lies just right of it
-//    (from the right of the largest root of a real-rooted polynomial Newton
-//    decreases monotonically onto it), in float, then polished in
-//    double-float (the polynomial in double-float, the derivative in float:
-//    each step gains the float precision again).
-//  * The eigenvector: a column of the adjugate of N - l I (rank one at a
-//    simple eigenvalue), all sixteen cofactors at once (lane k: cofactor
-//    (k / 4, k % 4)), the column of the largest diagonal cofactor taken.
-//  * R from the unnormalised quaternion q = (w, v), n = |q|^2:
-//    R_aa = (2 (w^2 + v_a^2) - n) / n, R_ab = 2 (v_a v_b - e_abc w v_c) / n.
-//  * t = qbar - R sbar, and lanes 0..11 compose pose <- dT * pose in FP64
-//    (lane 4a + b: entry (a, b)).
-// Returns false, leaving the pose untouched, when the geometry is degenerate
-// (rank(H) < 2).  rmse = the RMSE of the m correspondences, on every lane.
-// Every lane of the warp must call it.  Not inlined: one copy of its code
-// per kernel, which the single-pair kernel fetches ahead of the real solve.
-// ---------------------------------------------------------------------------
-static __device__ __noinline__ bool solve_update(const dfl *s_tot, int m, float3 cf, double *pose, double &rmse)
+// Horn's quaternion (unnormalised, on every lane) from H on lanes 0..8,
+// scaled to |H|_F ~ 1: s2 = |H|_F^2, dH = det H, E the centred residual in the
+// same scale (on every lane).  The steps are described at solve_update.
+__device__ __forceinline__ void horn_vector(dfl h, dfl s2, dfl dH, dfl E, dfl (&v)[4])
 {
     const int lane = threadIdx.x & 31;
-    // the pose column this lane composes, loaded first
-    const int pc = lane & 3;
-    double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
-    if (lane < 12) {
-        P0 = pose[pc];
-        P1 = pose[4 + pc];
-        P2 = pose[8 + pc];
-        P3 = pose[12 + pc];
-    }
-    const float mh = (float)m;
-    const dfl invM = df_rcp(dfl{mh, (float)((long long)m - (long long)mh)});
-
-    // H entry (a, b) on lane 3a + b < 9:
-    //   sum (s - c)_a (q - c)_b - (sum (s - c)_a)(sum (q - c)_b) / M;
-    // lanes 0..2: the centring term (sum (s - q)_a)^2 / M of the residual
-    const int a = lane < 9 ? lane / 3 : 0, b = lane < 9 ? lane - 3 * a : 0;
-    dfl h = {0.0f, 0.0f}, e = {0.0f, 0.0f};
-    if (lane < 9)
-        h = df_sub(s_tot[6 + lane], df_mul(df_mul(s_tot[a], invM), s_tot[3 + b]));
-    if (lane < 3) {
-        const dfl d = df_sub(s_tot[lane], s_tot[3 + lane]);
-        e = df_mul(df_mul(d, invM), d);
-    }
-    dfl s2 = df_mul(h, h);
-    warp_sum_df2(s2, e);
-    const dfl S15 = s_tot[15];
-    rmse = df_to_double(df_sqrt(df_mul(S15, invM)));
-    dfl E = df_sub(S15, e);
-    if (!(s2.hi > 0.0f) || !isfinite(s2.hi))
-        return false;
-    {
-        int ex;
-        frexpf(__fsqrt_rn(s2.hi), &ex);
-        const float sc = ldexpf(1.0f, -ex);
-        h = df_scale(h, sc);
-        s2 = df_scale(s2, sc * sc);
-        E = df_scale(E, sc);
-    }
-
-    // cofactors of H (cyclic index order gives the sign), the rank test and
-    // det H = sum_b H_0b C_0b
-    dfl cof = {0.0f, 0.0f}, dH = {0.0f, 0.0f};
-    {
-        const int a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
-        const int b1 = b == 2 ? 0 : b + 1, b2 = b == 0 ? 2 : b - 1;
-        const dfl h11 = df_shfl(h, 3 * a1 + b1), h22 = df_shfl(h, 3 * a2 + b2);
-        const dfl h12 = df_shfl(h, 3 * a1 + b2), h21 = df_shfl(h, 3 * a2 + b1);
-        if (lane < 9) {
-            cof = df_sub(df_mul(h11, h22), df_mul(h12, h21));
-            if (lane < 3)
-                dH = df_mul(h, cof);
-        }
-    }
-    dfl c2s = df_mul(cof, cof);
-    warp_sum_df2(c2s, dH);
-    // rank(H) < 2: every 2x2 minor negligible against |H|_F^2 (a definition
-    // shared with the oracle, not its code): |cof(H)|_F <= 1e-12 |H|_F^2
-    if (c2s.hi <= 1e-24f * (s2.hi * s2.hi))
-        return false;
-
     // N entry (ni, nj) on lane 4 ni + nj (lanes 16..31 repeat lanes 0..15):
     // a signed sum of two or three entries of H
     const int ni = (lane >> 2) & 3, nj = lane & 3;
@@ -399,7 +304,6 @@ static __device__ __noinline__ bool solve_update(const dfl *s_tot, int m, float3
             }
         }
     }
-    dfl v[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
         v[k] = df_shfl(ca, 4 * k + col);
@@ -412,6 +316,111 @@ static __device__ __noinline__ bool solve_update(const dfl *s_tot, int m, float3
         for (int k = 0; k < 4; ++k)
             v[k] = df_scale(v[k], sc);
     }
+}
+
+// ---------------------------------------------------------------------------
+// The rigid update of Eq. 1 from the sums s_tot (shared memory) of m
+// correspondences, by one warp, every lane holding one entry of the
+// matrices involved so that the whole solve is one short stream of
+// instructions (a solve is latency-bound, and its code is fetched cold once
+// per iteration):
+//  * lanes 0..8: H = sum (s - sbar)(q - qbar)^T, entry (k / 3, k % 3), and
+//    its cofactors (rank test, det H); H, |H|_F^2 and the centred residual E
+//    are scaled by one power of two to |H|_F ~ 1, which changes neither the
+//    rotation nor any rounding.
+//  * Horn's closed form: the rotation minimising Eq. 1 is the unit
+//    quaternion (w, x, y, z) of the largest eigenvalue of the symmetric,
+//    traceless 4x4
+//      [ Sxx+Syy+Szz  Syz-Szy      Szx-Sxz      Sxy-Syx     ]
+//      [ Syz-Szy      Sxx-Syy-Szz  Sxy+Syx      Szx+Sxz     ]
+//      [ Szx-Sxz      Sxy+Syx     -Sxx+Syy-Szz  Syz+Szy     ]
+//      [ Sxy-Syx      Szx+Sxz      Syz+Szy     -Sxx-Syy+Szz ]
+//    (S = H), entry (k / 4, k % 4) on lane k < 16.  Its characteristic
+//    polynomial is l^4 + c2 l^2 + c1 l + c0, c2 = -2 |S|_F^2, c1 = -8 det S,
+//    c0 = det N (Laplace expansion over the 2x2 minors of rows 0-1 and 2-3,
+//    one column pair per lane).  The largest root: Newton's method from the
+//    upper bound (Ga + Gb) / 2 = E/2 + tr S, which lies just right of it
+//    (from the right of the largest root of a real-rooted polynomial Newton
+//    decreases monotonically onto it), in float, then polished in
+//    double-float (the polynomial in double-float, the derivative in float:
+//    each step gains the float precision again).
+//  * The eigenvector: a column of the adjugate of N - l I (rank one at a
+//    simple eigenvalue), all sixteen cofactors at once (lane k: cofactor
+//    (k / 4, k % 4)), the column of the largest diagonal cofactor taken.
+//  * R from the unnormalised quaternion q = (w, v), n = |q|^2:
+//    R_aa = (2 (w^2 + v_a^2) - n) / n, R_ab = 2 (v_a v_b - e_abc w v_c) / n.
+//  * t = qbar - R sbar, and lanes 0..11 compose pose <- dT * pose in FP64
+//    (lane 4a + b: entry (a, b)).
+// Returns false, leaving the pose untouched, when the geometry is degenerate
+// (rank(H) < 2).  rmse = the RMSE of the m correspondences, on every lane.
+// Every lane of the warp must call it.  Not inlined: one copy of its code
+// per kernel, which the single-pair kernel fetches ahead of the real solve.
+// ---------------------------------------------------------------------------
+static __device__ __noinline__ bool solve_update(const dfl *s_tot, int m, float3 cf, double *pose, double &rmse)
+{
+    const int lane = threadIdx.x & 31;
+    // the pose column this lane composes, loaded first
+    const int pc = lane & 3;
+    double P0 = 0.0, P1 = 0.0, P2 = 0.0, P3 = 0.0;
+    if (lane < 12) {
+        P0 = pose[pc];
+        P1 = pose[4 + pc];
+        P2 = pose[8 + pc];
+        P3 = pose[12 + pc];
+    }
+    const float mh = (float)m;
+    const dfl invM = df_rcp(dfl{mh, (float)((long long)m - (long long)mh)});
+
+    // H entry (a, b) on lane 3a + b < 9:
+    //   sum (s - c)_a (q - c)_b - (sum (s - c)_a)(sum (q - c)_b) / M;
+    // lanes 0..2: the centring term (sum (s - q)_a)^2 / M of the residual
+    const int a = lane < 9 ? lane / 3 : 0, b = lane < 9 ? lane - 3 * a : 0;
+    dfl h = {0.0f, 0.0f}, e = {0.0f, 0.0f};
+    if (lane < 9)
+        h = df_sub(s_tot[6 + lane], df_mul(df_mul(s_tot[a], invM), s_tot[3 + b]));
+    if (lane < 3) {
+        const dfl d = df_sub(s_tot[lane], s_tot[3 + lane]);
+        e = df_mul(df_mul(d, invM), d);
+    }
+    dfl s2 = df_mul(h, h);
+    warp_sum_df2(s2, e);
+    const dfl S15 = s_tot[15];
+    rmse = df_to_double(df_sqrt(df_mul(S15, invM)));
+    dfl E = df_sub(S15, e);
+    if (!(s2.hi > 0.0f) || !isfinite(s2.hi))
+        return false;
+    {
+        int ex;
+        frexpf(__fsqrt_rn(s2.hi), &ex);
+        const float sc = ldexpf(1.0f, -ex);
+        h = df_scale(h, sc);
+        s2 = df_scale(s2, sc * sc);
+        E = df_scale(E, sc);
+    }
+
+    // cofactors of H (cyclic index order gives the sign), the rank test and
+    // det H = sum_b H_0b C_0b
+    dfl cof = {0.0f, 0.0f}, dH = {0.0f, 0.0f};
+    {
+        const int a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
+        const int b1 = b == 2 ? 0 : b + 1, b2 = b == 0 ? 2 : b - 1;
+        const dfl h11 = df_shfl(h, 3 * a1 + b1), h22 = df_shfl(h, 3 * a2 + b2);
+        const dfl h12 = df_shfl(h, 3 * a1 + b2), h21 = df_shfl(h, 3 * a2 + b1);
+        if (lane < 9) {
+            cof = df_sub(df_mul(h11, h22), df_mul(h12, h21));
+            if (lane < 3)
+                dH = df_mul(h, cof);
+        }
+    }
+    dfl c2s = df_mul(cof, cof);
+    warp_sum_df2(c2s, dH);
+    // rank(H) < 2: every 2x2 minor negligible against |H|_F^2 (a definition
+    // shared with the oracle, not its code): |cof(H)|_F <= 1e-12 |H|_F^2
+    if (c2s.hi <= 1e-24f * (s2.hi * s2.hi))
+        return false;
+
+    dfl v[4];
+    horn_vector(h, s2, dH, E, v);
     const dfl nq = df_add(df_add(df_mul(v[0], v[0]), df_mul(v[1], v[1])), df_add(df_mul(v[2], v[2]), df_mul(v[3], v[3])));
     const dfl inv_nq = df_rcp(nq);
 
