@@ -413,7 +413,7 @@ VICP_API vicp_status vicp_fixed_view(vicp_ctx *ctx, const float **slots_out, con
  * 4x4x4-brick groups per axis); larger grids return VICP_ERR_GRID_TOO_LARGE.
  * Every call, on any stream or host thread, shares that one array: calls on
  * one device that overlap in time race and give wrong results, so callers
- * must serialise them.  Each call clears the parts that must start at zero.
+ * must serialise them.  Each call clears what the last one left.
  * The first call on a device looks up the array's device address (once per
  * device, with that device current).  The address is kept for the life of
  * the process, so the library must not be used on a device after

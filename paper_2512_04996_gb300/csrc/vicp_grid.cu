@@ -144,28 +144,30 @@ __global__ void __launch_bounds__(256) k_histogram(const float4 *__restrict__ pt
     }
     if (idx >= 0 && lane == __ffs(peers) - 1)
         atomicAdd(counts + idx, (unsigned)__popc(peers));
-    const unsigned bpeers = __match_any_sync(FULL_MASK, bk);
-    // the brick's exact bounds: the group's min and max of each coordinate
-    // (order-preserving unsigned images of the floats; maxima as their
-    // complements, so every word is an atomicMin from all ones)
-    const unsigned ox = float_to_ordered(q.x), oy = float_to_ordered(q.y), oz = float_to_ordered(q.z);
-    const unsigned mnx = __reduce_min_sync(bpeers, ox), mny = __reduce_min_sync(bpeers, oy),
-                   mnz = __reduce_min_sync(bpeers, oz);
-    const unsigned cmx = __reduce_min_sync(bpeers, ~ox), cmy = __reduce_min_sync(bpeers, ~oy),
-                   cmz = __reduce_min_sync(bpeers, ~oz);
-    if (bk >= 0 && lane == __ffs(bpeers) - 1) {
-        // the group that makes a brick non-empty counts it for its super-brick
-        // (the scatter writes a super-brick's box when its last brick is done)
-        if (atomicAdd(bcounts + bk, (unsigned)__popc(bpeers)) == 0u && sb_left)
-            atomicAdd(sb_left + bk / SUPER_BRICKS, 1u);
-        if (boxk) {
-            unsigned *b = boxk + 8 * bk;
-            atomicMin(b + 0, mnx);
-            atomicMin(b + 1, mny);
-            atomicMin(b + 2, mnz);
-            atomicMin(b + 4, cmx);
-            atomicMin(b + 5, cmy);
-            atomicMin(b + 6, cmz);
+    if (bcounts) {   // (null: a caller without the brick level)
+        const unsigned bpeers = __match_any_sync(FULL_MASK, bk);
+        // the brick's exact bounds: the group's min and max of each coordinate
+        // (order-preserving unsigned images of the floats; maxima as their
+        // complements, so every word is an atomicMin from all ones)
+        const unsigned ox = float_to_ordered(q.x), oy = float_to_ordered(q.y), oz = float_to_ordered(q.z);
+        const unsigned mnx = __reduce_min_sync(bpeers, ox), mny = __reduce_min_sync(bpeers, oy),
+                       mnz = __reduce_min_sync(bpeers, oz);
+        const unsigned cmx = __reduce_min_sync(bpeers, ~ox), cmy = __reduce_min_sync(bpeers, ~oy),
+                       cmz = __reduce_min_sync(bpeers, ~oz);
+        if (bk >= 0 && lane == __ffs(bpeers) - 1) {
+            // the group that makes a brick non-empty counts it for its super-brick
+            // (the scatter writes a super-brick's box when its last brick is done)
+            if (atomicAdd(bcounts + bk, (unsigned)__popc(bpeers)) == 0u && sb_left)
+                atomicAdd(sb_left + bk / SUPER_BRICKS, 1u);
+            if (boxk) {
+                unsigned *b = boxk + 8 * bk;
+                atomicMin(b + 0, mnx);
+                atomicMin(b + 1, mny);
+                atomicMin(b + 2, mnz);
+                atomicMin(b + 4, cmx);
+                atomicMin(b + 5, cmy);
+                atomicMin(b + 6, cmz);
+            }
         }
     }
     // occupancy bit of the voxel (one atomicOr per word and warp)
@@ -442,8 +444,8 @@ cudaError_t launch_brick_scan(const unsigned *bcounts, const GridGeom &g, unsign
 // untouched while the scan runs (predecessors are read throughout); the
 // scatter, which runs next, zeroes them for the following build.
 //
-// Output.  Dense (512 threads x 1 word): every off[v], staged in shared
-// memory and written with coalesced 16-byte stores.  Sparse (256 threads x
+// Output.  Dense (512 threads x 1 word): every off[v], written with coalesced
+// 16-byte stores, staged in shared memory where a warp's voxels hold points.  Sparse (256 threads x
 // 2 words, the build's form): only the entries the build and the searches
 // read -- off[v] and off[v + 1] of every occupied voxel v, off[32 k] for
 // every occupancy word k, and off[V] -- about 1/15 of the array's bytes at
@@ -592,7 +594,7 @@ template <int THREADS, int WPT, bool DENSE>
 __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
     k_scan(const unsigned *__restrict__ counts, long long V, unsigned *__restrict__ off,
            const unsigned *__restrict__ occ, const unsigned *__restrict__ tile_sum,
-           unsigned long long *__restrict__ desc, const DevCtl *__restrict__ ctl)
+           unsigned long long *__restrict__ desc, const DevCtl *__restrict__ ctl, unsigned *__restrict__ mismatch)
 {
     static_assert(THREADS * WPT * 32 == SCAN_TILE, "tile");
     static_assert(!DENSE || WPT == 1, "the dense output stages one word per thread");
@@ -667,6 +669,8 @@ __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
     }
     unsigned tile_total;
     const unsigned thread_excl = block_excl_scan<WARPS>(sum, s_w, &tile_total);   // also orders s_epoch
+    if (DENSE && mismatch && tid == 0 && tile_total != __ldg(tile_sum + tile))
+        atomicOr(mismatch, DEVERR_BOUNDS);   // the counts are not this cloud's alone
     const unsigned long long tag = (unsigned long long)s_epoch << 34;
 
     // lookback: LOOKBACK predecessors per round, nearest first (thread i
@@ -757,50 +761,101 @@ __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
         return;
     }
 
-    // the 32 offsets of this thread, staged in shared memory (row stride 33
-    // words: conflict-free both ways) and written out with coalesced 16-byte
-    // stores
-    extern __shared__ unsigned s_off[];   // [THREADS][33]
+    // the 32 offsets of each thread, written with coalesced 16-byte stores by
+    // warps: a warp's 1024 voxels without a point (nearly all of them: half a
+    // percent of the voxels hold one) all have the warp's first offset, the
+    // others are staged in the warp's shared memory (row stride 33 words:
+    // conflict-free both ways)
+    extern __shared__ unsigned s_off[];   // [WARPS][32][33]
+    unsigned *own = s_off + warp * (32 * 33);
+    const long long wbase = (long long)tile * SCAN_TILE + 1024 * warp;
+    const bool empty = !__any_sync(FULL_MASK, bits[0] != 0u);
+    const unsigned first = run;
+    if (!empty) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {   // the counts again, from L1
-        s_off[tid * 33 + i] = run;
-        run += ((bits[0] >> i) & 1u) ? __ldg(counts + base + i) : 0u;
+        for (int i = 0; i < 32; ++i) {   // the counts again, from L1
+            own[lane * 33 + i] = run;
+            run += ((bits[0] >> i) & 1u) ? __ldg(counts + base + i) : 0u;
+        }
+        __syncwarp();
     }
     if (base < V && base + 32 >= V)   // the thread holding voxel V-1 closes the array
         off[V] = run;
-    __syncthreads();
-    const long long tbase = (long long)tile * SCAN_TILE;
 #pragma unroll
-    for (int j = 0; j < SCAN_TILE / (4 * THREADS); ++j) {
-        const int v = 4 * tid + 4 * THREADS * j;   // voxel within the tile
-        const unsigned *r = s_off + (v >> 5) * 33 + (v & 31);
-        const long long gv = tbase + v;
+    for (int j = 0; j < 8; ++j) {
+        const int v = 4 * lane + 128 * j;   // voxel within the warp's
+        const unsigned *r = own + (v >> 5) * 33 + (v & 31);
+        const uint4 o = empty ? make_uint4(first, first, first, first) : make_uint4(r[0], r[1], r[2], r[3]);
+        const long long gv = wbase + v;
         if (gv + 4 <= V) {
-            *reinterpret_cast<uint4 *>(off + gv) = make_uint4(r[0], r[1], r[2], r[3]);
+            *reinterpret_cast<uint4 *>(off + gv) = o;
         } else {
+            const unsigned x[4] = {o.x, o.y, o.z, o.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (gv + i < V)
-                    off[gv + i] = r[i];
+                    off[gv + i] = x[i];
         }
     }
 }
 
+// ---------------------------------------------------------------------------
+// Puts counts and occupancy bits back to zero from the occupancy bits (a
+// counted voxel's bit is set), with the tile totals and the control block:
+// one pass over the bits and the few words they name instead of a memset of
+// every array.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_clear_counted(unsigned *__restrict__ counts, unsigned *__restrict__ occ,
+                                                       long long words, unsigned *__restrict__ tile_sum, int n_tiles,
+                                                       DevCtl *__restrict__ ctl)
+{
+    pdl_begin();
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (t < n_tiles)
+        tile_sum[t] = 0u;
+    if (t < (long long)(sizeof(DevCtl) / 4))
+        reinterpret_cast<unsigned *>(ctl)[t] = 0u;
+    uint4 *o4 = reinterpret_cast<uint4 *>(occ) + t;   // four words a thread
+    if (4 * t + 4 > words)
+        return;
+    const uint4 b = *o4;
+    if (!(b.x | b.y | b.z | b.w))
+        return;
+    *o4 = make_uint4(0u, 0u, 0u, 0u);
+    const unsigned w[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!w[k])
+            continue;
+        uint4 *c4 = reinterpret_cast<uint4 *>(counts + 32 * (4 * t + k));
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            c4[q] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
+cudaError_t launch_clear_counted(unsigned *counts, unsigned *occ, long long words, unsigned *tile_sum, int n_tiles,
+                                 DevCtl *ctl, cudaStream_t st)
+{
+    return launch_kernel(k_clear_counted, dim3((unsigned)((words / 4 + 255) / 256)), dim3(256), 0, st, counts, occ,
+                         words, tile_sum, n_tiles, ctl);
+}
+
 cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off, const unsigned *occ,
                         const unsigned *tile_sum, unsigned long long *desc, const DevCtl *ctl, cudaStream_t st,
-                        bool dense)
+                        bool dense, unsigned *mismatch)
 {
     const long long tiles = scan_tiles(g.V);
     if (!dense)
         return launch_kernel(k_scan<256, 2, false>, dim3((unsigned)tiles), dim3(256), 0, st, counts, g.V, off, occ,
-                             tile_sum, desc, ctl);
+                             tile_sum, desc, ctl, mismatch);
     constexpr int T = 512;
     const size_t smem = (size_t)T * 33 * sizeof(unsigned);
     cudaError_t e = cudaFuncSetAttribute(k_scan<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
     return launch_kernel(k_scan<T, 1, true>, dim3((unsigned)tiles), dim3(T), smem, st, counts, g.V, off, occ,
-                         tile_sum, desc, ctl);
+                         tile_sum, desc, ctl, mismatch);
 }
 
 // ---------------------------------------------------------------------------

@@ -68,6 +68,7 @@ inline int reduce_blocks(int m, int sms)
 
 cudaError_t launch_bbox(const float4 *pts, int n, unsigned *bbox6, cudaStream_t st);
 // occ must hold zeros (the previous build's scatter clears it).
+// bcounts null: no brick level.
 // sb_left and boxk (may be null): per super-brick, its non-empty bricks are
 // counted up (the scatter counts them down again); per brick key, 8 words of
 // bounds are merged into boxk (all ones before the build).  after_solve:
@@ -86,10 +87,17 @@ cudaError_t launch_histogram(const float4 *pts, int n, const GridGeom &g, int *k
                              float4 *copy_out = nullptr);
 // dense: every off[v]; sparse: only off[v] and off[v + 1] of occupied voxels,
 // off[32 k] and off[V] (what the build and the searches read) -- the rest
-// is completed by launch_offsets_fill on the same occupancy bits.
+// is completed by launch_offsets_fill on the same occupancy bits.  mismatch
+// (dense; may be null): DEVERR_BOUNDS is set in it when a tile's counts do not
+// add up to its total.  desc may be null up to 4096 tiles.
 cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off, const unsigned *occ,
                         const unsigned *tile_sum, unsigned long long *desc, const DevCtl *ctl, cudaStream_t st,
-                        bool dense);
+                        bool dense, unsigned *mismatch = nullptr);
+// Zeroes the counts of the voxels whose bits are set in occ (words of it, a
+// multiple of four; both arrays 16-byte aligned), those words, the tile totals
+// (n_tiles <= words / 4) and the control block.
+cudaError_t launch_clear_counted(unsigned *counts, unsigned *occ, long long words, unsigned *tile_sum, int n_tiles,
+                                 DevCtl *ctl, cudaStream_t st);
 cudaError_t launch_offsets_fill(unsigned *off, const unsigned *occ, long long V, cudaStream_t st);
 // sums: brick_tiles(slots) words of scratch (used by large grids).
 constexpr int BM_MAX_BRICKS = 65536;   // up to this many slots one launch, past it two

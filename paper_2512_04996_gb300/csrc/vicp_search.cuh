@@ -446,19 +446,21 @@ __device__ __forceinline__ unsigned long long scan_chunk(const float4 *__restric
     return best;
 }
 
-// Lane `sub` of a group of G lanes: its part of the run [a, b) (four loads in
-// flight); the group's minimum is the run's.
+// Lane `sub` of a group of G lanes: its part of the run [a, b) (GROUP_AHEAD
+// loads in flight); the group's minimum is the run's.
+constexpr int GROUP_AHEAD = 8;
+
 __device__ __forceinline__ unsigned long long group_scan(const float4 *__restrict__ pts, unsigned a, unsigned b,
                                                          float3 s, int sub, int G)
 {
     unsigned long long best = ~0ull;
-    for (unsigned i = a + (unsigned)sub; i < b; i += 4u * G) {
-        float4 q[4];
+    for (unsigned i = a + (unsigned)sub; i < b; i += (unsigned)(GROUP_AHEAD * G)) {
+        float4 q[GROUP_AHEAD];
 #pragma unroll
-        for (int u = 0; u < 4; ++u)   // (past the end: the run's last point again)
+        for (int u = 0; u < GROUP_AHEAD; ++u)   // (past the end: the run's last point again)
             q[u] = __ldg(pts + min(i + (unsigned)(u * G), b - 1u));
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < GROUP_AHEAD; ++u)
             best = umin64(best, nn_key(dist2(s, q[u]), __float_as_int(q[u].w)));
     }
     return best;

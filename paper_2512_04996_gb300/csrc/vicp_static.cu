@@ -8,7 +8,7 @@
 // inside another framework that owns all device memory through its own
 // allocator.  This entry point therefore uses only a scratch area that the
 // library holds in static device memory: the per-voxel counts, occupancy
-// bits, scan tile sums and descriptors, brick counts and a control block.
+// bits, scan tile sums and a control block.
 // The caller passes the inputs and the outputs.
 #include <cmath>
 #include <cstdint>
@@ -26,16 +26,17 @@ constexpr long long MAX_BRICK_SLOTS = VICP_STATIC_MAX_BRICK_SLOTS;
 
 constexpr size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Scratch layout (bytes from the start of the array).
+// Scratch layout (bytes from the start of the array).  (So few scan tiles
+// need no descriptors.)
+constexpr long long MAX_TILES = (MAX_V + SCAN_TILE - 1) / SCAN_TILE;
+constexpr long long OCC_WORDS = ((MAX_V + 31) / 32 + 2 + 3) / 4 * 4;
 constexpr size_t OFF_CTL = 0;
 constexpr size_t OFF_COUNTS = OFF_CTL + align256(sizeof(DevCtl));
-constexpr size_t OFF_OCC = OFF_COUNTS + align256(MAX_V * 4);
-constexpr size_t OFF_TILES = OFF_OCC + align256(((MAX_V + 31) / 32 + 2) * 4);
-constexpr size_t OFF_DESC = OFF_TILES + align256(((MAX_V + SCAN_TILE - 1) / SCAN_TILE) * 4);
-constexpr size_t OFF_BRICKS = OFF_DESC + align256(((MAX_V + SCAN_TILE - 1) / SCAN_TILE) * 8);
-constexpr size_t SCRATCH_BYTES = OFF_BRICKS + align256(MAX_BRICK_SLOTS * 4);
+constexpr size_t OFF_OCC = OFF_COUNTS + align256((size_t)OCC_WORDS * 32 * 4);   // (whole words' voxels)
+constexpr size_t OFF_TILES = OFF_OCC + align256((size_t)OCC_WORDS * 4);
+constexpr size_t SCRATCH_BYTES = OFF_TILES + align256((size_t)MAX_TILES * 4);
 
-// About 70 MiB, held on every GPU that loads the library until the process
+// About 66 MiB, held on every GPU that loads the library until the process
 // exits.  Host code never hands `g_scratch` itself to a kernel: kernels get
 // the address that cudaGetSymbolAddress returns for the current device.
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
@@ -112,33 +113,33 @@ extern "C" VICP_API vicp_status vicp_offsets_static(const float *target_xyzw, in
     unsigned *counts = reinterpret_cast<unsigned *>(base + OFF_COUNTS);
     unsigned *occ = reinterpret_cast<unsigned *>(base + OFF_OCC);
     unsigned *tiles = reinterpret_cast<unsigned *>(base + OFF_TILES);
-    unsigned long long *desc = reinterpret_cast<unsigned long long *>(base + OFF_DESC);
-    unsigned *bcounts = reinterpret_cast<unsigned *>(base + OFF_BRICKS);
 
     // The scratch keeps the last call's contents: clear everything that must
-    // start at zero.
-    const long long nt = scan_tiles(g.V);
-    cudaError_t e = cudaMemsetAsync(ctl, 0, sizeof(DevCtl), st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(counts, 0, (size_t)g.V * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(tiles, 0, (size_t)nt * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(desc, 0, (size_t)nt * 8, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(bcounts, 0, (size_t)brick_slots(g) * 4, st);
-    if (e == cudaSuccess)
-        e = cudaMemsetAsync(occ, 0, (size_t)occ_words(g.V) * 4, st);
-    if (e == cudaSuccess)
-        e = launch_histogram(reinterpret_cast<const float4 *>(target_xyzw), n, g, keys_out, counts, bcounts, occ,
-                             tiles, nullptr, nullptr, ctl, st, false);
-    if (e == cudaSuccess)
-        e = launch_scan(counts, g, offsets_out, occ, tiles, desc, ctl, st, true);
+    // start at zero, found by the occupancy bits (all of them: the last grid
+    // may have been the larger one).  (Six memsets, of 4 bytes a voxel among
+    // them, were about a third of a call on the 226k scene.)  The scan checks
+    // that the counts add up to the points counted: calls that overlapped, or
+    // one that failed half way, may have left counts without a bit, and then
+    // the whole scratch is cleared and the work done again.
     unsigned err = 0;
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(&err, &ctl->err, sizeof err, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess)
-        e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaSuccess;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        if (attempt > 0)
+            e = cudaMemsetAsync(base, 0, SCRATCH_BYTES, st);
+        if (e == cudaSuccess)
+            e = launch_clear_counted(counts, occ, OCC_WORDS, tiles, (int)MAX_TILES, ctl, st);
+        if (e == cudaSuccess)
+            e = launch_histogram(reinterpret_cast<const float4 *>(target_xyzw), n, g, keys_out, counts, nullptr, occ,
+                                 tiles, nullptr, nullptr, ctl, st, false);
+        if (e == cudaSuccess)
+            e = launch_scan(counts, g, offsets_out, occ, tiles, nullptr, ctl, st, true, &ctl->err);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(&err, &ctl->err, sizeof err, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess)
+            e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess || !(err & DEVERR_BOUNDS))
+            break;
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return VICP_ERR_CUDA;
