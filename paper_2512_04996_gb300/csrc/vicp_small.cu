@@ -22,8 +22,10 @@
 // points 384-459 us against 709-753, 16,384 points 479-618 against 725-839
 // (objects, by their share of global queries); one step of 1,000 points 17.8
 // against 22.5.  What bounds it now is the chain of an iteration: root,
-// offset, points, the lists' rows, and the solve.  Past 16,384 points the
-// cluster's share of the SMs is the limit and the separate kernels serve.
+// offset, points, the lists' rows, and the solve.  Past 16,384 points 16
+// SMs are too few for clouds with many global queries and the separate kernels
+// serve (three points a thread, 24,576 points: 565-914 us against 775-1,025;
+// five, 40,960: an object 762 against 821, but a scene 1,497 against 952).
 // The sums are bit-reproducible from run to run.  The slots of two
 // iterations alternate: a block overwrites a slot only after the barrier
 // that every reader of it has passed.
@@ -35,9 +37,8 @@ namespace vicp {
 
 constexpr int SM_THREADS = 512, SM_WARPS = SM_THREADS / 32;
 constexpr int SM_CLUSTER = 16;
-constexpr int SM_PPT = SMALL_MAX_POINTS / (SM_CLUSTER * SM_THREADS);   // points per thread
-constexpr int SM_POINTS = SM_THREADS * SM_PPT;                         // points per block
-static_assert(SM_PPT * SM_CLUSTER * SM_THREADS == SMALL_MAX_POINTS, "points per thread");
+constexpr int SM_PPT_MAX = SMALL_MAX_POINTS / (SM_CLUSTER * SM_THREADS);   // points per thread, at most
+static_assert(SM_PPT_MAX * SM_CLUSTER * SM_THREADS == SMALL_MAX_POINTS, "points per thread");
 constexpr size_t SM_SMEM = (size_t)2 * SM_WARPS * N_SUMS * 33 * sizeof(float);   // transposed per-lane sums
 
 __device__ __forceinline__ unsigned cluster_rank()
@@ -62,8 +63,10 @@ __device__ __forceinline__ void store_remote(dfl *p, unsigned rank, dfl v)
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(r), "f"(v.hi), "f"(v.lo) : "memory");
 }
 
+template <int SM_PPT>
 __global__ void __launch_bounds__(SM_THREADS, 1) k_small_iters(const SmallArgs a)
 {
+    constexpr int SM_POINTS = SM_THREADS * SM_PPT;   // points per block
     pdl_begin();
     if (a.honor_stop && *(volatile int *)&a.ctl->stop)   // (the same for every block)
         return;
@@ -334,6 +337,15 @@ static int small_blocks(int m)
     return b;
 }
 
+using SmallKernel = void (*)(const SmallArgs);
+
+// Points per thread for m points: as few as a full cluster needs.
+static SmallKernel small_kernel(int m)
+{
+    constexpr int per = SM_CLUSTER * SM_THREADS;
+    return m <= per ? k_small_iters<1> : k_small_iters<SM_PPT_MAX>;
+}
+
 static cudaLaunchConfig_t small_config(int blocks, cudaLaunchAttribute (&attr)[2], cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
@@ -356,24 +368,27 @@ static cudaLaunchConfig_t small_config(int blocks, cudaLaunchAttribute (&attr)[2
 // kernels serve.
 bool small_iters_usable()
 {
-    if (cudaFuncSetAttribute(k_small_iters, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_SMEM) == cudaSuccess &&
-        cudaFuncSetAttribute(k_small_iters, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    for (int m : {1, SMALL_MAX_POINTS}) {
+        const SmallKernel k = small_kernel(m);
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = small_config(SM_CLUSTER, attr, nullptr);
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, k_small_iters, &cfg) == cudaSuccess && n >= 1)
-            return true;
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess || n < 1) {
+            cudaGetLastError();
+            return false;
+        }
     }
-    cudaGetLastError();
-    return false;
+    return true;
 }
 
 cudaError_t launch_small_iters(const SmallArgs &a, cudaStream_t st)
 {
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = small_config(small_blocks(a.m), attr, st);
-    return cudaLaunchKernelEx(&cfg, k_small_iters, a);
+    return cudaLaunchKernelEx(&cfg, small_kernel(a.m), a);
 }
 
 }  // namespace vicp
