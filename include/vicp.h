@@ -265,7 +265,7 @@ VICP_API vicp_status vicp_register_host(vicp_ctx *ctx, const float *src_xyzw_hos
 
 /* Synchronous: waits for the stream and fills *out (n_stored is read back).
  * The build itself writes only the offsets its searches read (those of the
- * occupied voxels and the ones just past them, every 32nd, and offsets[V]);
+ * occupied voxels and the ones just past them, and offsets[V]);
  * the first vicp_get_grid or vicp_memory_report after a build completes the
  * array (one kernel on the context's stream), so out->offsets holds all
  * V + 1 entries. */

@@ -59,7 +59,7 @@ struct vicp_ctx {
     const float4 *target = nullptr;   // caller's target of the last build (global search)
 
     // V-sized
-    Buf counts, off, root, ring, desc, tile_sum, inter, uflag, zdirty;
+    Buf counts, off, root, ring, desc, tile_sum, tile_off, inter, uflag, zdirty;
     bool labels_clean = false;   // root/ring "unlabelled" except where zdirty marks labels
     int lab_dims[3] = {0, 0, 0};   // grid dimensions that state belongs to
     Buf occ[2];       // occupancy bits: the current build's, and the next build's (kept zeroed)
@@ -312,6 +312,7 @@ vicp_status ensure_voxel_buffers(vicp_ctx *c, long long V, long long n_bricks)
         TRY(buf_zero(c, c->desc, "zero scan descriptors"));
         TRY(buf_alloc(c, c->tile_sum, (size_t)scan_tiles(V) * 4, "scan tile sums"));
         TRY(buf_zero(c, c->tile_sum, "zero scan tile sums"));   // kept at zero between builds
+        TRY(buf_alloc(c, c->tile_off, (size_t)scan_tiles(V) * 4, "scan tile offsets"));
         c->cap_V = V;
     }
     if (dilate_units(c->geom) * 4 > (long long)c->uflag.bytes) {
@@ -695,7 +696,8 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
         if (sparse)
             return launch_scan(counts, slot_geom(c->cap_o), off, socc, tiles, (unsigned long long *)c->sdesc.p, d,
                                c->stream, false);
-        return launch_scan(counts, g, off, occ, tiles, (unsigned long long *)c->desc.p, d, c->stream, false);
+        return launch_scan(counts, g, off, occ, tiles, (unsigned long long *)c->desc.p, d, c->stream, false, nullptr,
+                           (unsigned *)c->tile_off.p);
     }));
     c->off_dense = false;
     TRY(launch(c, K_BRICK_SCAN, [&] {
@@ -811,7 +813,8 @@ vicp_status dense_offsets(vicp_ctx *c)
         return VICP_OK;
     const GridGeom &g = c->geom;
     TRY(launch(c, K_OFFSETS_FILL, [&] {
-        return launch_offsets_fill((unsigned *)c->off.p, (const unsigned *)c->occ[c->occ_cur].p, g.V, c->stream);
+        return launch_offsets_fill_tiles((unsigned *)c->off.p, (const unsigned *)c->occ[c->occ_cur].p,
+                                         (const unsigned *)c->tile_off.p, g.V, c->stream);
     }));
     c->off_dense = true;
     return VICP_OK;
@@ -1300,7 +1303,7 @@ void vicp_destroy(vicp_ctx *c)
     cudaStreamSynchronize(c->stream);
     if (c->side)
         cudaStreamSynchronize(c->side);
-    Buf *all[] = {&c->counts,  &c->off,      &c->root,       &c->ring,       &c->occ[0],    &c->occ[1], &c->desc, &c->tile_sum,
+    Buf *all[] = {&c->counts,  &c->off,      &c->root,       &c->ring,       &c->occ[0],    &c->occ[1], &c->desc, &c->tile_sum, &c->tile_off,
                   &c->inter,       &c->uflag,      &c->zdirty,
                   &c->bcounts, &c->bsums, &c->boff,     &c->brick_list, &c->brick_range, &c->brick_box, &c->bslot,
                   &c->boxk[0], &c->boxk[1], &c->sb_box,     &c->sb_left,    &c->keys,

@@ -605,7 +605,8 @@ template <int THREADS, int WPT, bool DENSE>
 __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
     k_scan(const unsigned *__restrict__ counts, long long V, unsigned *__restrict__ off,
            const unsigned *__restrict__ occ, const unsigned *__restrict__ tile_sum,
-           unsigned long long *__restrict__ desc, const DevCtl *__restrict__ ctl, unsigned *__restrict__ mismatch)
+           unsigned long long *__restrict__ desc, const DevCtl *__restrict__ ctl, unsigned *__restrict__ mismatch,
+           unsigned *__restrict__ tile_off)
 {
     static_assert(THREADS * WPT * 32 == SCAN_TILE, "tile");
     static_assert(!DENSE || WPT == 1, "the dense output stages one word per thread");
@@ -745,16 +746,27 @@ __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
 
     unsigned run = excl + thread_excl;
     if (!DENSE) {
+        if (tile_off && tid == 0)
+            tile_off[tile] = excl;
         // the entries the build and the searches read, straight from registers
 #pragma unroll
         for (int w = 0; w < WPT; ++w) {
             const long long b = base + 32 * w;
             if (b > V)
                 break;
+            const bool last = b < V && b + 32 >= V;   // the word holding voxel V-1 closes the array
+            if (tile_off && bits[w] == 0u) {
+                if (last)
+                    off[V] = run;
+                continue;
+            }
+            // (an occupied voxel's next entry is the next word's first, which
+            // that word's thread leaves out when it is empty)
+            const bool carry = tile_off && (bits[w] >> 31) && !last;
             if (__popc(bits[w]) > SCAN_DENSE_BITS && b + 32 <= V) {   // every entry of the word
                 run = word_offsets_vec(counts, off, b, run);
-                if (b + 32 == V)
-                    off[V] = run;
+                if (carry || last)
+                    off[b + 32] = run;   // (off[V] itself when b + 32 == V)
                 continue;
             }
             off[b] = run;   // the word's first entry (off[V] itself when b == V)
@@ -766,7 +778,9 @@ __global__ void __launch_bounds__(THREADS, DENSE ? 3 : 1024 / THREADS)
                 if (i < 31 && !((bits[w] >> (i + 1)) & 1u))
                     off[b + i + 1] = run;
             }
-            if (b < V && b + 32 >= V)   // the word holding voxel V-1 closes the array
+            if (carry)
+                off[b + 32] = run;
+            if (last)
                 off[V] = run;
         }
         return;
@@ -854,19 +868,19 @@ cudaError_t launch_clear_counted(unsigned *counts, unsigned *occ, long long word
 
 cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off, const unsigned *occ,
                         const unsigned *tile_sum, unsigned long long *desc, const DevCtl *ctl, cudaStream_t st,
-                        bool dense, unsigned *mismatch)
+                        bool dense, unsigned *mismatch, unsigned *tile_off)
 {
     const long long tiles = scan_tiles(g.V);
     if (!dense)
         return launch_kernel(k_scan<256, 2, false>, dim3((unsigned)tiles), dim3(256), 0, st, counts, g.V, off, occ,
-                             tile_sum, desc, ctl, mismatch);
+                             tile_sum, desc, ctl, mismatch, tile_off);
     constexpr int T = 512;
     const size_t smem = (size_t)T * 33 * sizeof(unsigned);
     cudaError_t e = cudaFuncSetAttribute(k_scan<T, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess)
         return e;
     return launch_kernel(k_scan<T, 1, true>, dim3((unsigned)tiles), dim3(T), smem, st, counts, g.V, off, occ,
-                         tile_sum, desc, ctl, mismatch);
+                         tile_sum, desc, ctl, mismatch, (unsigned *)nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -894,6 +908,62 @@ __global__ void __launch_bounds__(256) k_offsets_fill(unsigned *__restrict__ off
 cudaError_t launch_offsets_fill(unsigned *off, const unsigned *occ, long long V, cudaStream_t st)
 {
     return launch_kernel(k_offsets_fill, dim3((unsigned)((V + 255) / 256)), dim3(256), 0, st, off, occ, V);
+}
+
+// The same for a scan that left out the empty words (a block per scan tile,
+// a thread per word): a word's first offset is the largest of the tile's and
+// the ends of the words before it, and an empty word's entries all have it.
+__global__ void __launch_bounds__(SCAN_TILE / 32) k_offsets_fill_tiles(unsigned *__restrict__ off,
+                                                                       const unsigned *__restrict__ occ,
+                                                                       const unsigned *__restrict__ tile_off,
+                                                                       long long V)
+{
+    pdl_begin();
+    constexpr int WARPS = SCAN_TILE / 32 / 32;
+    __shared__ unsigned s_w[WARPS];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long b = (long long)blockIdx.x * SCAN_TILE + 32ll * tid;
+    const unsigned bits = b < V ? __ldg(occ + (b >> 5)) : 0u;
+    unsigned end = bits ? off[b + 32 - __clz((int)bits)] : 0u;   // past the last occupied voxel: written
+    unsigned incl = end;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned y = __shfl_up_sync(FULL_MASK, incl, d);
+        if (lane >= d)
+            incl = max(incl, y);
+    }
+    if (lane == 31)
+        s_w[warp] = incl;
+    __syncthreads();
+    unsigned first = __ldg(tile_off + blockIdx.x);
+    for (int w = 0; w < warp; ++w)
+        first = max(first, s_w[w]);
+    const unsigned before = __shfl_up_sync(FULL_MASK, incl, 1);
+    if (lane > 0)
+        first = max(first, before);
+    if (b >= V)
+        return;
+    const int n = (int)min(32ll, V - b);
+    if (!bits) {
+        for (int i = 0; i < n; ++i)
+            off[b + i] = first;
+        return;
+    }
+    const unsigned written = 1u | bits | (bits << 1);
+    unsigned cur = 0u;
+    for (int i = 0; i < n; ++i) {
+        if ((written >> i) & 1u)
+            cur = off[b + i];
+        else
+            off[b + i] = cur;
+    }
+}
+
+cudaError_t launch_offsets_fill_tiles(unsigned *off, const unsigned *occ, const unsigned *tile_off, long long V,
+                                      cudaStream_t st)
+{
+    return launch_kernel(k_offsets_fill_tiles, dim3((unsigned)scan_tiles(V)), dim3(SCAN_TILE / 32), 0, st, off, occ,
+                         tile_off, V);
 }
 
 // ---------------------------------------------------------------------------

@@ -89,15 +89,19 @@ cudaError_t launch_histogram(const float4 *pts, int n, const GridGeom &g, int *k
 // off[32 k] and off[V] (what the build and the searches read) -- the rest
 // is completed by launch_offsets_fill on the same occupancy bits.  mismatch
 // (dense; may be null): DEVERR_BOUNDS is set in it when a tile's counts do not
-// add up to its total.  desc may be null up to 4096 tiles.
+// add up to its total.  desc may be null up to 4096 tiles.  tile_off (sparse;
+// may be null): the words without a point are left out, every tile's first
+// offset is written there, and launch_offsets_fill_tiles completes the array.
 cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off, const unsigned *occ,
                         const unsigned *tile_sum, unsigned long long *desc, const DevCtl *ctl, cudaStream_t st,
-                        bool dense, unsigned *mismatch = nullptr);
+                        bool dense, unsigned *mismatch = nullptr, unsigned *tile_off = nullptr);
 // Zeroes the counts of the voxels whose bits are set in occ (words of it, a
 // multiple of four; both arrays 16-byte aligned), those words, the tile totals
 // (n_tiles <= words / 4) and the control block.
 cudaError_t launch_clear_counted(unsigned *counts, unsigned *occ, long long words, unsigned *tile_sum, int n_tiles,
                                  DevCtl *ctl, cudaStream_t st);
+cudaError_t launch_offsets_fill_tiles(unsigned *off, const unsigned *occ, const unsigned *tile_off, long long V,
+                                      cudaStream_t st);
 cudaError_t launch_offsets_fill(unsigned *off, const unsigned *occ, long long V, cudaStream_t st);
 // sums: brick_tiles(slots) words of scratch (used by large grids).
 constexpr int BM_MAX_BRICKS = 65536;   // up to this many slots one launch, past it two
