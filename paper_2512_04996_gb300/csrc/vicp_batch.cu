@@ -1135,10 +1135,11 @@ static size_t iter_smem(int threads) { return (size_t)(threads / 32) * sizeof(Wa
 
 int batch_tile_points(int shape, int blocks, long long m)
 {
-    const long long warps = (long long)blocks * (BATCH_SHAPES[shape].threads / 32);
-    const long long most = std::min(64 * BATCH_SHAPES[shape].ppt, BATCH_TILE_MAX);
-    const long long rounds = (m + 64 * warps - 1) / std::max(64 * warps, 1ll);   // two tiles a warp where the batch is small
-    return (int)std::min(std::max(32 * rounds, 32ll), most);
+    // whole rounds of all warps: k tiles a warp, of as few points as k needs
+    const long long lanes = std::max((long long)blocks * BATCH_SHAPES[shape].threads, 32ll);
+    const long long most = std::min(2 * BATCH_SHAPES[shape].ppt, BATCH_TILE_MAX / 32);   // points a lane
+    const long long k = std::max((m + lanes * most - 1) / (lanes * most), 1ll);
+    return (int)(32 * std::min(std::max((m + lanes * k - 1) / (lanes * k), 1ll), most));
 }
 
 int batch_iter_blocks(int shape, BatchMode mode)

@@ -205,7 +205,7 @@ struct FallbackArgs {
 cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st);
 // Iterations of a small source cloud on the dense grid by one cluster
 // (vicp_small.cu): searches, sums (double-float), solve, stopping test.
-constexpr int SMALL_MAX_POINTS = 16384;
+constexpr int SMALL_MAX_POINTS = 24576;
 bool small_iters_usable();   // whether the current device takes the cluster (asked once per context)
 struct SmallArgs {
     const float4 *src;

@@ -20,12 +20,12 @@
 //       same bits, and block 0 writes the results.
 // Measured (30 iterations, grid kept, against the separate kernels): 4,096
 // points 384-459 us against 709-753, 16,384 points 479-618 against 725-839
-// (objects, by their share of global queries); one step of 1,000 points 17.8
-// against 22.5.  What bounds it now is the chain of an iteration: root,
-// offset, points, the lists' rows, and the solve.  Past 16,384 points 16
-// SMs are too few for clouds with many global queries and the separate kernels
-// serve (three points a thread, 24,576 points: 565-914 us against 775-1,025;
-// five, 40,960: an object 762 against 821, but a scene 1,497 against 952).
+// (objects, by their share of global queries), 24,576 points (three a thread)
+// 565-914 against 775-1,025; one step of 1,000 points 17.0 against 22.5.
+// What bounds it now is the chain of an iteration: root, offset, points, the
+// lists' rows, and the solve.  Past 24,576 points 16 SMs are too few for
+// clouds with many global queries (40,960 points: an object 762 against 821,
+// but a scene 1,497 against 952) and the separate kernels serve.
 // The sums are bit-reproducible from run to run.  The slots of two
 // iterations alternate: a block overwrites a slot only after the barrier
 // that every reader of it has passed.
@@ -343,7 +343,7 @@ using SmallKernel = void (*)(const SmallArgs);
 static SmallKernel small_kernel(int m)
 {
     constexpr int per = SM_CLUSTER * SM_THREADS;
-    return m <= per ? k_small_iters<1> : k_small_iters<SM_PPT_MAX>;
+    return m <= per ? k_small_iters<1> : (m <= 2 * per ? k_small_iters<2> : k_small_iters<SM_PPT_MAX>);
 }
 
 static cudaLaunchConfig_t small_config(int blocks, cudaLaunchAttribute (&attr)[2], cudaStream_t st)
@@ -368,7 +368,7 @@ static cudaLaunchConfig_t small_config(int blocks, cudaLaunchAttribute (&attr)[2
 // kernels serve.
 bool small_iters_usable()
 {
-    for (int m : {1, SMALL_MAX_POINTS}) {
+    for (int m : {1, 2 * SM_CLUSTER * SM_THREADS, SMALL_MAX_POINTS}) {
         const SmallKernel k = small_kernel(m);
         cudaLaunchAttribute attr[2];
         cudaLaunchConfig_t cfg = small_config(SM_CLUSTER, attr, nullptr);

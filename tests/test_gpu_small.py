@@ -1,4 +1,4 @@
-"""ICP iterations of a small source cloud by one thread-block cluster (up to 16384 points) against the separate kernels,
+"""ICP iterations of a small source cloud by one thread-block cluster (up to 24576 points) against the separate kernels,
 which a context with kernel timing enabled runs, and against the oracle.  Same matches, so the sums differ only by
 their order: poses within 1e-12 (double-float sums carry about 2^-46), the same iteration counts and statuses."""
 import numpy as np
@@ -23,7 +23,8 @@ def _close(a, b, tol=1e-12):
     return float(np.abs(np.asarray(a) - np.asarray(b)).max()) <= tol
 
 
-@pytest.mark.parametrize("m", [1, 2, 3, 31, 32, 33, 127, 128, 129, 255, 257, 1000, 2047, 2049, 8191, 16383, 16384, 16385])
+@pytest.mark.parametrize("m", [1, 2, 3, 31, 32, 33, 127, 128, 129, 255, 257, 1000, 2047, 2049, 8191, 8193, 16384, 16385, 24575, 24576,
+                               24577])
 def test_step_and_registration_equal_the_separate_kernels(m):
     p, s, t, src = _pair(m)
     out = []
