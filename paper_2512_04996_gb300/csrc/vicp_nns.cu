@@ -17,10 +17,22 @@ namespace vicp {
 // for it.  Both lists get one global atomic per block.
 // ---------------------------------------------------------------------------
 constexpr int CORR_THREADS = 512;
-// Up to this many source points the global queries are so few that each has
-// a warp of its own, and the brick search (with the seed) is as short a chain
-// (one step of 1,000 points on a 4k object 24.2 to 24.6 us either way).
-constexpr int NEAR_MIN_QUERIES = 16384;
+// Whether a search of m points on grid g takes its near queries by rows of
+// voxels (NEAR below).  Up to 16,384 points the global queries are so few that
+// each has a warp of its own, and the brick search is as short a chain; and
+// where a grid has many voxels for a query, few queries crowd round the same
+// faces, and what the rows save does not pay for the longer code of both
+// kernels, which is fetched cold in every iteration (the reduction's after it,
+// too).  One search and update, grid kept, without / with: sphere and plane of
+// 60,000 points (V = 17 m) 57.1 / 34.0 us, of 34,457 (V = m, 20 iterations)
+// 1,381 / 984; an object of 40,000 (V = 50 m) 27.0 / 26.1; scenes (V = 48 m to
+// 103 m) of 30,982 points 29.2 / 31.1, 60,000 31.2 / 33.5, 120,000 47.6 / 49.2.
+constexpr int NEAR_MIN_QUERIES = 16384, NEAR_MAX_VOXELS = 32;
+
+static bool near_by_rows(int m, const GridGeom &g)
+{
+    return m > NEAR_MIN_QUERIES && g.V <= (long long)NEAR_MAX_VOXELS * m;
+}
 
 // Segment of a root voxel in the CSR store: [off[r], off[r + 1]) (clamped to
 // the store's length).
@@ -82,7 +94,7 @@ struct HashedRoot {
     }
 };
 
-template <class Seg, class Root>
+template <bool NEAR, class Seg, class Root>
 __global__ void __launch_bounds__(CORR_THREADS) k_correspond(const float4 *__restrict__ src, int m,
                                                              const double *__restrict__ pose, GridGeom g,
                                                              Root root, Seg seg,
@@ -101,7 +113,7 @@ __global__ void __launch_bounds__(CORR_THREADS) k_correspond(const float4 *__res
     if (threadIdx.x == 32) {   // (not the warp that loads the pose: the round trips overlap)
         s_cand = 0ull;
         s_fb = s_nr = s_hv = 0;
-        s_no = __ldcg(&ctl->n_outside);
+        s_no = NEAR ? __ldcg(&ctl->n_outside) : 0;
     }
     load_pose_f_block(pose, sp);   // also orders the initialisation above
     const PoseF P = sp;
@@ -111,8 +123,8 @@ __global__ void __launch_bounds__(CORR_THREADS) k_correspond(const float4 *__res
     unsigned cand = 0u, a = 0u, b = 0u;
     if (i < m) {
         const float3 s = transform_pt(P, __ldg(src + i));
-        bool inside;
-        const int v = nearest_voxel(g, s, inside);
+        bool inside = true;
+        const int v = NEAR ? nearest_voxel(g, s, inside) : voxel_key(g, s.x, s.y, s.z);
         const int r = v >= 0 ? root(v) : -1;
         far = true;
         unsigned dense = 0u;
@@ -125,11 +137,11 @@ __global__ void __launch_bounds__(CORR_THREADS) k_correspond(const float4 *__res
             heavy = cand > HEAVY;
             far = !inside;
         }
-        if (!heavy) {   // (far without a label: an empty run, no seed)
+        if (NEAR ? !heavy : !heavy && !far) {   // (far without a label: an empty run, no seed)
             const unsigned long long best = segment_min(csr, a, b, s);
             nn[i] = (int)(unsigned)best;
             d2[i] = __uint_as_float((unsigned)(best >> 32));
-            near = far && dense && m > NEAR_MIN_QUERIES && s_no <= NEAR_OUTSIDE_MAX &&
+            near = NEAR && far && dense && s_no <= NEAR_OUTSIDE_MAX &&
                    near_seed(s, __uint_as_float((unsigned)(best >> 32)), g.inv_h, dense);
             far = far && !near;
         }
@@ -203,7 +215,7 @@ cudaError_t launch_correspond(const float4 *src, int m, const double *pose, cons
                               int *fb_list, int *hv_list, uint2 *hv_range, DevCtl *ctl, int honor_stop,
                               cudaStream_t st)
 {
-    return launch_kernel(k_correspond<CsrSeg, DenseRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
+    return launch_kernel(near_by_rows(m, g) ? k_correspond<true, CsrSeg, DenseRoot> : k_correspond<false, CsrSeg, DenseRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
                          dim3(CORR_THREADS), 0, st, src, m, pose, g, DenseRoot{root}, CsrSeg{off, (unsigned)n_cap},
                          csr, nn, d2, fb_list, hv_list, hv_range, ctl, honor_stop);
 }
@@ -216,7 +228,7 @@ cudaError_t launch_correspond_hashed(const float4 *src, int m, const double *pos
 {
     const HashedRoot root{labelled.keys, labelled.mask, labelled.shift, lseg, lroot,
                           occupied.keys, occupied.mask, occupied.shift, g.nx, (g.nx + 31) / 32};
-    return launch_kernel(k_correspond<CsrSeg, HashedRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
+    return launch_kernel(near_by_rows(m, g) ? k_correspond<true, CsrSeg, HashedRoot> : k_correspond<false, CsrSeg, HashedRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
                          dim3(CORR_THREADS), 0, st, src, m, pose, g, root, CsrSeg{off, (unsigned)n_cap}, csr, nn, d2,
                          fb_list, hv_list, hv_range, ctl, honor_stop);
 }
@@ -225,7 +237,7 @@ cudaError_t launch_correspond_fixed(const float4 *src, int m, const double *pose
                                     const unsigned *count, unsigned C, const float4 *slots, int *nn, float *d2,
                                     int *fb_list, int *hv_list, uint2 *hv_range, DevCtl *ctl, cudaStream_t st)
 {
-    return launch_kernel(k_correspond<FixedSeg, DenseRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
+    return launch_kernel(near_by_rows(m, g) ? k_correspond<true, FixedSeg, DenseRoot> : k_correspond<false, FixedSeg, DenseRoot>, dim3((m + CORR_THREADS - 1) / CORR_THREADS),
                          dim3(CORR_THREADS), 0, st, src, m, pose, g, DenseRoot{root}, FixedSeg{count, C}, slots, nn,
                          d2, fb_list, hv_list, hv_range, ctl, 0);
 }
@@ -258,7 +270,7 @@ __device__ __forceinline__ int strided_share(int n, int b, int B)
     return n <= b ? 0 : (n - b <= B ? 1 : (n - 1 - b) / B + 1);
 }
 
-template <class Rows>
+template <bool NEAR, class Rows>
 __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__restrict__ src,
                                                          const double *__restrict__ pose, GridGeom g, Rows rows,
                                                          const float4 *__restrict__ bpts,
@@ -293,7 +305,7 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
     load_pose_f_block(pose, sp);   // also orders the initialisation above
     const PoseF P = sp;
     const int lane = threadIdx.x & 31;
-    const int F = min(s_n[0], m), N = min(s_n[1], m - F), Hv = min(s_n[2], m), ns = s_n[3], no = s_n[4];
+    const int F = min(s_n[0], m), N = NEAR ? min(s_n[1], m - F) : 0, Hv = min(s_n[2], m), ns = s_n[3], no = s_n[4];
     const int B = (int)gridDim.x, b = (int)blockIdx.x;
     // lanes a near query and a dense segment get (2^...), and how many of
     // them a warp takes at a time (2^...)
@@ -320,13 +332,14 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
             }
             const float3 s = transform_pt(P, __ldg(src + i));
             const unsigned long long best = global_search(s, bpts, bbox, sb_box, ns, tgt, n_tgt, outside, no, lane,
-                                                          examined, nn_key(d2[i], nn[i]));
-            __syncwarp();   // every lane has read the seed
+                                                          examined, NEAR ? nn_key(d2[i], nn[i]) : ~0ull);
+            if (NEAR)
+                __syncwarp();   // every lane has read the seed
             if (lane == 0) {
                 nn[i] = (int)(unsigned)best;
                 d2[i] = __uint_as_float((unsigned)(best >> 32));
             }
-        } else if (k < nG + nN) {   // near queries
+        } else if (NEAR && k < nG + nN) {   // near queries
             const int G = 1 << gN, q = ((b + (k - nG) * B) << packN) + (lane >> gN), sub = lane & (G - 1);
             const int i = q < N ? __ldg(fb_list + m - 1 - q) : -1;
             const bool on = (unsigned)i < (unsigned)m;
@@ -392,13 +405,13 @@ __global__ void __launch_bounds__(FB_THREADS, 4) k_fallback(const float4 *__rest
     }
 }
 
-template <class Rows>
+template <bool NEAR, class Rows>
 static cudaError_t run_fallback(const FallbackArgs &a, const Rows &rows, cudaStream_t st)
 {
     // as many warps as can be resident, and no more than there are queries
     static int per_sm = 0;
     if (per_sm == 0) {
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fallback<Rows>, FB_THREADS, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fallback<NEAR, Rows>, FB_THREADS, 0);
         if (e != cudaSuccess || per_sm < 1)
             per_sm = 1;
     }
@@ -406,17 +419,19 @@ static cudaError_t run_fallback(const FallbackArgs &a, const Rows &rows, cudaStr
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int blocks = min(sms * per_sm, (a.m + FB_THREADS / 32 - 1) / (FB_THREADS / 32));
-    return launch_kernel(k_fallback<Rows>, dim3(blocks), dim3(FB_THREADS), 0, st, a.src, a.pose, a.g, rows, a.bpts,
+    return launch_kernel(k_fallback<NEAR, Rows>, dim3(blocks), dim3(FB_THREADS), 0, st, a.src, a.pose, a.g, rows, a.bpts,
                          a.bbox, a.sb_box, a.tgt, a.n_tgt, a.outside, a.fb_list, a.hv_list, a.hv_range, a.hv_store,
                          a.ctl, a.nn, a.d2, a.m, a.honor_stop, a.n_global_out);
 }
 
 cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st)
 {
+    if (!near_by_rows(a.m, a.g))   // no rows read
+        return run_fallback<false>(a, CsrRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr}, st);
     if (a.okeys.keys)
-        return run_fallback(a, HashedRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr, a.okeys.keys, a.okeys.mask,
+        return run_fallback<true>(a, HashedRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr, a.okeys.keys, a.okeys.mask,
                                           a.okeys.shift}, st);
-    return run_fallback(a, CsrRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr}, st);
+    return run_fallback<true>(a, CsrRows{a.occ, a.off, (unsigned)a.n_tgt, a.csr}, st);
 }
 
 }  // namespace vicp

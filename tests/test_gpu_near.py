@@ -1,7 +1,7 @@
 """The near form of the global search (points just outside the grid, answered from the voxel rows round them) against
 the oracle: same neighbours, same squared distances and the same number of global searches, on the dense and the
 sparse grid, at every face, edge and corner, from touching distances to where the brick search takes over.  (The near
-form serves searches of more than 16384 points.)"""
+form serves searches of more than 16,384 points with at most 32 voxels of grid for each.)"""
 import numpy as np
 import pytest
 import torch
@@ -103,4 +103,19 @@ def test_grids_far_from_the_origin(offset):
     target = _cloud(rng, 2000, o, hi)
     ctx, g = gpu_grid(target, L=6, voxel_size=h, origin=tuple(float(x) for x in o), dims=dims)
     src = np.concatenate([_round_the_box(rng, o, hi, 3 * h, 17000), _cloud(rng, 200, o, hi)])
+    _check(ctx, target, 6, src, oracle_grid_for(g, target, 6))
+
+
+@pytest.mark.parametrize("nz", [80, 81])
+@pytest.mark.parametrize("n", [16384, 16385, 17000])
+def test_where_the_rows_begin(n, nz):
+    """32 voxels a query (80 x 85 x 80 for 17,000) and 16,384 queries: either side of both lines."""
+    rng = np.random.default_rng(n + nz)
+    h, o, dims = 0.05, np.array([0.1, -0.2, 0.3], np.float32), (80, 85, nz) if n == 17000 else (20, 24, nz)
+    hi = o + h * np.asarray(dims)
+    target = _cloud(rng, 4000, o, hi)
+    src = np.concatenate([_round_the_box(rng, o, hi, 2 * h, n - 1000), _cloud(rng, 500, o, hi),
+                          _round_the_box(rng, o - 20 * h, hi + 20 * h, h, 500)])
+    rng.shuffle(src)
+    ctx, g = gpu_grid(target, L=6, voxel_size=h, origin=tuple(float(x) for x in o), dims=dims)
     _check(ctx, target, 6, src, oracle_grid_for(g, target, 6))
