@@ -407,7 +407,7 @@ VICP_API vicp_status vicp_fixed_view(vicp_ctx *ctx, const float **slots_out, con
  * needed.
  *
  * Working memory is one static device array inside the library (about
- * 70 MiB on every GPU the library is loaded on, held until the process
+ * 66 MiB on every GPU the library is loaded on, held until the process
  * exits); the grid is therefore limited to VICP_STATIC_MAX_VOXELS voxels and
  * VICP_STATIC_MAX_BRICK_SLOTS 8^3-voxel brick slots (bricks padded to whole
  * 4x4x4-brick groups per axis); larger grids return VICP_ERR_GRID_TOO_LARGE.
