@@ -155,9 +155,10 @@ long long dilate_units(const GridGeom &g);
 long long dilate_column_units(const GridGeom &g);
 // The localised search lists queries whose root segment is long (with the
 // segment) in hv_list / hv_range, and queries without a root in fb_list: far
-// ones from its front, near ones (vicp_search.cuh) from its back, each with
-// a known point's key or all ones as the seed in its nn / d2 entries.  The
-// fallback kernel then answers the lists.
+// ones from its front and, where they are searched by rows of voxels
+// (near_by_rows), near ones from its back, each then with a known point's key
+// or all ones as the seed in its nn / d2 entries.  The fallback kernel, which
+// must be launched for the same m and g, answers the lists.
 cudaError_t launch_correspond(const float4 *src, int m, const double *pose, const GridGeom &g, const int *root,
                               const unsigned *off, const float4 *csr, int n_cap, int *nn, float *d2,
                               int *fb_list, int *hv_list, uint2 *hv_range, DevCtl *ctl, int honor_stop,

@@ -12,9 +12,9 @@ namespace vicp {
 // of (x, y, z, index), eight in flight.  A few dense voxels hold far more
 // points than the rest, and a warp waits for its longest segment: a query
 // whose segment has more than HEAVY points is not scanned here but listed,
-// with its segment, for the next kernel, whose warps take such segments one
-// at a time with all lanes.  Points that need the global search are listed
-// for it.  Both lists get one global atomic per block.
+// with its segment, for the next kernel, which gives each 4 to 32 lanes.
+// Points that need the global search are listed for it.  Every list gets one
+// global atomic per block.
 // ---------------------------------------------------------------------------
 constexpr int CORR_THREADS = 512;
 // Whether a search of m points on grid g takes its near queries by rows of
