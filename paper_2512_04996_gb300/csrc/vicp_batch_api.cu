@@ -111,9 +111,22 @@ vicp_status bcuda(vicp_batch *b, cudaError_t e, const char *what)
             return bcuda((b), _e, (what));   \
     } while (0)
 
+void drop_graph(vicp_batch *b)
+{
+    if (b->graph)
+        cudaGraphExecDestroy(b->graph);
+    b->graph = nullptr;
+    b->g_shape = b->g_iters = b->g_M = b->g_items = -1;
+    b->g_src = nullptr;
+}
+
+// Gives a buffer up, and with it the captured iterations, which hold the
+// buffers' addresses (a search of a larger source cloud, the loss and the
+// autotuner grow the same workspace as a registration).
 void bfree(vicp_batch *b, BBuf &x)
 {
     if (x.p) {
+        drop_graph(b);
         if (b->custom_alloc)
             b->alloc.free(x.p, x.bytes, (void *)b->stream, b->alloc.user);
         else
@@ -161,15 +174,6 @@ vicp_status bensure(vicp_batch *b, BBuf &x, size_t bytes, const char *what, bool
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 DevCtl *bctl(vicp_batch *b) { return static_cast<DevCtl *>(b->ctl.p); }
-
-void drop_graph(vicp_batch *b)
-{
-    if (b->graph)
-        cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-    b->g_shape = b->g_iters = b->g_M = b->g_items = -1;
-    b->g_src = nullptr;
-}
 
 vicp_status check_counts(vicp_batch *b, const int32_t *n, int P, const char *what, long long *total)
 {
