@@ -161,9 +161,15 @@ vicp_status cuda_fail(vicp_ctx *c, cudaError_t e, const char *what)
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // --- allocation ------------------------------------------------------------
+// Gives a buffer up, and with it the captured registration, which holds the
+// buffers' addresses (searches, builds and registrations of larger clouds
+// grow the same workspace).
 vicp_status buf_free(vicp_ctx *c, Buf &b)
 {
     if (b.p) {
+        if (c->rg_exec)
+            cudaGraphExecDestroy(c->rg_exec);
+        c->rg_exec = nullptr;
         if (c->custom_alloc)
             c->alloc.free(b.p, b.bytes, (void *)c->stream, c->alloc.user);
         else

@@ -47,3 +47,35 @@ def test_batch_registration_after_the_workspace_grew(between):
     assert all(np.array_equal(x, y) for x, y in zip(again[1:], ref[1:]))
     if shape < 0:
         assert all(np.array_equal(x, y) for x, y in zip(again[1:], first[1:]))
+
+
+@pytest.mark.parametrize("between", ["register_host", "correspond", "build"])
+def test_registration_after_the_workspace_grew(between):
+    v = vicp()
+    small, large = synth.sphere_plane(seed=73, n=30000), synth.sphere_plane(seed=74, n=90000)
+    kw = dict(grid_divisions=64, dilation_layers=10, max_iters=5, rmse_eps=0.0)
+    ctx = v.Context(flags=v.VICP_FLAG_KEEP_GRID, **kw)
+    plain = v.Context(flags=v.VICP_FLAG_KEEP_GRID | v.VICP_FLAG_NO_GRAPH, **kw)
+    host = between == "register_host"
+
+    def cloud(a):
+        t = torch.from_numpy(a)
+        return t.pin_memory() if host else t.cuda()
+
+    s, t, s2, t2 = (cloud(a) for a in (small.source, small.target, large.source, large.target))
+
+    def run(c):
+        return c.register_host(s.numpy(), t.numpy()) if host else c.register(s, t)
+
+    first = [run(ctx) for _ in range(3)]
+    assert ctx.graph_replayed() == 1
+    if host:
+        assert ctx.register_host(s2.numpy(), t2.numpy())[0] == 0
+    elif between == "correspond":
+        ctx.correspond(s2, torch.eye(4, dtype=torch.float64, device="cuda"))
+    else:
+        ctx.build_grid(t2)
+    again = [run(ctx) for _ in range(3)]
+    ref = run(plain)
+    for r in first + again:
+        assert r[0] == ref[0] == 0 and r[2:] == ref[2:] and np.array_equal(r[1], ref[1])
