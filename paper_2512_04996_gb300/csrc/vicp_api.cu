@@ -65,6 +65,8 @@ struct vicp_ctx {
     Buf occ[2];       // occupancy bits: the current build's, and the next build's (kept zeroed)
     int occ_cur = 0;
     bool after_solve = false;   // the last kernel launched on `stream` is the reduction + solve
+    int64_t grid_steps = 0;     // iterations on the present grid
+    bool step_loop = false;     // the grid before this one was built for a single iteration
     bool off_dense = false;   // the build writes sparse offsets; vicp_get_grid completes them
     long long cap_V = -1;
     // brick level (V / 512)
@@ -591,13 +593,27 @@ vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, i
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
 }
 
-// Whether m source points take the one-cluster iterations (vicp_small.cu):
-// few enough, the dense grid, double-float sums.  (Kernel timing keeps the
-// separate kernels, which it names.)
+// Whether the update of m source points is summed in the order of the
+// one-cluster iterations (vicp_small.cu): few enough, double-float sums.
+// The searches may then run in the cluster too or as separate kernels: the
+// result is the same, bit for bit.
+bool small_sums(const vicp_ctx *c, int m)
+{
+    return c->small_ok && m <= SMALL_MAX_POINTS && !(c->params.flags & VICP_FLAG_FP64_SOLVE);
+}
+
+// Whether `iters` iterations of m source points on the present grid run in
+// the cluster altogether.  Not on the sparse grid, nor with kernel timing on
+// (it names the separate kernels).  And not where the grid is built anew for
+// every iteration: the next build's histogram starts beside the reduction of
+// the separate kernels (after_solve), but not beside a cluster that still
+// searches.  Build, dilation and step in a loop, cluster / separate kernels:
+// sphere and plane of 1,000 points 49.2 / 45.2 us, 4,096 51.3 / 43.5, 24,576
+// 65.3 / 51.3; objects 60.7 / 55.0, 64.9 / 54.3, 73.6 / 60.9.  A kept grid:
+// the figures in vicp_small.cu.
 bool takes_small(const vicp_ctx *c, int m)
 {
-    return c->small_ok && m <= SMALL_MAX_POINTS && !sparse_of(c) && !(c->params.flags & VICP_FLAG_FP64_SOLVE) &&
-           !c->profiling;
+    return small_sums(c, m) && !sparse_of(c) && !c->profiling && !(c->step_loop && c->grid_steps == 0);
 }
 
 vicp_status run_small(vicp_ctx *c, const float4 *src, int m, double *pose, double *rmse, int iters, int honor_stop)
@@ -624,6 +640,7 @@ vicp_status run_small(vicp_ctx *c, const float4 *src, int m, double *pose, doubl
     a.rmse_out = rmse;
     a.ctl = ctl_of(c);
     TRY(launch(c, K_SMALL_ITERS, [&] { return launch_small_iters(a, c->stream); }));
+    c->grid_steps += iters;
     cudaError_t e = cudaEventRecord(c->ev_nns, c->stream);   // a later dilation waits for these searches
     c->nns_in_capture = c->capturing;
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
@@ -633,6 +650,7 @@ vicp_status run_step(vicp_ctx *c, const float4 *src, int m, double *pose, double
 {
     if (takes_small(c, m))
         return run_small(c, src, m, pose, rmse, 1, honor_stop);
+    c->grid_steps += 1;
     TRY(ensure_query_buffers(c, m));
     int *nn = (int *)c->nn.p;
     TRY(run_nns(c, src, m, pose, nn, (float *)c->d2.p, honor_stop));
@@ -647,7 +665,7 @@ vicp_status run_step(vicp_ctx *c, const float4 *src, int m, double *pose, double
     }
     TRY(launch(c, K_REDUCE_SOLVE, [&] {
         return launch_reduce_solve(src, m, pose, c->target, c->n_target, nn, ctr, (float2 *)c->partials.p, nparts,
-                                   rmse, ctl_of(c), honor_stop, c->params.rmse_eps, c->stream);
+                                   rmse, ctl_of(c), honor_stop, c->params.rmse_eps, small_sums(c, m), c->stream);
     }));
     return VICP_OK;
 }
@@ -727,6 +745,8 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
     }));
     c->built = true;
     c->dilated_L = -1;
+    c->step_loop = c->grid_steps == 1;
+    c->grid_steps = 0;
     c->n_target = n;
     c->target = tgt;
     return VICP_OK;
@@ -921,7 +941,8 @@ vicp_status registration_work(vicp_ctx *c, const float4 *src, int32_t m, const f
     e = cudaStreamWaitEvent(c->stream, c->ev_src, 0);
     if (e != cudaSuccess)
         return cuda_fail(c, e, "stream wait");
-    const bool rebuild = (c->params.flags & VICP_FLAG_REBUILD_EACH_ITER) != 0;
+    const bool rebuild = (c->params.flags & VICP_FLAG_REBUILD_EACH_ITER) != 0 && c->params.max_iters > 1;
+    c->step_loop = rebuild;
     const bool one = !rebuild && c->params.max_iters > 0 && takes_small(c, m);   // all iterations in one launch
     if (one)
         TRY(run_small(c, src, m, pose, nullptr, c->params.max_iters, 1));

@@ -206,7 +206,19 @@ struct FallbackArgs {
 cudaError_t launch_fallback(const FallbackArgs &a, cudaStream_t st);
 // Iterations of a small source cloud on the dense grid by one cluster
 // (vicp_small.cu): searches, sums (double-float), solve, stopping test.
+// Block b of the cluster's B takes the tiles b, b + B, ... of 32 points, its
+// warp w the tiles w, w + 16, ... of those.
 constexpr int SMALL_MAX_POINTS = 24576;
+constexpr int SMALL_THREADS = 512, SMALL_CLUSTER = 16;
+// Blocks of the cluster for m points: few points a block, so that its warps
+// are free for the global queries among them.
+inline int small_blocks(int m)
+{
+    int b = 2;
+    while (b < SMALL_CLUSTER && b * 128 < m)
+        b *= 2;
+    return b;
+}
 bool small_iters_usable();   // whether the current device takes the cluster (asked once per context)
 struct SmallArgs {
     const float4 *src;
@@ -232,9 +244,11 @@ cudaError_t launch_small_iters(const SmallArgs &a, cudaStream_t st);
 // 1 per-block shared-memory hash; adds to counts.
 cudaError_t launch_voxel_histogram(const float4 *pts, int n, const GridGeom &g, int method, int *keys,
                                    unsigned *counts, cudaStream_t st);
+// small: the sums in the order of the one-cluster iterations (m at most
+// SMALL_MAX_POINTS; nparts is not used).
 cudaError_t launch_reduce_solve(const float4 *src, int m, double *pose, const float4 *tgt, int n_tgt, const int *nn,
                                 float3 center, float2 *partials, int nparts, double *rmse_out, DevCtl *ctl,
-                                int honor_stop, double eps, cudaStream_t st);
+                                int honor_stop, double eps, bool small, cudaStream_t st);
 // The same update with FP64 sums and an FP64 solve (vicp_solve64.cu);
 // partials holds nparts x 16 doubles.
 cudaError_t launch_reduce_solve_f64(const float4 *src, int m, double *pose, const float4 *tgt, int n_tgt,

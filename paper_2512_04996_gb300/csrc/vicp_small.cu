@@ -26,7 +26,9 @@
 // lists' rows, and the solve.  Past 24,576 points 16 SMs are too few for
 // clouds with many global queries (40,960 points: an object 762 against 821,
 // but a scene 1,497 against 952) and the separate kernels serve.
-// The sums are bit-reproducible from run to run.  The slots of two
+// The sums are bit-reproducible from run to run, and k_reduce_solve adds those
+// of a small cloud in the same order, so that an iteration by the separate
+// kernels gives the same bits.  The slots of two
 // iterations alternate: a block overwrites a slot only after the barrier
 // that every reader of it has passed.
 #include "vicp_df.cuh"
@@ -35,8 +37,8 @@
 
 namespace vicp {
 
-constexpr int SM_THREADS = 512, SM_WARPS = SM_THREADS / 32;
-constexpr int SM_CLUSTER = 16;
+constexpr int SM_THREADS = SMALL_THREADS, SM_WARPS = SM_THREADS / 32;
+constexpr int SM_CLUSTER = SMALL_CLUSTER;
 constexpr int SM_PPT_MAX = SMALL_MAX_POINTS / (SM_CLUSTER * SM_THREADS);   // points per thread, at most
 static_assert(SM_PPT_MAX * SM_CLUSTER * SM_THREADS == SMALL_MAX_POINTS, "points per thread");
 constexpr size_t SM_SMEM = (size_t)2 * SM_WARPS * N_SUMS * 33 * sizeof(float);   // transposed per-lane sums
@@ -325,16 +327,6 @@ __global__ void __launch_bounds__(SM_THREADS, 1) k_small_iters(const SmallArgs a
         if (st_far)
             atomicAdd(&a.ctl->stat_fallbacks, st_far);
     }
-}
-
-// Blocks of the cluster for m points: few points a block, so that its warps
-// are free for the global queries among them.
-static int small_blocks(int m)
-{
-    int b = 2;
-    while (b < SM_CLUSTER && b * 128 < m)
-        b *= 2;
-    return b;
 }
 
 using SmallKernel = void (*)(const SmallArgs);

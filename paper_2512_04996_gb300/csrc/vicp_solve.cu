@@ -9,6 +9,39 @@ namespace vicp {
 constexpr int RED_THREADS = 256;
 static_assert(N_SUMS == REDUCE_VALUES, "sum layout");
 
+// One warp solves (a matrix entry per lane), composes the update with the
+// pose, and writes the RMSE and the registration's loop state.
+__device__ __forceinline__ void finish_update(const dfl *s_tot, int m, float3 cf, double *pose, double *rmse_out,
+                                              DevCtl *ctl, int honor_stop, double eps)
+{
+    const int lane = threadIdx.x & 31;
+    double rmse;
+    const bool ok = solve_update(s_tot, m, cf, pose, rmse);
+    if (lane == 0) {
+        ctl->red_done = 0u;
+        if (rmse_out)
+            *rmse_out = rmse;
+    }
+    if (!ok) {
+        if (lane == 0) {
+            atomicOr(&ctl->err, DEVERR_DEGENERATE);
+            if (honor_stop) {
+                ctl->stop = 1;
+                ctl->last_rmse = rmse;
+            }
+        }
+        return;
+    }
+    if (lane == 0 && honor_stop) {
+        const int it = ctl->iters;
+        ctl->iters = it + 1;
+        ctl->last_rmse = rmse;
+        if (eps > 0.0 && it >= 1 && fabs(rmse - ctl->prev_rmse) < eps)
+            ctl->stop = 1;
+        ctl->prev_rmse = rmse;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Reduction and solve in one launch.  Relative to a fixed centre c (the grid
 // centre rounded to float; s - c is then exact as a double-float), every
@@ -21,7 +54,12 @@ static_assert(N_SUMS == REDUCE_VALUES, "sum layout");
 // solves Eq. 1 (a matrix entry per lane) and composes the update with the
 // pose in FP64, so the result is bit-identical from run to run whichever
 // block finishes last.
+//
+// SMALL adds the sums of a small cloud in the order of the one-cluster
+// iterations (vicp_small.cu), whose results it then equals bit for bit: two
+// blocks here are a block of the cluster, half of its warps each.
 // ---------------------------------------------------------------------------
+template <bool SMALL>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_solve(const float4 *__restrict__ src, int m,
                                                               double *__restrict__ pose,
                                                               const float4 *__restrict__ tgt, int n_tgt,
@@ -43,8 +81,13 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_solve(const float4 *__re
     for (int k = 0; k < REDUCE_VALUES; ++k)
         acc[k] = {0.0f, 0.0f};
     // this thread's points, four per round with all their loads issued first
-    const int stride = gridDim.x * RED_THREADS;
-    for (int i0 = blockIdx.x * RED_THREADS + threadIdx.x; i0 < m; i0 += 4 * stride) {
+    static_assert(!SMALL || SMALL_THREADS == 2 * RED_THREADS, "half a block of the cluster");
+    const int blocks = gridDim.x / 2;   // SMALL: of the cluster
+    const int first =
+        SMALL ? ((((blockIdx.x & 1) * RED_THREADS + threadIdx.x) >> 5) * blocks + (blockIdx.x >> 1)) * 32 + (threadIdx.x & 31)
+              : blockIdx.x * RED_THREADS + threadIdx.x;
+    const int stride = gridDim.x * RED_THREADS;   // (SMALL: as many points as the cluster has threads)
+    for (int i0 = first; i0 < m; i0 += 4 * stride) {
         int j[4];
         float4 p[4], q[4];
 #pragma unroll
@@ -131,6 +174,34 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_solve(const float4 *__re
         return;
     __threadfence();
 
+    if constexpr (SMALL) {   // the cluster's blocks in order, half of them by each half of the warp
+        if (warp != 0)
+            return;
+        __shared__ dfl s_tot[REDUCE_VALUES];
+        constexpr int HALF = SMALL_CLUSTER / 2;
+        const int k = lane & 15, half = blocks / 2, c0 = (lane >> 4) * half;
+        float2 x[HALF], y[HALF];
+#pragma unroll
+        for (int c = 0; c < HALF; ++c) {
+            x[c] = y[c] = make_float2(0.0f, 0.0f);
+            if (c < half) {
+                x[c] = __ldcg(partials + 2 * (c0 + c) * REDUCE_VALUES + k);
+                y[c] = __ldcg(partials + (2 * (c0 + c) + 1) * REDUCE_VALUES + k);
+            }
+        }
+        dfl v = {0.0f, 0.0f};
+#pragma unroll
+        for (int c = 0; c < HALF; ++c)
+            if (c < half)
+                v = df_acc(v, df_acc(dfl{x[c].x, x[c].y}, dfl{y[c].x, y[c].y}));
+        v = df_acc(v, df_shfl_xor(v, 16));
+        if (lane < 16)
+            s_tot[lane] = v;
+        __syncwarp();
+        finish_update(s_tot, m, cf, pose, rmse_out, ctl, honor_stop, eps);
+        return;
+    }
+
     // Last block: fixed-order sum of all partials.  Thread t adds value t % 16
     // of partials t/16, t/16 + 16, ...; the 16 groups are then added in order.
     __shared__ float s_rhi[RED_THREADS / 32][REDUCE_VALUES], s_rlo[RED_THREADS / 32][REDUCE_VALUES];
@@ -168,41 +239,16 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_solve(const float4 *__re
     if (warp != 0)
         return;
 
-    // Warp 0 solves (a matrix entry per lane) and composes the update with
-    // the pose.
-    double rmse;
-    const bool ok = solve_update(s_tot, m, cf, pose, rmse);
-    if (lane == 0) {
-        ctl->red_done = 0u;
-        if (rmse_out)
-            *rmse_out = rmse;
-    }
-    if (!ok) {
-        if (lane == 0) {
-            atomicOr(&ctl->err, DEVERR_DEGENERATE);
-            if (honor_stop) {
-                ctl->stop = 1;
-                ctl->last_rmse = rmse;
-            }
-        }
-        return;
-    }
-    if (lane == 0 && honor_stop) {
-        const int it = ctl->iters;
-        ctl->iters = it + 1;
-        ctl->last_rmse = rmse;
-        if (eps > 0.0 && it >= 1 && fabs(rmse - ctl->prev_rmse) < eps)
-            ctl->stop = 1;
-        ctl->prev_rmse = rmse;
-    }
+    finish_update(s_tot, m, cf, pose, rmse_out, ctl, honor_stop, eps);
 }
 
 cudaError_t launch_reduce_solve(const float4 *src, int m, double *pose, const float4 *tgt, int n_tgt, const int *nn,
                                 float3 center, float2 *partials, int nparts, double *rmse_out, DevCtl *ctl,
-                                int honor_stop, double eps, cudaStream_t st)
+                                int honor_stop, double eps, bool small, cudaStream_t st)
 {
-    return launch_kernel(k_reduce_solve, dim3(nparts), dim3(RED_THREADS), 0, st, src, m, pose, tgt, n_tgt, nn, center,
-                         partials, rmse_out, ctl, honor_stop, eps);
+    return launch_kernel(small ? k_reduce_solve<true> : k_reduce_solve<false>,
+                         dim3(small ? 2 * small_blocks(m) : nparts), dim3(RED_THREADS), 0, st, src, m, pose, tgt,
+                         n_tgt, nn, center, partials, rmse_out, ctl, honor_stop, eps);
 }
 
 }  // namespace vicp
