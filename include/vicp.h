@@ -541,7 +541,9 @@ VICP_API vicp_status vicp_batch_correspond(vicp_batch *b, const float *src_xyzw,
  * context's stream (the first call for other sizes than the last still
  * synchronises to upload them), and what vicp_batch_correspond would report
  * from the device is returned by the next call that synchronises
- * (vicp_batch_correspond, vicp_batch_register). */
+ * (vicp_batch_correspond, vicp_batch_register), or, once a vicp_batch_loss
+ * enqueued behind the search has run, by the next vicp_batch_correspond_async,
+ * vicp_batch_loss or vicp_batch_build (which then does nothing else). */
 VICP_API vicp_status vicp_batch_correspond_async(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
                                                  const double *poses_dev, int32_t *nn_out, float *d2_out);
 
@@ -623,7 +625,10 @@ VICP_API vicp_status vicp_se3_left_jacobian_t(int32_t n, const double *xi_dev, c
  *   grad_src_out: dev float[sum n_src * 4], 16-byte aligned, or NULL:
  *     dloss_k (2/M) R^T r_i in x, y, z and 0 in w.
  * s_i and r_i are formed in double-float arithmetic from the FP64 pose; the
- * sums are double-float and deterministic. */
+ * sums are double-float and deterministic.  Where an earlier call on this
+ * context has failed on the device without having been reported yet (a
+ * search enqueued by vicp_batch_correspond_async that gave up at its time
+ * limit, for one, whose nn is then not filled), every output is NaN. */
 VICP_API vicp_status vicp_batch_loss(vicp_batch *b, const float *src_xyzw, const int32_t *n_src,
                                      const double *poses_dev, const int32_t *nn_dev, const double *dloss_dev,
                                      double *loss_out, double *grad_pose_out, float *grad_src_out);

@@ -135,13 +135,16 @@ int batch_iter_blocks(int shape, BatchMode mode);
 cudaError_t launch_batch_iter(int shape, BatchMode mode, int blocks, const BatchIterArgs &a, cudaStream_t st);
 
 // Differentiable loss (vicp_diff.cu): SE(3) exponential T = Exp(xi) T0 and
-// J(xi)^T g (J the left Jacobian), one thread per pose; the loss of Eq. 1
-// per pair with its left-perturbation and per-point gradients.
+// J(xi)^T g (J the left Jacobian), a warp per pose; the loss of Eq. 1
+// per pair with its left-perturbation and per-point gradients.  Where the
+// search or the build before it has failed (ctl->err: a time limit, a bounds
+// check) they are all NaN.  host_err (may be null): a word of mapped host
+// memory that receives the status word where it is not zero.
 cudaError_t launch_se3_exp(int n, const double *xi, const double *T0, double *T, cudaStream_t st);
 cudaError_t launch_se3_jlt(int n, const double *xi, const double *g, double *out, cudaStream_t st);
 cudaError_t launch_batch_loss(const float4 *src, const float4 *tgt, const BatchPair *pairs, BatchState *state,
                               const BatchItem *items, int n_items, const double *pose, const int *nn,
                               const double *dloss, float2 *partials, double *loss_out, double *grad_pose,
-                              float4 *grad_src, DevCtl *ctl, cudaStream_t st);
+                              float4 *grad_src, DevCtl *ctl, unsigned *host_err, cudaStream_t st);
 
 }  // namespace vicp

@@ -75,6 +75,11 @@ struct vicp_batch {
     BBuf nn, d2, fb_list, hv_list, partials, sitems, posef, left, open_items;
     BBuf pairs_d, state, pose, pose_save, titems, ustart_xy_d, ustart_z_d, bb, ctl;
     BBuf hsrc, htgt;
+
+    // The status word as the loss kernel found it (mapped page-locked memory,
+    // since the first build): calls that wait for nothing are followed by
+    // none that reads it back.  Zero when nothing has failed.
+    unsigned *h_err = nullptr;
 };
 
 namespace {
@@ -198,6 +203,8 @@ vicp_status read_status(vicp_batch *b)
     DevCtl *d = bctl(b);
     BCUDA(b, cudaMemcpyAsync(&err, &d->err, sizeof err, cudaMemcpyDeviceToHost, b->stream), "status read-back");
     BCUDA(b, cudaStreamSynchronize(b->stream), "synchronise");
+    if (b->h_err)
+        *(volatile unsigned *)b->h_err = 0u;   // reported here
     if (err) {
         cudaMemsetAsync(&d->err, 0, sizeof(unsigned), b->stream);
         if (err & DEVERR_TIMEOUT) {
@@ -205,12 +212,22 @@ vicp_status read_status(vicp_batch *b)
             cudaMemsetAsync(&d->bar_count, 0, sizeof(unsigned), b->stream);
             return bfail(b, VICP_ERR_TIMEOUT, "a grid barrier of the iteration kernel gave up (status 0x%x)", err);
         }
-        if (err & DEVERR_BOUNDS)
+        if (err & (DEVERR_BOUNDS | DEVERR_MATCH))
             return bfail(b, VICP_ERR_CUDA, "a device-side bounds check failed (device status 0x%x)", err);
         if (err & DEVERR_DEGENERATE)
             return VICP_ERR_DEGENERATE;   // per pair; the caller decides
     }
     return VICP_OK;
+}
+
+// The failure of an earlier search or loss that nobody waited for, if the
+// loss kernel has met it by now.
+vicp_status earlier_failure(vicp_batch *b)
+{
+    if (!b->h_err || *(volatile unsigned *)b->h_err == 0u)
+        return VICP_OK;
+    const vicp_status s = read_status(b);
+    return s == VICP_ERR_DEGENERATE ? VICP_OK : s;
 }
 
 // --- build -----------------------------------------------------------------
@@ -227,6 +244,12 @@ vicp_status build(vicp_batch *b, int P, const float *tgt, const int32_t *n_tgt, 
         const bool vs = voxel_size && voxel_size[k] > 0.0f && std::isfinite(voxel_size[k]);
         if (!vs && (!divisions || divisions[k] < 1))
             return bfail(b, VICP_ERR_INVALID, "pair %d: need voxel_size > 0 or grid_divisions >= 1", k);
+    }
+    BTRY(earlier_failure(b));
+    if (!b->h_err) {
+        BCUDA(b, cudaHostAlloc((void **)&b->h_err, sizeof(unsigned), cudaHostAllocMapped | cudaHostAllocPortable),
+              "status word");
+        *b->h_err = 0u;
     }
     b->built = false;
     drop_graph(b);
@@ -723,6 +746,8 @@ void vicp_batch_destroy(vicp_batch *b)
                    &b->titems, &b->ustart_xy_d, &b->ustart_z_d, &b->bb, &b->ctl, &b->hsrc, &b->htgt};
     for (BBuf *x : all)
         bfree(b, *x);
+    if (b->h_err)
+        cudaFreeHost(b->h_err);
     delete b;
 }
 
@@ -773,6 +798,7 @@ vicp_status vicp_batch_correspond_async(vicp_batch *b, const float *src_xyzw, co
         return bfail(b, VICP_ERR_STATE, "vicp_batch_correspond before vicp_batch_build");
     if (!src_xyzw || !aligned16(src_xyzw) || !poses_dev || !nn_out || !d2_out)
         return bfail(b, VICP_ERR_INVALID, "vicp_batch_correspond: NULL or misaligned pointer");
+    BTRY(earlier_failure(b));
     const int shape = pick_shape(b);
     BTRY(prepare_items(b, n_src, shape));
     BTRY(reset_lists(b));
@@ -959,12 +985,13 @@ vicp_status vicp_batch_loss(vicp_batch *b, const float *src_xyzw, const int32_t 
     if (!src_xyzw || !aligned16(src_xyzw) || !poses_dev || !nn_dev || !loss_out ||
         (grad_src_out && !aligned16(grad_src_out)))
         return bfail(b, VICP_ERR_INVALID, "vicp_batch_loss: NULL or misaligned pointer");
+    BTRY(earlier_failure(b));
     BTRY(prepare_items(b, n_src, pick_shape(b)));
     BCUDA(b,
           launch_batch_loss(reinterpret_cast<const float4 *>(src_xyzw), b->target, (const BatchPair *)b->pairs_d.p,
                             (BatchState *)b->state.p, (const BatchItem *)b->sitems.p, b->n_items, poses_dev, nn_dev,
                             dloss_dev, (float2 *)b->partials.p, loss_out, grad_pose_out,
-                            reinterpret_cast<float4 *>(grad_src_out), bctl(b), b->stream),
+                            reinterpret_cast<float4 *>(grad_src_out), bctl(b), b->h_err, b->stream),
           "launch of the batched loss");
     b->launches += 1;
     return VICP_OK;

@@ -54,6 +54,7 @@ constexpr unsigned DEVERR_TIMEOUT = 1u;      // a bounded wait gave up
 constexpr unsigned DEVERR_DEGENERATE = 2u;   // rank(H) < 2 in a solve
 constexpr unsigned DEVERR_BOUNDS = 4u;       // an index failed its bounds check (write skipped)
 constexpr unsigned DEVERR_CAPACITY = 8u;     // a hashed voxel table could not take a key (insert skipped)
+constexpr unsigned DEVERR_MATCH = 16u;       // the loss was given an index outside its target (point left out)
 
 // Per-context control block in device memory.  Kernels of one stream use it
 // in launch order; the comments say which kernel writes each field.

@@ -226,10 +226,20 @@ __global__ void __launch_bounds__(LOSS_THREADS) k_batch_loss(const float4 *__res
                                                              float2 *__restrict__ partials,
                                                              double *__restrict__ loss_out,
                                                              double *__restrict__ grad_pose,
-                                                             float4 *__restrict__ grad_src, DevCtl *__restrict__ ctl)
+                                                             float4 *__restrict__ grad_src, DevCtl *__restrict__ ctl,
+                                                             unsigned *__restrict__ host_err)
 {
     pdl_begin();
     constexpr int SUMS = POSE_GRAD ? LOSS_SUMS : 1;
+    // A failed search (nobody has waited for it) has left nn as it was: no
+    // number formed from it may look like a loss.  The status word also goes
+    // to the host, whose next call of this context reports it.  (The kernel
+    // itself sets DEVERR_MATCH alone, so every warp reads the same here.)
+    const unsigned err = __ldcg(&ctl->err);
+    const bool bad = (err & (DEVERR_TIMEOUT | DEVERR_BOUNDS)) != 0u;
+    if ((err & ~DEVERR_DEGENERATE) && host_err && blockIdx.x == 0 && threadIdx.x == 0)
+        *(volatile unsigned *)host_err = err;
+    const float nan_f = __int_as_float(0x7fffffff);
     __shared__ dfl s_T[LOSS_WARPS][12];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long W = (long long)gridDim.x * LOSS_WARPS, gw = (long long)blockIdx.x * LOSS_WARPS + warp;
@@ -251,7 +261,7 @@ __global__ void __launch_bounds__(LOSS_THREADS) k_batch_loss(const float4 *__res
                 acc[k] = {0.0f, 0.0f};
         }
         const dfl *T = s_T[warp];
-        const double scale = 2.0 / (double)M * (dloss ? dloss[it.pair] : 1.0);
+        const double scale = bad ? (double)nan_f : 2.0 / (double)M * (dloss ? dloss[it.pair] : 1.0);
         const float scale_f = (float)scale;
 #pragma unroll 1
         for (int i0 = it.i0 + lane; i0 < it.i1; i0 += 32 * LOSS_AHEAD) {
@@ -271,8 +281,14 @@ __global__ void __launch_bounds__(LOSS_THREADS) k_batch_loss(const float4 *__res
             for (int u = 0; u < LOSS_AHEAD; ++u) {
                 if ((unsigned)jj[u] < (unsigned)n_tgt)
                     qq[u] = __ldg(tgt + tbase + jj[u]);
-                else if (i0 + 32 * u < it.i1)
-                    atomicOr(&ctl->err, DEVERR_BOUNDS);
+                else if (i0 + 32 * u < it.i1) {
+                    if (bad) {
+                        if (grad_src)
+                            grad_src[i0 + 32 * u] = make_float4(nan_f, nan_f, nan_f, 0.0f);
+                    } else {
+                        atomicOr(&ctl->err, DEVERR_MATCH);
+                    }
+                }
             }
 #pragma unroll
             for (int u = 0; u < LOSS_AHEAD; ++u) {
@@ -352,7 +368,7 @@ __global__ void __launch_bounds__(LOSS_THREADS) k_batch_loss(const float4 *__res
             v = df_add(v, df_shfl_xor(v, 16));
             const double sum = df_to_double(v);
             if (lane == 0)
-                loss_out[it.pair] = sum / (double)M;
+                loss_out[it.pair] = bad ? (double)nan_f : sum / (double)M;
             else if (POSE_GRAD && lane < LOSS_SUMS && grad_pose)
                 grad_pose[6 * it.pair + lane - 1] = scale * sum;
             if (lane == 0)
@@ -376,13 +392,13 @@ static int loss_blocks()
 cudaError_t launch_batch_loss(const float4 *src, const float4 *tgt, const BatchPair *pairs, BatchState *state,
                               const BatchItem *items, int n_items, const double *pose, const int *nn,
                               const double *dloss, float2 *partials, double *loss_out, double *grad_pose,
-                              float4 *grad_src, DevCtl *ctl, cudaStream_t st)
+                              float4 *grad_src, DevCtl *ctl, unsigned *host_err, cudaStream_t st)
 {
     static const int resident[2] = {loss_blocks<false>(), loss_blocks<true>()};
     const int blocks = std::min(resident[grad_pose != nullptr], (n_items + LOSS_WARPS - 1) / LOSS_WARPS);
     return launch_kernel(grad_pose ? k_batch_loss<true> : k_batch_loss<false>, dim3(blocks), dim3(LOSS_THREADS), 0, st,
                          src, tgt, pairs, state, items, n_items, pose, nn, dloss, partials, loss_out, grad_pose,
-                         grad_src, ctl);
+                         grad_src, ctl, host_err);
 }
 
 }  // namespace vicp

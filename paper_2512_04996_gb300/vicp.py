@@ -589,9 +589,15 @@ class Batch:
             raise VicpError(st, "vicp_batch_create failed")
         self.handle = h
         self.n_pairs = 0
+        self.failures = 0   # device failures reported so far
+
+    def _note(self, st: int) -> int:
+        self.failures += st in (VICP_ERR_TIMEOUT, VICP_ERR_CUDA)
+        return st
 
     def _check(self, st: int, what: str):
         if st != VICP_OK:
+            self._note(st)
             raise VicpError(st, f"{what}: {self._lib.vicp_batch_last_error(self.handle).decode()}")
 
     def close(self):
@@ -641,6 +647,7 @@ class Batch:
         rm = np.zeros(P, np.float64)
         ps = np.zeros(P, np.int32)
         st = self._lib.vicp_batch_register(self.handle, s.data_ptr(), _ptr(n), _ptr(T), _ptr(it), _ptr(rm), _ptr(ps))
+        self._note(st)
         return st, T, it, rm, ps
 
     def register_host(self, source, n_src, target, n_tgt, voxel_size=None, grid_divisions=None, poses=None):
@@ -657,7 +664,7 @@ class Batch:
         st = self._lib.vicp_batch_register_host(self.handle, P, _ptr(s), _ptr(ns), _ptr(t), _ptr(nt),
                                                 None if vs is None else _ptr(vs), None if dv is None else _ptr(dv),
                                                 _ptr(T), _ptr(it), _ptr(rm), _ptr(ps))
-        if st == VICP_OK:
+        if self._note(st) == VICP_OK:
             self.n_pairs = P
         return st, T, it, rm, ps
 
@@ -850,7 +857,10 @@ class PointToPointLoss(torch.autograd.Function):
     held fixed.  Differentiable in xi ((P, 6), translation part first) and
     in the source points ((M, 4); the w column gets no gradient).  With
     recompute=True the correspondences are not kept between forward and
-    backward but searched again (same poses, the same result)."""
+    backward but searched again (same poses, the same result).  Nothing is
+    waited for on the batch's own stream: if the search fails on the device,
+    the loss and its gradients are NaN, and a later call on the batch raises
+    what happened."""
 
     @staticmethod
     def forward(ctx, xi, source, batch, n_src, T0, recompute=False):
@@ -859,7 +869,7 @@ class PointToPointLoss(torch.autograd.Function):
         src = source.detach()
         nn, _ = batch._correspond_enqueued(src, n_src, T)
         loss, _, _ = batch.loss(src, n_src, T, nn)
-        ctx.batch, ctx.n_src, ctx.recompute = batch, n_src, recompute
+        ctx.batch, ctx.n_src, ctx.recompute, ctx.failures = batch, n_src, recompute, batch.failures
         ctx.xi_dtype = xi.dtype
         if recompute:
             del nn
@@ -875,6 +885,8 @@ class PointToPointLoss(torch.autograd.Function):
             nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T)
         else:
             xi64, T, src, nn = ctx.saved_tensors
+            if ctx.batch.failures != ctx.failures:   # one reported since: perhaps of the search that made nn
+                nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T)
         dl = dloss.detach().to(torch.float64).contiguous()
         _, g_left, g_src = ctx.batch.loss(src, ctx.n_src, T, nn, dloss=dl, grad_pose=ctx.needs_input_grad[0],
                                           grad_src=ctx.needs_input_grad[1])
