@@ -110,16 +110,20 @@ __device__ __noinline__ static void jacobi_vector(double x, double (&q)[4])
 }
 
 // The same eigenvector from Horn's closed form in double-float (horn_vector,
-// good to about 1e-13) and one Newton step on (N - l I) q = 0 in FP64: with
-// l = q^T N q and the residual r = N q - l q formed in FP64, the correction
-// solves (N - l I - q q^T) dq = -r, a negative definite system that only has
-// to be right to a few digits and is solved in float (LDL^T, every lane
-// alike).  What is left is the error of r over the eigenvalue gap, as after
-// any backward stable method.  A sweep of Jacobi is six rotations of two
-// divisions and two square roots each in FP64 software sequences, and four or
-// five sweeps were about 40k cycles of one warp; this is a tenth.  Returns
-// false where the closed form's vector is no good start or the gap is under
-// 1e-4 of |H| (the caller then sweeps).
+// good to about 1e-13 on ordinary geometry) and one Newton step on
+// (N - l I) q = 0 in FP64: with l = q^T N q and the residual r = N q - l q
+// formed in FP64, the correction solves (N - l I - q q^T) dq = -r, a negative
+// definite system solved in float (LDL^T, every lane alike).  The float
+// solution is wrong by some 2^-24 over the eigenvalue gap (of |H| = 1) of
+// itself, and the step leaves dq^2 besides.  So it is taken where
+// dq <= 1e-9: what is left of dq is then some 2^-53 over the gap, as the error
+// of r is, and as after any backward stable method.  Past that, and where the
+// elimination does not prove N - l I definite away from q (a pivot of 1e-4 or
+// less; the gap is at most the least pivot), the closed form has lost its
+// digits to a small gap, above all with det H < 0, and the caller sweeps:
+// returns false.  A sweep of Jacobi is six rotations of two divisions and two
+// square roots each in FP64 software sequences, and four or five sweeps were
+// about 40k cycles of one warp; this is a tenth.
 __device__ __forceinline__ bool refined_vector(double h, double E, double x, double (&q)[4])
 {
     const int lane = threadIdx.x & 31, ri = (lane >> 2) & 3, cj = lane & 3;
@@ -170,10 +174,7 @@ __device__ __forceinline__ bool refined_vector(double h, double E, double x, dou
         for (int k = 0; k < 4; ++k)
             A[i][k] = __shfl_sync(FULL_MASK, af, 4 * i + k);
     }
-    float least = 1e30f, worst = 0.0f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        worst = fmaxf(worst, fabsf(b[i]));
+    float least = 1e30f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {   // elimination without pivoting
         least = fminf(least, A[k][k]);
@@ -187,8 +188,6 @@ __device__ __forceinline__ bool refined_vector(double h, double E, double x, dou
             b[i] -= f * b[k];
         }
     }
-    if (!(least >= 1e-4f) || !(worst <= 1e-6f))   // (also where anything is not a number)
-        return false;
 #pragma unroll
     for (int k = 3; k >= 0; --k) {
 #pragma unroll
@@ -196,6 +195,10 @@ __device__ __forceinline__ bool refined_vector(double h, double E, double x, dou
             b[k] -= A[k][c] * b[c];
         b[k] = __fdividef(b[k], A[k][k]);
     }
+    const float dq = fmaxf(fmaxf(fabsf(b[0]), fabsf(b[1])), fmaxf(fabsf(b[2]), fabsf(b[3])));
+    // (the sum besides: a maximum passes over what is not a number)
+    if (!(least >= 1e-4f) || !(dq <= 1e-9f) || !isfinite((b[0] + b[1]) + (b[2] + b[3])))
+        return false;
 #pragma unroll
     for (int r = 0; r < 4; ++r)
         q[r] += (double)b[r];
