@@ -578,8 +578,15 @@ vicp_status run_global(vicp_ctx *c, const float4 *src, int m, const double *pose
     a.d2 = d2;
     a.m = m;
     a.honor_stop = honor_stop;
-    a.n_global_out = n_global_out;
-    return launch(c, K_FALLBACK, [&] { return launch_fallback(a, c->stream); });
+    // a counter of any alignment: one that the kernel cannot store to is copied
+    const bool aligned = ((uintptr_t)n_global_out & 3u) == 0;
+    a.n_global_out = aligned ? n_global_out : &ctl_of(c)->n_global;
+    TRY(launch(c, K_FALLBACK, [&] { return launch_fallback(a, c->stream); }));
+    if (aligned)
+        return VICP_OK;
+    const cudaError_t e = cudaMemcpyAsync(n_global_out, a.n_global_out, sizeof(int32_t), cudaMemcpyDeviceToDevice,
+                                          c->stream);
+    return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "fallback count copy");
 }
 
 // Correspond + global search into nn/d2 (shared by vicp_correspond and the step).

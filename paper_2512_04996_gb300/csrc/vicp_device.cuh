@@ -77,7 +77,7 @@ struct DevCtl {
     unsigned item_next;     // batched iteration: next item; reset with fb_count
     int open_count;         // batched iteration: items with points left to phase 2; reset with fb_count
     unsigned bar_count;     // batched iteration: blocks arrived at the grid barrier
-    unsigned pad;
+    int n_global;           // fallback: global searches, for a caller's counter that it cannot store to itself
     // Work counters (added by the search kernels, read and cleared by the host).
     unsigned long long stat_queries;       // source points searched
     unsigned long long stat_fallbacks;     // of which took the global search
