@@ -46,7 +46,6 @@ struct vicp_ctx {
     cudaEvent_t ev_fork = nullptr, ev_clr = nullptr;      // graph capture: the buffer resets beside the copy
     int device = 0;
     int sms = 152;
-    bool small_ok = false;   // the device runs the one-cluster iterations of small clouds
     std::string last_error;
     uint64_t cur_bytes = 0, peak_bytes = 0;
 
@@ -606,7 +605,7 @@ vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, i
 // result is the same, bit for bit.
 bool small_sums(const vicp_ctx *c, int m)
 {
-    return c->small_ok && m <= SMALL_MAX_POINTS && !(c->params.flags & VICP_FLAG_FP64_SOLVE);
+    return m <= SMALL_MAX_POINTS && !(c->params.flags & VICP_FLAG_FP64_SOLVE) && small_iters_usable(c->device);
 }
 
 // Whether `iters` iterations of m source points on the present grid run in
@@ -1312,7 +1311,6 @@ vicp_status vicp_create(vicp_ctx **out, const vicp_params *params, const vicp_al
         cudaGetLastError();
         c->sms = 152;
     }
-    c->small_ok = small_iters_usable();
     s = buf_alloc(c, c->ctl, sizeof(vicp_ctx::RegOut), "control block and registration pose");
     if (s == VICP_OK)
         s = buf_zero(c, c->ctl, "zero control block");

@@ -219,7 +219,7 @@ inline int small_blocks(int m)
         b *= 2;
     return b;
 }
-bool small_iters_usable();   // whether the current device takes the cluster (asked once per context)
+bool small_iters_usable(int device);   // whether `device`, the current one, takes the cluster
 struct SmallArgs {
     const float4 *src;
     int m;

@@ -31,6 +31,8 @@
 // kernels gives the same bits.  The slots of two
 // iterations alternate: a block overwrites a slot only after the barrier
 // that every reader of it has passed.
+#include <mutex>
+
 #include "vicp_df.cuh"
 #include "vicp_launch.h"
 #include "vicp_search.cuh"
@@ -358,7 +360,7 @@ static cudaLaunchConfig_t small_config(int blocks, cudaLaunchAttribute (&attr)[2
 // A cluster of 16 is past the portable size and needs a device with that many
 // free SMs in one processing cluster: where it cannot be had, the separate
 // kernels serve.
-bool small_iters_usable()
+static bool small_iters_fit()
 {
     for (int m : {1, 2 * SM_CLUSTER * SM_THREADS, SMALL_MAX_POINTS}) {
         const SmallKernel k = small_kernel(m);
@@ -374,6 +376,22 @@ bool small_iters_usable()
         }
     }
     return true;
+}
+
+// The answer is the device's: asked once for each, by the first call that
+// wants it (it loads the kernels: the first context of a process took 1.08 ms
+// to create with it and takes 0.55 without, also where none ever needs them).
+bool small_iters_usable(int device)
+{
+    constexpr int MAX_DEVICES = 64;
+    static std::mutex lock;
+    static signed char known[MAX_DEVICES];   // 0: not asked; 1: yes; -1: no
+    if (device < 0 || device >= MAX_DEVICES)
+        return false;
+    std::lock_guard<std::mutex> hold(lock);
+    if (known[device] == 0)
+        known[device] = small_iters_fit() ? 1 : -1;
+    return known[device] > 0;
 }
 
 cudaError_t launch_small_iters(const SmallArgs &a, cudaStream_t st)
