@@ -299,9 +299,13 @@ GridGeom slot_geom(long long slots)
 }
 
 // --- workspace sizing ------------------------------------------------------
+// Buffers that share a capacity grow together.  The capacity is void while
+// they do: where one of them cannot be had the next call, of whatever size,
+// allocates them all again.
 vicp_status ensure_voxel_buffers(vicp_ctx *c, long long V, long long n_bricks)
 {
     if (V > c->cap_occV) {   // voxel occupancy bits: both grids (the dilation reads them)
+        c->cap_occV = -1;
         for (Buf &o : c->occ) {
             TRY(buf_alloc(c, o, (size_t)occ_words(V) * 4, "occupancy"));
             TRY(buf_zero(c, o, "zero occupancy"));
@@ -309,6 +313,7 @@ vicp_status ensure_voxel_buffers(vicp_ctx *c, long long V, long long n_bricks)
         c->cap_occV = V;
     }
     if (!sparse_of(c) && V > c->cap_V) {   // the dense grid's per-voxel arrays
+        c->cap_V = -1;
         TRY(buf_alloc(c, c->counts, (size_t)V * 4, "counts"));
         TRY(buf_zero(c, c->counts, "zero counts"));   // counts are kept at zero between builds
         TRY(buf_alloc(c, c->off, (size_t)(V + 1) * 4, "offsets"));
@@ -330,6 +335,7 @@ vicp_status ensure_voxel_buffers(vicp_ctx *c, long long V, long long n_bricks)
         c->labels_clean = false;
     }
     if (n_bricks > c->cap_bricks) {
+        c->cap_bricks = -1;
         TRY(buf_alloc(c, c->bcounts, (size_t)n_bricks * 4, "brick counts"));
         TRY(buf_zero(c, c->bcounts, "zero brick counts"));   // kept at zero between builds
         TRY(buf_alloc(c, c->bsums, (size_t)brick_tiles(n_bricks) * 8, "brick tile sums"));
@@ -358,6 +364,7 @@ vicp_status ensure_sparse_buffers(vicp_ctx *c, long long n)
 {
     const long long slots = pow2_at_least(n * 2 > 1024 ? n * 2 : 1024);
     if (slots > c->cap_o) {
+        c->cap_o = 0;
         for (Buf &k : c->okeys) {
             TRY(buf_alloc(c, k, (size_t)slots * 4, "occupied-voxel table"));
             const cudaError_t e = cudaMemsetAsync(k.p, 0xff, k.bytes, c->stream);   // empty
@@ -389,11 +396,13 @@ vicp_status ensure_sparse_buffers(vicp_ctx *c, long long n)
 vicp_status ensure_label_table(vicp_ctx *c, long long slots, long long roots, int L)
 {
     if (slots > c->cap_l) {
+        c->cap_l = 0;
         TRY(buf_alloc(c, c->lkeys, (size_t)slots * 4, "labelled-segment table"));
         TRY(buf_alloc(c, c->lseg, (size_t)slots * 8, "labelled-segment masks"));
         c->cap_l = slots;
     }
     if (roots > c->cap_r) {
+        c->cap_r = 0;
         TRY(buf_alloc(c, c->lroot, (size_t)roots * 4, "labelled roots"));
         c->cap_r = roots;
     }
@@ -406,6 +415,7 @@ vicp_status ensure_label_table(vicp_ctx *c, long long slots, long long roots, in
 vicp_status ensure_point_buffers(vicp_ctx *c, long long n)
 {
     if (n > c->cap_N) {
+        c->cap_N = -1;
         TRY(buf_alloc(c, c->keys, (size_t)n * 4, "keys"));
         TRY(buf_alloc(c, c->ids, (size_t)n * 4, "ids"));
         TRY(buf_alloc(c, c->csr, (size_t)n * 16, "csr points"));
@@ -419,6 +429,7 @@ vicp_status ensure_point_buffers(vicp_ctx *c, long long n)
 vicp_status ensure_query_buffers(vicp_ctx *c, long long m)
 {
     if (m > c->cap_M) {
+        c->cap_M = -1;
         TRY(buf_alloc(c, c->nn, (size_t)m * 4, "nn"));
         TRY(buf_alloc(c, c->d2, (size_t)m * 4, "d2"));
         TRY(buf_alloc(c, c->fb_list, (size_t)m * 4, "fallback list"));
@@ -692,6 +703,8 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
     }
     const GridGeom &g = c->geom;
     const bool sparse = sparse_of(c);
+    c->built = false;   // until everything is launched: what fails below leaves no grid behind
+    c->dilated_L = -1;
     TRY(ensure_voxel_buffers(c, g.V, brick_slots(g)));
     TRY(ensure_point_buffers(c, n));
     if (sparse)
@@ -750,7 +763,6 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
                               sparse ? occ_words(c->cap_o) : 0);
     }));
     c->built = true;
-    c->dilated_L = -1;
     c->step_loop = c->grid_steps == 1;
     c->grid_steps = 0;
     c->n_target = n;
@@ -773,6 +785,7 @@ vicp_status dilate_sparse(vicp_ctx *c, int L)
     const int blocks = dilate_hashed_blocks(g, L);
     unsigned *err = &ctl_of(c)->err;
     unsigned *parts_d = (unsigned *)c->lparts.p;
+    c->dilated_L = -1;   // (the table may grow)
     auto run = [&]() -> vicp_status {   // (pass XY zeroes the counts, the overflow flag and the root counter)
         parts_d = (unsigned *)c->lparts.p;
         return launch_on(c, K_DILATE, c->side, [&] {

@@ -334,6 +334,8 @@ vicp_status build(vicp_batch *b, int P, const float *tgt, const int32_t *n_tgt, 
     // workspace (grown, never shrunk); arrays that must start at zero are
     // cleared when new and kept at zero by the kernels (counts, brick counts
     // and tile totals by the scatter) or cleared per build (occupancy)
+    const bool same_dims = b->lab_dims == dims_key;
+    b->lab_dims.clear();   // (labels in arrays that a failed build allocated are not the last build's)
     bool fresh = false;
     BTRY(bensure(b, b->counts, (size_t)Vt * 4, "counts", &fresh));
     if (fresh)
@@ -409,12 +411,12 @@ vicp_status build(vicp_batch *b, int P, const float *tgt, const int32_t *n_tgt, 
                                       (float4 *)b->bbox.p, (float4 *)b->sb_box.p, st),
           "launch of the batched brick boxes");
     // labels: cleared in full when the arrays are new or any grid changed
-    if (fresh_lab || b->lab_dims != dims_key) {
+    if (fresh_lab || !same_dims) {
         BCUDA(b, cudaMemsetAsync(b->root.p, 0xff, (size_t)Vt * 4, st), "clear root");
         BCUDA(b, cudaMemsetAsync(b->ring.p, 0xff, (size_t)Vt, st), "clear ring");
         BCUDA(b, cudaMemsetAsync(b->dirty.p, 0, (size_t)Uz, st), "clear label flags");
-        b->lab_dims = dims_key;
     }
+    b->lab_dims = dims_key;
     BCUDA(b, launch_batch_dilate((const unsigned *)b->occ.p, pd, P, (const int *)b->ustart_xy_d.p,
                                  (const int *)b->ustart_z_d.p, L, b->inter.p, (unsigned *)b->rows.p,
                                  (unsigned char *)b->dirty.p, (int *)b->root.p, (unsigned char *)b->ring.p, st),
@@ -467,6 +469,7 @@ vicp_status prepare_items(vicp_batch *b, const int32_t *n_src, int shape)
     const std::vector<int> ns(n_src, n_src + P);
     if (shape == b->items_shape && ns == b->n_src_last)
         return VICP_OK;
+    b->items_shape = -1;   // until everything below is there: a call that fails half way is not the last one's layout
     const int T = batch_tile_points(shape, iter_blocks(b, shape, mode_of(b)), M);
     std::vector<BatchItem> items;
     long long s = 0;
