@@ -378,7 +378,8 @@ VICP_API const char *vicp_last_error(const vicp_ctx *ctx);
  *     dropped; store_bytes_out (host, may be NULL) = bytes of the store.
  *   vicp_fixed_correspond: as vicp_correspond, with the localised search
  *     reading the fixed store; with capacity >= the largest voxel count the
- *     results equal vicp_correspond's.  Needs vicp_dilate after the CSR build.
+ *     results equal vicp_correspond's.  Needs vicp_dilate after the CSR build,
+ *     and a grid of the dimensions vicp_fixed_build found (VICP_ERR_STATE).
  * Errors: VICP_ERR_INVALID, VICP_ERR_STATE, VICP_ERR_GRID_TOO_LARGE,
  * VICP_ERR_OOM, VICP_ERR_CUDA. */
 VICP_API vicp_status vicp_fixed_build(vicp_ctx *ctx, const float *target_xyzw, int32_t n, int32_t capacity,

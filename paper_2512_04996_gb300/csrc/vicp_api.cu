@@ -87,6 +87,7 @@ struct vicp_ctx {
     Buf fslots, fcount, fover;
     unsigned fixed_C = 0;
     bool fixed_built = false;
+    int fixed_dims[3] = {0, 0, 0};   // of the grid its slots are of
     // sparse grid (VICP_FLAG_SPARSE_GRID): hashed occupied voxels (keys of the
     // current and of the next build, counts, offsets by slot; the scan's slot
     // occupancy bits and tile state) and hashed labelled voxels (keys, root
@@ -1622,6 +1623,7 @@ vicp_status vicp_fixed_build(vicp_ctx *c, const float *target_xyzw, int32_t n, i
     if ((unsigned long long)g.V * (unsigned long long)capacity >= (1ull << 32))
         return fail(c, VICP_ERR_GRID_TOO_LARGE, "%lld voxels x %d slots exceed 2^32 slots", g.V, capacity);
     const size_t slot_bytes = (size_t)g.V * (size_t)capacity * 16;
+    c->fixed_built = false;   // until the slots are there
     if (c->fslots.bytes < slot_bytes)
         TRY(buf_alloc(c, c->fslots, slot_bytes, "fixed-capacity slots"));
     if (c->fcount.bytes < (size_t)g.V * 4)
@@ -1640,6 +1642,9 @@ vicp_status vicp_fixed_build(vicp_ctx *c, const float *target_xyzw, int32_t n, i
                                     c->stream);
     }));
     c->fixed_built = true;
+    c->fixed_dims[0] = g.nx;
+    c->fixed_dims[1] = g.ny;
+    c->fixed_dims[2] = g.nz;
     unsigned over = 0;
     e = cudaMemcpyAsync(&over, c->fover.p, 4, cudaMemcpyDeviceToHost, c->stream);
     if (e != cudaSuccess)
@@ -1678,6 +1683,9 @@ vicp_status vicp_fixed_correspond(vicp_ctx *c, const float *src_xyzw, int32_t n_
         return fail(c, VICP_ERR_INVALID, "pose, nn and d2 pointers must be non-NULL");
     if (!c->fixed_built || c->dilated_L < 0)
         return fail(c, VICP_ERR_STATE, "vicp_fixed_correspond needs vicp_fixed_build and vicp_dilate first");
+    // (the labels of a larger grid would lead past the end of the slots)
+    if (c->geom.nx != c->fixed_dims[0] || c->geom.ny != c->fixed_dims[1] || c->geom.nz != c->fixed_dims[2])
+        return fail(c, VICP_ERR_STATE, "vicp_fixed_correspond: other grid dimensions than vicp_fixed_build's");
     TRY(ensure_query_buffers(c, n_src));
     const float4 *src = reinterpret_cast<const float4 *>(src_xyzw);
     DevCtl *d = ctl_of(c);
