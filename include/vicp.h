@@ -55,7 +55,7 @@ typedef enum vicp_status {
     VICP_ERR_CUDA = 2,            /* a CUDA runtime call failed (see vicp_last_error) */
     VICP_ERR_OOM = 3,             /* the allocator returned NULL */
     VICP_ERR_GRID_TOO_LARGE = 4,  /* nx*ny*nz >= 2^31 voxels */
-    VICP_ERR_TIMEOUT = 5,         /* a bounded device-side wait gave up (no current kernel waits) */
+    VICP_ERR_TIMEOUT = 5,         /* a bounded device-side wait gave up (the batched iterations' grid barrier) */
     VICP_ERR_STATE = 6,           /* call order: e.g. correspond before build_grid */
     VICP_ERR_DEGENERATE = 7       /* rank(H) < 2 in the rigid solve; pose left unchanged */
 } vicp_status;
@@ -77,7 +77,9 @@ typedef struct vicp_allocator {
 #define VICP_FLAG_REBUILD_EACH_ITER (1u << 1) /* vicp_register: rebuild + dilate every iteration */
 #define VICP_FLAG_FP64_SOLVE        (1u << 2) /* vicp_step / vicp_register: centroid and cross-covariance
                                                  sums in FP64 and the rigid solve in FP64 (Horn's
-                                                 quaternion by Jacobi sweeps); default: double-float
+                                                 quaternion by a Newton step from the closed form, by
+                                                 Jacobi sweeps where that is ill-conditioned);
+                                                 default: double-float
                                                  (~48-bit) sums and solve on the FP32 pipes */
 #define VICP_FLAG_SPARSE_GRID       (1u << 3) /* the sparse (hashed) grid, see vicp_get_sparse_grid: no
                                                  per-voxel count, offset, root or ring arrays */
@@ -344,7 +346,10 @@ VICP_API vicp_status vicp_memory_report(vicp_ctx *ctx, vicp_memory *out);
 /* Kernel timing: while enabled, every kernel launch is bracketed by CUDA
  * events on the context's stream.  vicp_profile_read synchronises, writes
  * per-kernel launch counts and summed milliseconds into arrays of
- * vicp_kernel_count() entries (either may be NULL) and resets the tallies. */
+ * vicp_kernel_count() entries (either may be NULL) and resets the tallies.
+ * Small source clouds, whose iterations otherwise run in one launch, then
+ * take the separate kernels (the results are the same bits), so the entry of
+ * that launch ("small_iterations") stays at zero. */
 VICP_API vicp_status vicp_profile_enable(vicp_ctx *ctx, int32_t enable);
 VICP_API int32_t vicp_kernel_count(void);
 VICP_API const char *vicp_kernel_name(int32_t kernel);
@@ -484,7 +489,9 @@ VICP_API void vicp_batch_default_params(vicp_batch_params *p);
 
 /* Threads per block, source points per thread and resident blocks (on the
  * current device; of the double-float variant) of iteration kernel shape
- * `shape`.  Errors: VICP_ERR_INVALID. */
+ * `shape`.  (The points per thread are those of the shape's name: a warp's
+ * tile has at most 128 points whatever the shape, so shapes that differ in
+ * nothing else run alike.)  Errors: VICP_ERR_INVALID. */
 VICP_API vicp_status vicp_batch_shape_info(int32_t shape, int32_t *threads, int32_t *points_per_thread,
                                            int32_t *resident_blocks);
 

@@ -656,7 +656,6 @@ struct WarpTile {
             unsigned char near[BATCH_TILE_MAX], far[BATCH_TILE_MAX];
         };
         double lanes[N_SUMS][33];        // a row per sum (row stride 33: no bank conflicts either way)
-        double total[N_SUMS];
     };
 };
 
@@ -1099,17 +1098,17 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const __grid_constant__
     }
 }
 
-// (Tiles have at most 64 x ppt and at most BATCH_TILE_MAX points, fewer where
-// the batch has few points: 64 to 256 differ by under 3% on 256 pairs, and the
-// searches alone prefer 128, 64 x 20k points 107 us against 125 with 256.)
+// (Tiles have at most BATCH_TILE_MAX points, fewer where the batch has few: 64
+// to 256 differ by under 3% on 256 pairs, and the searches alone prefer 128,
+// 64 x 20k points 107 us against 125 with 256.)
 const BatchShape BATCH_SHAPES[BATCH_N_SHAPES] = {
     {256, 4, 2},   // 128 registers
-    {256, 2, 3},   // 80 registers, more warps per SM
+    {256, 2, 3},   // 80 registers, more warps per SM (196 bytes of spill stores, 248 of loads)
     {512, 2, 1},   // wide blocks
     {128, 4, 4},   // narrow blocks
     {256, 8, 2},   // as 0
-    {256, 2, 4},   // 64 registers
-    {256, 2, 5},   // 48 registers (spills some of the sums)
+    {256, 2, 4},   // 64 registers (492 bytes of spill stores, 652 of loads)
+    {256, 2, 5},   // 48 registers (over 1 KB of either: most of the sums)
 };
 
 using IterKernel = void (*)(const BatchIterArgs);

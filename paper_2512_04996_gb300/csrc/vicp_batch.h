@@ -38,7 +38,7 @@ struct BatchState {
     int n_bricks;          // brick scan: non-empty bricks
     int n_super;           // brick boxes: super-brick records
     int n_outside;         // scatter: target points outside the grid
-    unsigned items_done;   // iteration: items reduced (the last one solves and resets it)
+    unsigned items_done;   // loss: items done (the last one adds the sums and resets it)
     int stop;              // 1 once converged or degenerate
     int iters;             // iterations applied
     unsigned err;          // DEVERR_* bits of this pair
@@ -60,8 +60,9 @@ constexpr int BATCH_TILE_MAX = 128;      // source points per iteration item, at
 constexpr int BATCH_SMEM_PAIRS = 2048;   // unit-start tables up to this many pairs go to shared memory
 
 // Iteration kernel shapes the autotuner chooses from: threads per block,
-// source points per thread (an item is a warp's tile of at most 64 times as
-// many) and the blocks per SM the registers are budgeted for.
+// source points per thread of the shape's name (every one of them allows a
+// warp's tile of BATCH_TILE_MAX points, so it decides nothing any more, and
+// shapes 0 and 4 are one) and the blocks per SM the registers are budgeted for.
 struct BatchShape {
     int threads, ppt, min_blocks;
 };
@@ -127,11 +128,10 @@ cudaError_t launch_batch_brick_boxes(const uint4 *boxord, const int *list, const
 cudaError_t launch_batch_dilate(const unsigned *occ, const BatchPair *pairs, int P, const int *ustart_xy,
                                 const int *ustart_z, int L, void *inter, unsigned *rows, unsigned char *dirty,
                                 int *root, unsigned char *ring, cudaStream_t st);
-// Resident blocks of the iteration kernel of a shape (0 if it cannot run);
-// f64: the variant with FP64 sums and solve.
+// Resident blocks of the iteration kernel of a shape (0 if it cannot run).
 int batch_iter_blocks(int shape, BatchMode mode);
 // One iteration of every pair (or the search alone): a cooperative
-// persistent launch of `blocks` blocks (<= batch_iter_blocks(shape, f64)).
+// persistent launch of `blocks` blocks (<= batch_iter_blocks(shape, mode)).
 cudaError_t launch_batch_iter(int shape, BatchMode mode, int blocks, const BatchIterArgs &a, cudaStream_t st);
 
 // Differentiable loss (vicp_diff.cu): SE(3) exponential T = Exp(xi) T0 and

@@ -456,13 +456,15 @@ cudaError_t launch_brick_scan(const unsigned *bcounts, const GridGeom &g, unsign
 // scatter, which runs next, zeroes them for the following build.
 //
 // Output.  Dense (512 threads x 1 word): every off[v], written with coalesced
-// 16-byte stores, staged in shared memory where a warp's voxels hold points.  Sparse (256 threads x
-// 2 words, the build's form): only the entries the build and the searches
-// read -- off[v] and off[v + 1] of every occupied voxel v, off[32 k] for
-// every occupancy word k, and off[V] -- about 1/15 of the array's bytes at
-// the scene workloads' 0.5% occupancy.  Every other entry equals the nearest
-// written entry before it in its word (an empty voxel adds nothing), which
-// is how k_offsets_fill completes the array when a caller asks for it.
+// 16-byte stores, staged in shared memory where a warp's voxels hold points.
+// Sparse (256 threads x 2 words, the build's form): only the entries the
+// build and the searches read -- off[v] and off[v + 1] of every occupied voxel
+// v, off[32 k] of the occupancy words k with a point, and off[V] -- and every
+// tile's first offset (tile_off).  Every other entry equals the nearest
+// written entry before it or its tile's first offset (an empty voxel adds
+// nothing), which is how k_offsets_fill_tiles completes the array when a
+// caller asks for it.  Without tile_off (the batch) off[32 k] is written of
+// every word k, and k_offsets_fill completes the array from those.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long DESC_PREFIX = 2ull << 32;
 constexpr int LOOKBACK = 512;   // predecessors examined per lookback round
@@ -884,8 +886,8 @@ cudaError_t launch_scan(const unsigned *counts, const GridGeom &g, unsigned *off
 }
 
 // ---------------------------------------------------------------------------
-// Completes a sparse offsets array (k_scan's sparse output): an entry the
-// scan did not write equals the nearest written one before it in its
+// Completes a sparse offsets array (k_scan's sparse output without tile_off):
+// an entry the scan did not write equals the nearest written one before it in its
 // occupancy word.  Thread per voxel; reads only written entries and writes
 // only the others, so threads never touch an entry another one writes.
 // ---------------------------------------------------------------------------

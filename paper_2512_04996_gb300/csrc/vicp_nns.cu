@@ -245,8 +245,8 @@ cudaError_t launch_correspond_fixed(const float4 *src, int m, const double *pose
 // ---------------------------------------------------------------------------
 // Global search ("Globalsearch" of Alg. 4) of the queries the localised
 // search listed (global_search: a warp per query over the brick levels), and
-// the near queries and dense root segments it listed (a group of 8 to 32
-// lanes each).
+// the near queries (a group of 1 to 32 lanes each) and dense root segments
+// (4 to 32) it listed.
 //
 // Scheduling without global atomics: block b takes the items b, b + B,
 // b + 2B, ... of every list (B blocks; strided, so that a block's share
