@@ -684,6 +684,17 @@ __device__ __forceinline__ typename IterSum<F64>::T tile_sum(const typename Iter
     return v;
 }
 
+// Points of a root segment examined for the seed of a query outside the grid:
+// all of them wherever the query can be near (near_seed, whose other factor
+// is at least 2), and the first NEAR_SEED of a longer one.  The order of a
+// voxel's points in the store varies from build to build.  A seed from some of
+// them would decide, by that order, whether the query is near and summed in
+// phase 1, or far and summed in phase 3, and the last bits of the pose would
+// vary with it (from the first 16: of 24 to 31 of 256 pairs).  256 pairs, 40
+// iterations: 25.9 ms from the first 16, 26.0 from all.  (The searches alone
+// form no sums.)
+constexpr unsigned TILE_SEED = NEAR_WORK / 2;
+
 // The near queries of a tile, 1 to 32 lanes each; returns the candidates
 // this lane examined.  (Out of line, it and the sums below spill less and
 // are slower: 256 pairs 28.8 ms a batch against 25.9.)
@@ -836,7 +847,7 @@ __global__ void __launch_bounds__(TH, MINB) k_batch_iter(const __grid_constant__
                     x1 = max(x0, min(__ldg(rows.off + r + 1), rows.cap));
                     dense = x1 - x0;
                     if (!inside)   // only a seed
-                        x1 = min(x1, x0 + (unsigned)NEAR_SEED);
+                        x1 = min(x1, x0 + (SEARCH_ONLY || dense > TILE_SEED ? (unsigned)NEAR_SEED : TILE_SEED));
                 }
                 const bool local = inside && r >= 0;
                 cand += local ? dense : 0u;
