@@ -126,6 +126,8 @@ struct vicp_ctx {
     bool rg_replayed = false;         // the last registration call replayed the graph
     cudaGraphExec_t rg_exec = nullptr;
     int64_t rg_launches = 0;
+    const float4 *rg_target = nullptr;   // what a replay leaves behind: the target the searches read
+    int rg_occ = 0;                      // ... and which of the double-buffered build state is current
     cudaStream_t gstream = nullptr;
     double *h_pose = nullptr;         // page-locked, 16 doubles
     RegOut *h_out = nullptr;          // page-locked
@@ -1133,6 +1135,8 @@ vicp_status capture_registration(vicp_ctx *c, const vicp_ctx::RegKey &key, const
         return VICP_ERR_CUDA;
     }
     c->rg_key = key;
+    c->rg_target = c->target;
+    c->rg_occ = c->occ_cur;
     return VICP_OK;
 }
 
@@ -1148,6 +1152,15 @@ vicp_status replay_registration(vicp_ctx *c, double pose_host[16], int32_t *iter
         return cuda_fail(c, e, "graph replay");
     c->launches += c->rg_launches;
     c->after_solve = false;
+    // the grid on the device is this call's now, whatever was built since the
+    // call was captured (its geometry is the context's: same_call)
+    c->occ_cur = c->rg_occ;
+    c->target = c->rg_target;
+    c->n_target = c->rg_key.n;
+    c->built = true;
+    c->dilated_L = c->rg_key.L;
+    c->off_dense = false;
+    c->grid_steps = c->rg_key.max_iters;
     std::memcpy(pose_host, c->h_out->pose, 16 * sizeof(double));
     if (iters_out)
         *iters_out = c->h_out->ctl.iters;
