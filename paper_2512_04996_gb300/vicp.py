@@ -671,11 +671,22 @@ class Batch:
     def correspond(self, source: torch.Tensor, n_src, poses: torch.Tensor):
         return self._correspond(source, n_src, poses, self._lib.vicp_batch_correspond)
 
-    def _correspond_enqueued(self, source, n_src, poses):
-        """correspond without waiting for its end, where the caller works on the context's own stream (on another one
-        the end is waited for, as nothing else orders the two)."""
-        own = torch.cuda.current_stream(self.device) == self.stream
-        return self._correspond(source, n_src, poses, self._lib.vicp_batch_correspond_async if own
+    def _enter(self):
+        """Orders the context's stream after the caller's current one; the caller's stream where it is another, for
+        _leave, which orders it after the context's."""
+        cur = torch.cuda.current_stream(self.device)
+        if cur == self.stream:
+            return None
+        self.stream.wait_stream(cur)
+        return cur
+
+    def _leave(self, cur):
+        if cur is not None:
+            cur.wait_stream(self.stream)
+
+    def _correspond_enqueued(self, source, n_src, poses, cur):
+        """correspond without waiting for its end, where the caller works on the context's own stream."""
+        return self._correspond(source, n_src, poses, self._lib.vicp_batch_correspond_async if cur is None
                                 else self._lib.vicp_batch_correspond)
 
     def _correspond(self, source, n_src, poses, call):
@@ -860,15 +871,18 @@ class PointToPointLoss(torch.autograd.Function):
     backward but searched again (same poses, the same result).  Nothing is
     waited for on the batch's own stream: if the search fails on the device,
     the loss and its gradients are NaN, and a later call on the batch raises
-    what happened."""
+    what happened.  On another stream than the batch's the two are ordered one
+    after the other, in both directions."""
 
     @staticmethod
     def forward(ctx, xi, source, batch, n_src, T0, recompute=False):
         xi64 = xi.detach().to(torch.float64).contiguous()
         T = vicp_se3_exp(xi64, T0)
         src = source.detach()
-        nn, _ = batch._correspond_enqueued(src, n_src, T)
+        cur = batch._enter()
+        nn, _ = batch._correspond_enqueued(src, n_src, T, cur)
         loss, _, _ = batch.loss(src, n_src, T, nn)
+        batch._leave(cur)
         ctx.batch, ctx.n_src, ctx.recompute, ctx.failures = batch, n_src, recompute, batch.failures
         ctx.xi_dtype = xi.dtype
         if recompute:
@@ -880,16 +894,16 @@ class PointToPointLoss(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, dloss):
-        if ctx.recompute:
-            xi64, T, src = ctx.saved_tensors
-            nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T)
-        else:
-            xi64, T, src, nn = ctx.saved_tensors
-            if ctx.batch.failures != ctx.failures:   # one reported since: perhaps of the search that made nn
-                nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T)
+        xi64, T, src, *nn = ctx.saved_tensors   # (hooks may fill them on the caller's stream)
         dl = dloss.detach().to(torch.float64).contiguous()
+        cur = ctx.batch._enter()
+        if ctx.recompute or ctx.batch.failures != ctx.failures:   # (a failure since: perhaps of the search of nn)
+            nn, _ = ctx.batch._correspond_enqueued(src, ctx.n_src, T, cur)
+        else:
+            nn = nn[0]
         _, g_left, g_src = ctx.batch.loss(src, ctx.n_src, T, nn, dloss=dl, grad_pose=ctx.needs_input_grad[0],
                                           grad_src=ctx.needs_input_grad[1])
+        ctx.batch._leave(cur)
         g_xi = vicp_se3_left_jacobian_t(xi64, g_left).to(ctx.xi_dtype) if g_left is not None else None
         return g_xi, g_src, None, None, None, None
 
