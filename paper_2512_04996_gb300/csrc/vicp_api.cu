@@ -1474,8 +1474,10 @@ vicp_status vicp_register_host(vicp_ctx *c, const float *src_host, int32_t n_src
     const size_t sb = (size_t)n_src * 16, tb = (size_t)n_tgt * 16;
     if (c->hsrc.bytes < sb)
         TRY(buf_alloc(c, c->hsrc, sb, "source copy"));
-    if (c->htgt.bytes < tb)
+    if (c->htgt.bytes < tb) {
+        c->built = c->built && c->target != c->htgt.p;   // (a grid of the copy that is given up)
         TRY(buf_alloc(c, c->htgt, tb, "target copy"));
+    }
     // The target on the context's stream (the build needs it first); the
     // source on the copy stream, after everything issued so far on the
     // context's stream (earlier searches may still read the buffer), so it

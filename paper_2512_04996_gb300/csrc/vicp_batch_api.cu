@@ -783,6 +783,8 @@ vicp_status vicp_batch_register_host(vicp_batch *b, int32_t n_pairs, const float
     BTRY(check_counts(b, n_src, n_pairs, "sources", &M));
     BTRY(check_counts(b, n_tgt, n_pairs, "targets", &N));
     BTRY(bensure(b, b->hsrc, (size_t)M * 16, "source copy"));
+    if (b->htgt.bytes < (size_t)N * 16)
+        b->built = b->built && b->target != b->htgt.p;   // (grids of the copies that are given up)
     BTRY(bensure(b, b->htgt, (size_t)N * 16, "target copy"));
     BCUDA(b, cudaMemcpyAsync(b->hsrc.p, src_xyzw_host, (size_t)M * 16, cudaMemcpyHostToDevice, b->stream),
           "source upload");

@@ -130,3 +130,31 @@ def test_batch(what):
             break
         assert st == v.VICP_ERR_OOM
     assert st == 0 and k > 4
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_a_host_registration_that_gave_its_target_copy_up(batched):
+    v = vicp()
+    (s, t), (S, T) = _clouds(3000, 1.0), _clouds(40000, 1.0)
+    pool = Pool(v)
+    pose = torch.eye(4, dtype=torch.float64, device="cuda")
+    if batched:
+        b = v.Batch(v.batch_default_params(max_iters=2), allocator=pool.handle)
+        run = lambda x, y: b.register_host(x.cpu().numpy(), [x.shape[0]], y.cpu().numpy(), [y.shape[0]], None, [32])[0]
+        look = lambda: b.correspond(s, [s.shape[0]], pose[None].contiguous())
+    else:
+        b = v.Context(v.default_params(grid_divisions=32, max_iters=2), allocator=pool.handle)
+        run = lambda x, y: b.register_host(x.cpu().numpy(), y.cpu().numpy())[0]
+        look = lambda: b.step(s, pose.clone())
+    assert run(s, t) == 0
+    look()
+    pool.left = 1   # the source's copy fits, the target's does not
+    assert run(S, T) == v.VICP_ERR_OOM
+    pool.left = None
+    with pytest.raises(v.VicpError) as e:
+        look()
+    assert e.value.status == v.VICP_ERR_STATE
+    assert run(s, t) == 0
+    look()
+    b.close()
+    assert pool.live == {}
