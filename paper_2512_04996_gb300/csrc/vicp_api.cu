@@ -65,7 +65,7 @@ struct vicp_ctx {
     int occ_cur = 0;
     bool after_solve = false;   // the last kernel launched on `stream` is the reduction + solve
     int64_t grid_steps = 0;     // iterations on the present grid
-    bool step_loop = false;     // the grid before this one was built for a single iteration
+    bool step_loop = false;     // the grid before this one served a single iteration, and this one may, too
     bool off_dense = false;   // the build writes sparse offsets; vicp_get_grid completes them
     long long cap_V = -1;
     // brick level (V / 512)
@@ -613,6 +613,9 @@ vicp_status run_nns(vicp_ctx *c, const float4 *src, int m, const double *pose, i
     return e == cudaSuccess ? VICP_OK : cuda_fail(c, e, "event record");
 }
 
+// Whether every build fits the grid to its cloud (and reads the box back).
+bool refits(const vicp_ctx *c) { return c->params.dims[0] <= 0 && !(c->params.flags & VICP_FLAG_KEEP_GRID); }
+
 // Whether the update of m source points is summed in the order of the
 // one-cluster iterations (vicp_small.cu): few enough, double-float sums.
 // The searches may then run in the cluster too or as separate kernels: the
@@ -629,7 +632,9 @@ bool small_sums(const vicp_ctx *c, int m)
 // the separate kernels (after_solve), but not beside a cluster that still
 // searches.  Build, dilation and step in a loop, cluster / separate kernels:
 // sphere and plane of 1,000 points 49.2 / 45.2 us, 4,096 51.3 / 43.5, 24,576
-// 65.3 / 51.3; objects 60.7 / 55.0, 64.9 / 54.3, 73.6 / 60.9.  A kept grid:
+// 65.3 / 51.3; objects 60.7 / 55.0, 64.9 / 54.3, 73.6 / 60.9.  (Where every
+// build fits the grid anew the host waits between the two and nothing
+// overlaps: 28 such iterations of 1,515 points 2,040 / 2,204.)  A kept grid:
 // the figures in vicp_small.cu.
 bool takes_small(const vicp_ctx *c, int m)
 {
@@ -697,10 +702,8 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
 {
     TRY(check_cloud(c, target, n, "target"));
     const float4 *tgt = reinterpret_cast<const float4 *>(target);
-    const bool auto_grid = c->params.dims[0] <= 0;
-    if (auto_grid) {
-        if (!c->have_geom || !(c->params.flags & VICP_FLAG_KEEP_GRID))
-            TRY(fit_geometry(c, tgt, n));
+    if (refits(c) || (c->params.dims[0] <= 0 && !c->have_geom)) {
+        TRY(fit_geometry(c, tgt, n));
     } else if (!c->have_geom) {
         TRY(set_geometry(c, c->params.origin, c->params.voxel_size, c->params.dims));
     }
@@ -766,7 +769,7 @@ vicp_status build(vicp_ctx *c, const float *target, int32_t n, const float *load
                               sparse ? occ_words(c->cap_o) : 0);
     }));
     c->built = true;
-    c->step_loop = c->grid_steps == 1;
+    c->step_loop = c->grid_steps == 1 && !refits(c);
     c->grid_steps = 0;
     c->n_target = n;
     c->target = tgt;
@@ -964,7 +967,7 @@ vicp_status registration_work(vicp_ctx *c, const float4 *src, int32_t m, const f
     if (e != cudaSuccess)
         return cuda_fail(c, e, "stream wait");
     const bool rebuild = (c->params.flags & VICP_FLAG_REBUILD_EACH_ITER) != 0 && c->params.max_iters > 1;
-    c->step_loop = rebuild;
+    c->step_loop = rebuild && !refits(c);
     const bool one = !rebuild && c->params.max_iters > 0 && takes_small(c, m);   // all iterations in one launch
     if (one)
         TRY(run_small(c, src, m, pose, nullptr, c->params.max_iters, 1));

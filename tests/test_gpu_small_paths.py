@@ -57,3 +57,17 @@ def test_a_loop_of_builds_and_steps_and_its_launches(m):
     for _ in range(3):
         kept.step(s, b, q)
     assert kept.launch_count() - n0 == 3
+
+
+def test_a_loop_that_fits_its_grids_keeps_the_one_launch():
+    """(Nothing overlaps where the host reads every cloud's box, so there is nothing to gain from three.)"""
+    s, t = _clouds(1500)
+    ctx = context(divisions=64)
+    a = torch.eye(4, dtype=torch.float64, device="cuda")
+    for _ in range(3):
+        ctx.build_grid(t)
+        ctx.dilate()
+        n0 = ctx.launch_count()
+        ctx.step(s, a)
+        assert ctx.launch_count() - n0 == 1
+    assert ctx.sync() == 0
