@@ -638,7 +638,14 @@ bool small_sums(const vicp_ctx *c, int m)
 // the figures in vicp_small.cu.
 bool takes_small(const vicp_ctx *c, int m)
 {
-    return small_sums(c, m) && !sparse_of(c) && !c->profiling && !(c->step_loop && c->grid_steps == 0);
+    if (!small_sums(c, m) || sparse_of(c) || c->profiling)
+        return false;
+    if (!c->step_loop || c->grid_steps > 0)
+        return true;
+    // the separate kernels, unless their buffers are yet to be allocated and a
+    // caller is capturing the stream (the cluster needs none)
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    return m > c->cap_M && cudaStreamIsCapturing(c->stream, &st) == cudaSuccess && st != cudaStreamCaptureStatusNone;
 }
 
 vicp_status run_small(vicp_ctx *c, const float4 *src, int m, double *pose, double *rmse, int iters, int honor_stop)

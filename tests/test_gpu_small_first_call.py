@@ -41,6 +41,26 @@ ref.step(s, eager)
 assert ref.sync() == 0
 assert torch.equal(pose, eager)
 """
+CAPTURED_IN_A_LOOP = COMMON + """
+st = torch.cuda.Stream()
+st.wait_stream(torch.cuda.current_stream())
+with torch.cuda.stream(st):
+    c, pose = tracker()
+    c.step(s, pose)
+    c.build_grid(t)   # (a step would now take the separate kernels, whose buffers do not exist yet)
+    c.dilate()
+    assert c.sync() == 0
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        c.step(s, pose)
+    g.replay()
+torch.cuda.synchronize()
+ref, eager = tracker()
+ref.step(s, eager)
+ref.step(s, eager)
+assert ref.sync() == 0
+assert torch.equal(pose, eager)
+"""
 THREADS = COMMON + """
 out = [None] * 4
 
@@ -61,7 +81,7 @@ assert all(x is not None and torch.equal(x, out[0]) for x in out)
 """
 
 
-@pytest.mark.parametrize("code", [CAPTURED, THREADS], ids=["captured", "threads"])
+@pytest.mark.parametrize("code", [CAPTURED, CAPTURED_IN_A_LOOP, THREADS], ids=["captured", "loop", "threads"])
 def test_first_small_step_of_a_process(code):
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr[-2000:]
